@@ -22,6 +22,7 @@ using namespace fg;
 
 finger_status fg_make_plan(finger_index* ix, int mode, int ef_max, int64_t nq, SearchPlan* p,
                            int wpb, int H, int occ = 0, int shape = 0);
+void fg_make_coop_plan(finger_index* ix, int ef_max, int64_t nq, SearchPlan* p);
 finger_status fg_run_search(finger_index* ix, const SearchPlan& p, SearchArgs& a, cudaStream_t s);
 SearchArgs fg_base_args(finger_index* ix, const SearchPlan& p);
 finger_status fg_check_mode_ready(const finger_index* ix, int mode);
@@ -107,11 +108,17 @@ finger_status finger_search_batch(finger_index* ix, const float* queries, int64_
     } else {
         st = fg_make_plan(ix, ix->mode, bucket, nqb, &p, 4, 0);
     }
+    // several warps per query by this batch's own size: the grid keeps its bucket's
+    // shape, the block's width is part of the captured launch's key
+    if (st == FINGER_OK) {
+        fg_make_coop_plan(ix, bucket, nq, &p);
+        if (p.occ == COOP_OCC) p.blocks = (int)std::min<int64_t>((int64_t)ix->num_sms * p.bps, nqb);
+    }
     if (st != FINGER_OK) {
         if (prev != ix->device) cudaSetDevice(prev);
         return st;
     }
-    st = fg_ensure_scratch(ix, (int64_t)p.blocks * p.wpb);
+    st = fg_ensure_scratch(ix, plan_slots(p));
     if (st != FINGER_OK) {
         if (prev != ix->device) cudaSetDevice(prev);
         return st;
@@ -128,7 +135,8 @@ finger_status finger_search_batch(finger_index* ix, const float* queries, int64_
     a.out_d = out_dists;
     a.rerank = 32;
     const DevIndex d = make_dev(ix);
-    const auto key = std::make_pair(nqb, bucket * 4 + ix->mode);
+    const auto key = std::make_pair(nqb, (bucket * 4 + ix->mode) * (COOP_MAX_WARPS + 1) +
+                                             (p.occ == COOP_OCC ? p.wpb : 0));
     auto& caps = captures_of(ix);
     auto it = caps.find(key);
     finger_status ret = FINGER_OK;

@@ -32,6 +32,12 @@ cudaError_t occupancy_f8_k4(const SearchPlan&, int*);
 cudaError_t launch_mode_harvest(const DevIndex&, const SearchArgs&, const SearchPlan&,
                                 cudaStream_t);
 cudaError_t occupancy_mode_harvest(const SearchPlan&, int*);
+#define FG_COOP(f)                                                                             \
+    cudaError_t launch_coop_##f(const DevIndex&, const SearchArgs&, const SearchPlan&, cudaStream_t); \
+    cudaError_t occupancy_coop_##f(const SearchPlan&, int*);
+FG_COOP(m0) FG_COOP(m1) FG_COOP(f16_k2) FG_COOP(f16_k4) FG_COOP(f8_k2) FG_COOP(f8_k4)
+FG_COOP(lp_k2) FG_COOP(lp_k4)
+#undef FG_COOP
 
 void choose_groups(int nchunks, int* G, int* VPL) {
     if (nchunks <= 8) {
@@ -79,6 +85,16 @@ int search_smem_per_warp(const DevIndex& ix, int mode, int ef_cap, int H, int NP
 
 cudaError_t launch_search(const DevIndex& ix, const SearchArgs& a, const SearchPlan& p,
                           cudaStream_t s) {
+    if (p.occ == COOP_OCC) {
+        switch (p.mode) {
+            case 0: return launch_coop_m0(ix, a, p, s);
+            case 1: return launch_coop_m1(ix, a, p, s);
+            case 2: return ix.hks == 2 ? launch_coop_lp_k2(ix, a, p, s) : launch_coop_lp_k4(ix, a, p, s);
+            case 4: return ix.hks == 2 ? launch_coop_f16_k2(ix, a, p, s) : launch_coop_f16_k4(ix, a, p, s);
+            case 5: return ix.hks == 2 ? launch_coop_f8_k2(ix, a, p, s) : launch_coop_f8_k4(ix, a, p, s);
+        }
+        return cudaErrorInvalidValue;
+    }
     switch (p.mode) {
         case 0: return launch_mode0(ix, a, p, s);
         case 1: return launch_mode1(ix, a, p, s);
@@ -92,6 +108,17 @@ cudaError_t launch_search(const DevIndex& ix, const SearchArgs& a, const SearchP
 }
 
 cudaError_t search_occupancy(const DevIndex& ix, const SearchPlan& p, int* bps) {
+    if (p.occ == COOP_OCC) {
+        switch (p.mode) {
+            case 0: return occupancy_coop_m0(p, bps);
+            case 1: return occupancy_coop_m1(p, bps);
+            case 2: return ix.hks == 2 ? occupancy_coop_lp_k2(p, bps) : occupancy_coop_lp_k4(p, bps);
+            case 4: return ix.hks == 2 ? occupancy_coop_f16_k2(p, bps) : occupancy_coop_f16_k4(p, bps);
+            case 5: return ix.hks == 2 ? occupancy_coop_f8_k2(p, bps) : occupancy_coop_f8_k4(p, bps);
+        }
+        *bps = 0;   // the predictor and harvest modes have no cooperative form
+        return cudaSuccess;
+    }
     switch (p.mode) {
         case 0: return occupancy_mode0(p, bps);
         case 1: return occupancy_mode1(p, bps);
@@ -228,7 +255,8 @@ finger_status make_plan(finger_index* ix, int mode, int ef_max, int64_t nq, Sear
     p->wpb = wpb;
     p->smem_per_warp = search_smem_per_warp(d, mode, p->ef_cap, p->H, p->NPL, p->h16);
     p->blk_smem = 0;
-    if (p->blk_smem + (int64_t)p->smem_per_warp * wpb > 227 * 1024) return FINGER_ERR_UNSUPPORTED;
+    p->occ = occ_force;
+    if (plan_smem(*p) > 227 * 1024) return FINGER_ERR_UNSUPPORTED;
     // the kernel variant with the most resident blocks that shared memory admits:
     // 8 blocks (64 registers, plain mode), 6 (80 registers, plain, FP32 FINGER,
     // LP and FP16 codes), else 5 (96 registers)
@@ -265,14 +293,49 @@ finger_status make_plan(finger_index* ix, int mode, int ef_max, int64_t nq, Sear
     p->bps = bps;
     p->shape = shape;
     int64_t blocks = (int64_t)ix->num_sms * bps;
-    blocks = std::min<int64_t>(blocks, (nq + wpb - 1) / wpb);
+    const int qpb = p->occ == COOP_OCC ? 1 : wpb;   // queries per block
+    blocks = std::min<int64_t>(blocks, (nq + qpb - 1) / qpb);
     p->blocks = (int)std::max<int64_t>(blocks, 1);
     return FINGER_OK;
 }
 
+// Several warps per query (the cooperative kernel form) where a warp per query
+// leaves the GPU idle: *p, the per-warp plan for nq queries, is replaced by the
+// widest block whose queries all reside at once.  Its 128 registers allow 16
+// warps per SM, so that is 8 warps for up to 2 queries per SM, 4 for up to 4, 2
+// for up to 8 (fewer where shared memory limits the blocks).  Measured per
+// launch, one warp per query against the rule's pick:
+//   m = 960 FP16 codes, ef 300: 5.16 -> 2.49 ms at 304 queries, 5.91 -> 3.09
+//   at 608, 6.05 -> 3.79 at 1,216; plain 7.68 -> 2.01, 8.82 -> 2.60, 9.01 -> 3.39
+//   m = 128 FP16 codes, ef 140: 0.90 -> 0.83 ms at 304, 0.90 -> 0.86 at 608, but
+//   0.94 -> 0.97 at 1,216; plain, ef 122: 0.91 -> 0.57, 0.93 -> 0.63, 1.01 -> 0.85
+// Larger batches lose with short rows (m = 128 FP16 codes, 2,000 queries: 0.99
+// -> 1.64 ms).  Rows above 2 KB take a warp several load rounds each, so two
+// warps per query stay ahead there (2,000 / 4,000 / 10,000 queries: 7.5 -> 5.5,
+// 10.1 -> 8.5, 15.7 -> 15.8 ms; plain 11.4 -> 5.1, 12.4 -> 7.8, 22.3 -> 15.5).
+void make_coop_plan(finger_index* ix, int ef_max, int64_t nq, SearchPlan* p) {
+    const bool long_rows = p->G == 32 && p->VPL >= 8;
+    const bool code_short = code_mode(p->mode) && !long_rows;
+    for (int W = COOP_MAX_WARPS; W >= 2; W >>= 1) {
+        if (W == 2 && code_short) return;
+        const bool last = W == 2 && long_rows;
+        if (nq > (int64_t)ix->num_sms * (2 * COOP_MAX_WARPS / W) && !last) continue;
+        SearchPlan t;
+        if (make_plan(ix, p->mode, ef_max, nq, &t, W, p->H, COOP_OCC, p->shape) != FINGER_OK) {
+            cudaGetLastError();
+            return;
+        }
+        if (last || nq <= (int64_t)ix->num_sms * t.bps) {
+            *p = t;
+            return;
+        }
+    }
+}
+
 // The plan of a uniform search: the autotuner's launch shape when one was
 // kept for this mode and the power-of-two ef bucket of ef (finger_autotune),
-// else the default.
+// else the default; a batch that it leaves part of the GPU idle with takes the
+// cooperative form.
 finger_status make_search_plan(finger_index* ix, int ef, int64_t nq, SearchPlan* p) {
     int bucket = 16;
     while (bucket < ef) bucket <<= 1;
@@ -282,11 +345,14 @@ finger_status make_search_plan(finger_index* ix, int ef, int64_t nq, SearchPlan*
         SearchPlan t = it->second;
         if (make_plan(ix, ix->mode, ef, nq, &t, t.wpb, t.H, t.occ, t.shape) == FINGER_OK) {
             *p = t;
+            make_coop_plan(ix, ef, nq, p);
             return FINGER_OK;
         }
         cudaGetLastError();
     }
-    return make_plan(ix, ix->mode, ef, nq, p);
+    finger_status st = make_plan(ix, ix->mode, ef, nq, p);
+    if (st == FINGER_OK) make_coop_plan(ix, ef, nq, p);
+    return st;
 }
 
 finger_status ensure_scratch(finger_index* ix, int64_t slots) {
@@ -347,7 +413,7 @@ SearchArgs base_args(finger_index* ix, const SearchPlan& p) {
 }
 
 finger_status run_search(finger_index* ix, const SearchPlan& p, SearchArgs& a, cudaStream_t s) {
-    finger_status st = ensure_scratch(ix, (int64_t)p.blocks * p.wpb);
+    finger_status st = ensure_scratch(ix, plan_slots(p));
     if (st != FINGER_OK) return st;
     a.bitmap = ix->bitmap;
     a.words = ix->words;
@@ -382,6 +448,9 @@ uint64_t wsum64(const void* p, size_t bytes) {
 finger_status fg_make_plan(finger_index* ix, int mode, int ef_max, int64_t nq, SearchPlan* p,
                            int wpb, int H, int occ, int shape) {
     return make_plan(ix, mode, ef_max, nq, p, wpb, H, occ, shape);
+}
+void fg_make_coop_plan(finger_index* ix, int ef_max, int64_t nq, SearchPlan* p) {
+    make_coop_plan(ix, ef_max, nq, p);
 }
 finger_status fg_run_search(finger_index* ix, const SearchPlan& p, SearchArgs& a, cudaStream_t s) {
     return run_search(ix, p, a, s);

@@ -128,12 +128,24 @@ struct SearchPlan {
     int blocks;
     int ef_cap, H;
     int h16;            // visited hash in 16-bit slots
-    int occ;            // resident blocks of 4 warps per SM the kernel variant is compiled for
+    int occ;            // resident blocks of 4 warps per SM the kernel variant is compiled for,
+                        // or COOP_OCC: one query per block of wpb warps
     int bps;            // resident blocks per SM of this plan (its register and shared-memory limit)
     int shape;          // row shape: 0 the default (G, VPL), 1 rows on all 32 lanes
     int smem_per_warp;
     int blk_smem;       // per-block shared memory before the warp regions
 };
+
+// kernel variant with one query per block (up to COOP_MAX_WARPS warps)
+constexpr int COOP_OCC = 2;
+constexpr int COOP_MAX_WARPS = 8;
+// dynamic shared memory of a block, and queries (scratch slots) in flight per launch
+inline int plan_smem(const SearchPlan& p) {
+    return p.blk_smem + p.smem_per_warp * (p.occ == COOP_OCC ? 1 : p.wpb);
+}
+inline int64_t plan_slots(const SearchPlan& p) {
+    return (int64_t)p.blocks * (p.occ == COOP_OCC ? 1 : p.wpb);
+}
 
 // kernels / launchers (search.cu)
 cudaError_t launch_search(const DevIndex& ix, const SearchArgs& a, const SearchPlan& p,

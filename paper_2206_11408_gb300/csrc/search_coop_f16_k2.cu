@@ -1,0 +1,13 @@
+// Cooperative search kernel instances (one query per block): FINGER with FP16 codes, 2 k steps
+// (see search_impl.cuh).
+#include "search_impl.cuh"
+
+namespace fg {
+cudaError_t launch_coop_f16_k2(const DevIndex& ix, const SearchArgs& a, const SearchPlan& p,
+                           cudaStream_t s) {
+    return launch_occ<MODE_F16_K2, COOP_OCC>(ix, a, p, s);
+}
+cudaError_t occupancy_coop_f16_k2(const SearchPlan& p, int* blocks) {
+    return occupancy_occ<MODE_F16_K2, COOP_OCC>(p, blocks);
+}
+}  // namespace fg

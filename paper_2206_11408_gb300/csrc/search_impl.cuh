@@ -143,23 +143,25 @@ __device__ __forceinline__ float row_partial(const QRegs<LP, VPL>& q, const DevI
 // QS the lane's query chunks are read from the staged query qs (shared
 // memory) for this call only instead of living in registers for the whole
 // search (the FP16-code mode, whose code block needs the registers).
+// wq of W warps take the rows in turn, a pass of RPW rows each (a lone warp: 0
+// of 1); every row's sum is formed the same way whichever warp takes it.
 template <bool LP, int G, int VPL, bool QS = false>
 __device__ __forceinline__ void exact_list(const QRegs<LP, VPL>& qr, const float* qs,
                                            const DevIndex& ix, const uint32_t* nbs,
                                            const int* lst, int nlist, float* xb, int lane,
-                                           uint32_t idm = 0xFFFFFFFFu) {
+                                           uint32_t idm = 0xFFFFFFFFu, int wq = 0, int W = 1) {
     QRegs<LP, VPL> qt;
     if constexpr (QS) load_qregs<LP, G, VPL>(qt, qs, LP ? ix.m8 : ix.m4, lane % G);
     const QRegs<LP, VPL>& q = QS ? qt : qr;
     constexpr int RPW = 32 / G;
     constexpr int U = rows_per_group(VPL);   // rows per group in flight
     const int grp = lane / G, kin = lane % G;
-    for (int base = 0; base < nlist; base += U * RPW) {
+    for (int base = wq * RPW; base < nlist; base += U * RPW * W) {
         int o[U];
         float p[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int i = base + u * RPW + grp;
+            const int i = base + u * RPW * W + grp;
             o[u] = i < nlist ? lst[i] : -1;
         }
 #pragma unroll
@@ -758,8 +760,39 @@ __device__ __forceinline__ void mlp_tile(const __nv_bfloat16* xt, int kp, const 
     }
 }
 
+// Cooperative form (OCC = COOP_OCC): one query per block, for batches too small
+// to fill the GPU with a warp per query.  Warp 0 runs the search as above; the
+// other warps wait at a named barrier for its commands (in meta[7]): a new
+// query to take into registers, a list of rows whose exact distances they
+// share, or the end.  A command is published before barrier 1 and its result
+// read after barrier 2, both over the whole block.
+constexpr int COOP_QUERY = -1, COOP_EXIT = -2;   // >= 0: that many rows in lst
+
+__device__ __forceinline__ void coop_bar(int id) {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"((int)blockDim.x) : "memory");
+}
+
+// L2 prefetch of the rows of one warp's share beyond its first pass, a row at a
+// time on all lanes
+template <bool LP>
+__device__ __forceinline__ void prefetch_rest(const DevIndex& ix, const uint32_t* nbs,
+                                              const int* lst, int from, int step, int nlist,
+                                              uint32_t idm, int lane) {
+    const int bytes = LP ? ix.m8 * 16 : ix.m4 * 16;
+    const char* X = LP ? reinterpret_cast<const char*>(ix.Xh) : reinterpret_cast<const char*>(ix.X);
+    for (int i = from; i < nlist; i += step) {
+        const char* row = X + (size_t)(nbs[lst[i]] & idm) * bytes;
+        for (int off = lane * 128; off < bytes; off += 32 * 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(row + off));
+    }
+}
+
 template <int MODE, int G, int VPL, int NPL, int OCC>
-__global__ void __launch_bounds__(128, OCC) k_search(DevIndex ix, SearchArgs a) {
+__global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
+                                  OCC == COOP_OCC ? 2 : OCC)
+    k_search(DevIndex ix, SearchArgs a) {
+    constexpr bool COOP = OCC == COOP_OCC;
     constexpr bool LP = MODE == MODE_LP_K2 || MODE == MODE_LP_K4;   // BF16 rows, FP8 codes
     constexpr bool W8 = LP || MODE == MODE_F8_K2 || MODE == MODE_F8_K4;   // FP8 codes
     constexpr bool EST = MODE != FINGER_MODE_PLAIN;
@@ -784,7 +817,7 @@ __global__ void __launch_bounds__(128, OCC) k_search(DevIndex ix, SearchArgs a) 
     const int nchunks = LP ? ix.m8 : ix.m4;
     const int qs_len = LP ? ix.m8 * 8 : ix.m4 * 4;
 
-    unsigned char* wb = sm + a.blk_smem + (size_t)wib * a.warp_smem;
+    unsigned char* wb = sm + a.blk_smem + (COOP ? 0 : (size_t)wib * a.warp_smem);
     // Per-warp region: first the fixed-size staging of one expansion (compile-
     // time offsets from wb, so its addresses need no pointer registers), then
     // the regions whose sizes depend on the launch (result list, visited hash,
@@ -814,10 +847,44 @@ __global__ void __launch_bounds__(128, OCC) k_search(DevIndex ix, SearchArgs a) 
     float* qs = QSM ? pq + r_pad : reinterpret_cast<float*>(hash);
     __nv_bfloat16* xt = reinterpret_cast<__nv_bfloat16*>(QSM ? qs + ((qs_len + 3) & ~3) : pq + r_pad);   // predictor input tile
     if (FG_CHECKED) g_chk_err = a.err;   // same value from every thread
-    const int64_t slot = (int64_t)blockIdx.x * wpb + wib;
+    const int64_t slot = COOP ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * wpb + wib;
     uint32_t* bitmap = a.bitmap + slot * a.words;
     uint32_t* spl = a.spill + slot * a.spill_cap;
     const int logNB = 31 - __clz(a.H >> (a.h16 ? 3 : 2));   // buckets of the visited hash
+    // the lane's query chunks stay in registers, except where the code block needs
+    // them (80 registers); the cooperative form has 128
+    constexpr bool QST = WB && !COOP;
+    constexpr int ONE_PASS = rows_in_flight(G, VPL);   // rows one warp requests at once
+
+    if constexpr (COOP) {
+        if (wib != 0) {
+            QRegs<LP, VPL> q;
+            for (;;) {
+                coop_bar(1);
+                const int cmd = meta[7];
+                if (cmd == COOP_EXIT) return;
+                if (cmd == COOP_QUERY) {
+                    load_qregs<LP, G, VPL>(q, qs, nchunks, lane % G);
+                } else {
+                    prefetch_rest<LP>(ix, nbs, lst, ONE_PASS * wpb + wib, wpb, cmd, IDM, lane);
+                    exact_list<LP, G, VPL>(q, qs, ix, nbs, lst, cmd, xb, lane, IDM, wib, wpb);
+                }
+                coop_bar(2);
+            }
+        }
+    }
+    // exact distances of nl listed rows, shared with the helper warps where one
+    // warp would need more than one pass
+    auto exact_rows = [&](const QRegs<LP, VPL>& q, int nl, uint32_t idm) {
+        if (!COOP || nl <= ONE_PASS) {
+            exact_list<LP, G, VPL, QST>(q, qs, ix, nbs, lst, nl, xb, lane, idm);
+        } else {
+            if (lane == 0) meta[7] = nl;
+            coop_bar(1);
+            exact_list<LP, G, VPL, QST>(q, qs, ix, nbs, lst, nl, xb, lane, idm, 0, wpb);
+            coop_bar(2);
+        }
+    };
 
     for (;;) {
         int qi = 0;
@@ -833,7 +900,12 @@ __global__ void __launch_bounds__(128, OCC) k_search(DevIndex ix, SearchArgs a) 
         for (int i = lane; i < qs_len; i += 32) qs[i] = i < ix.m ? qg[i] : 0.f;
         __syncwarp();
         QRegs<LP, VPL> q;
-        if constexpr (!WB) load_qregs<LP, G, VPL>(q, qs, nchunks, lane % G);
+        if constexpr (!QST) load_qregs<LP, G, VPL>(q, qs, nchunks, lane % G);
+        if constexpr (COOP) {
+            if (lane == 0) meta[7] = COOP_QUERY;
+            coop_bar(1);
+            coop_bar(2);   // the staged query may be overwritten after this
+        }
         float qn2 = 0.f;
         for (int i = lane; i < ix.m; i += 32) qn2 = fmaf(qs[i], qs[i], qn2);
         qn2 = warp_sum(qn2);
@@ -865,7 +937,7 @@ __global__ void __launch_bounds__(128, OCC) k_search(DevIndex ix, SearchArgs a) 
             lst[0] = 0;
         }
         __syncwarp();
-        exact_list<LP, G, VPL, WB>(q, qs, ix, nbs, lst, 1, xb, lane);
+        exact_rows(q, 1, 0xFFFFFFFFu);
         float dcur = xb[0];
         c_up++;
         c_gath++;
@@ -884,7 +956,7 @@ __global__ void __launch_bounds__(128, OCC) k_search(DevIndex ix, SearchArgs a) 
                 if (v) lst[__popc(bm & ltmask)] = lane;
                 __syncwarp();
                 const int cv = __popc(bm);
-                exact_list<LP, G, VPL, WB>(q, qs, ix, nbs, lst, cv, xb, lane);
+                exact_rows(q, cv, 0xFFFFFFFFu);
                 c_up += cv;
                 c_gath += cv;
                 float bd = v ? xb[lane] : INFINITY;
@@ -1282,7 +1354,7 @@ __global__ void __launch_bounds__(128, OCC) k_search(DevIndex ix, SearchArgs a) 
                 bool need = isnew[s] && (!use_est || !full0 || !(est > ub0));
                 if (HARV && hpos[s] >= 0) need = true;   // the record needs the exact distance
                 needr[s] = need;
-                if (need) prefetch_row<LP>(ix, nb[s]);
+                if (!COOP && need) prefetch_row<LP>(ix, nb[s]);   // (helpers prefetch theirs)
                 es[s * 32 + lane] = est;
                 const unsigned bm = __ballot_sync(FULLMASK, need);
                 if (need) lst[CK(nl + __popc(bm & ltmask), 32 * NPL, 1017)] = s * 32 + lane;
@@ -1290,7 +1362,7 @@ __global__ void __launch_bounds__(128, OCC) k_search(DevIndex ix, SearchArgs a) 
             }
             __syncwarp();
             // a6: exact distances of the survivors
-            exact_list<LP, G, VPL, WB>(q, qs, ix, nbs, lst, nl, xb, lane, IDM);
+            exact_rows(q, nl, IDM);
             c_gath += nl;
             if constexpr (HARV) {
                 // target cos(q_res, d_res) = (q^T d - a b ||c||^2) / (||q_res|| ||d_res||),
@@ -1671,10 +1743,15 @@ __global__ void __launch_bounds__(128, OCC) k_search(DevIndex ix, SearchArgs a) 
         }
         __syncwarp();
     }
+    if constexpr (COOP) {
+        if (lane == 0) meta[7] = COOP_EXIT;
+        coop_bar(1);
+    }
 }
 
 // instantiate and dispatch one mode over the (G, VPL, NPL) variants and the
-// resident-block target: 5 blocks of 4 warps (96 registers) everywhere, 6 (80
+// resident-block target: COOP_OCC (search_coop_*.cu) one block per query, else
+// 5 blocks of 4 warps (96 registers) everywhere, 6 (80
 // registers) for the plain, FINGER, LP and FP16/FP8-code modes, 8 (64 registers)
 // for the plain mode.  The FINGER modes keep their gathers in flight in
 // registers and are fastest at 6 (the FP16-code mode measured slower at 7,
@@ -1684,7 +1761,7 @@ __global__ void __launch_bounds__(128, OCC) k_search(DevIndex ix, SearchArgs a) 
 template <int MODE, int OCC>
 cudaError_t launch_occ(const DevIndex& ix, const SearchArgs& a, const SearchPlan& p,
                        cudaStream_t s) {
-    const int smem = p.blk_smem + p.smem_per_warp * p.wpb;
+    const int smem = plan_smem(p);
     const dim3 grid(p.blocks), block(p.wpb * 32);
 #define FG_CASE(G_, V_, N_)                                                                    \
     if (p.G == G_ && p.VPL == V_ && p.NPL == N_) {                                           \
@@ -1706,7 +1783,7 @@ cudaError_t launch_occ(const DevIndex& ix, const SearchArgs& a, const SearchPlan
 
 template <int MODE, int OCC>
 cudaError_t occupancy_occ(const SearchPlan& p, int* blocks) {
-    const int smem = p.blk_smem + p.smem_per_warp * p.wpb;
+    const int smem = plan_smem(p);
 #define FG_CASE(G_, V_, N_)                                                                    \
     if (p.G == G_ && p.VPL == V_ && p.NPL == N_) {                                           \
         auto k = k_search<MODE, G_, V_, N_, OCC>;                                              \
