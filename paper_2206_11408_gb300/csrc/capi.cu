@@ -78,8 +78,9 @@ int search_smem_per_warp(const DevIndex& ix, int mode, int ef_cap, int H, int NP
     const bool own_qs = code_mode(mode);
     const int qs_bytes = own_qs ? 4 * ((qs_len + 3) & ~3) : 0;
     const int tile = mode == FINGER_MODE_FINGER_MLP ? 2 * 16 * (ix.mlp_kp + MLP_PAD) : 0;
-    int b = 8 * ef_cap + (h16 ? 2 : 4) * H + 4 * (uq_len + r_pad) + qs_bytes + 32 * 32 * NPL +
-            32 + tile;
+    const int yo = mode == FINGER_MODE_FINGER_MLP ? 4 * 32 * NPL : 0;   // predictor outputs
+    int b = 8 * ef_cap + (h16 ? 2 : 4) * H + 4 * (uq_len + r_pad) + qs_bytes + 16 * 32 * NPL +
+            16 + yo + tile;
     return (b + 15) & ~15;
 }
 

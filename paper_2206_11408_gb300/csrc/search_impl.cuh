@@ -7,7 +7,7 @@
 //     worst entry of T (Algorithm 1's admission test read together with the
 //     eviction that keeps |T| <= ef); entries evicted from T are never
 //     expanded, so the candidate queue C is exactly the unexpanded part of T
-//     and one sorted array holds both;
+//     and one array holds both;
 //   * a neighbour is marked visited before it is evaluated, so one skipped by
 //     the estimate is never examined again;
 //   * from the (warmup+1)-th expansion on, while |T| = ef, a new neighbour
@@ -17,7 +17,7 @@
 //
 // GB300 mapping.  A warp owns one query from an atomic work counter until the
 // batch is drained (grid = SMs x resident blocks).  Per warp in shared memory:
-// the result list T (keys and ids, the EXP bit marks expanded entries), an
+// the result list T (keys and ids, unsorted, a flag marks expanded entries), an
 // exact visited hash (16-bit slots, one bucket of eight per id, where the ids
 // fit; else 32-bit slots in probed buckets of four) that spills to a per-warp
 // global bitmap once 3/4 full, the unit residual projection of the query, and
@@ -29,11 +29,10 @@
 // tensor-core product -- and last the full rows of the neighbours whose
 // estimate passes (groups of G lanes per row, 16-byte loads, shuffle
 // reduction).  Estimates are formed for every new neighbour against the ub
-// at the start of the expansion; the sequential gate is then replayed on the
-// whole warp in adjacency order (the running ub read from a 32-deep pool of
-// T's tail and the admitted keys), so the traversal is exactly the
-// per-neighbour one of Algorithm 4, and the admitted keys are merged into T
-// once.
+// at the start of the expansion; the sequential gate is then run on the whole
+// warp over the neighbours that can still be admitted, in adjacency order (an
+// admission replaces T's largest key and finds the next), so the traversal is
+// exactly the per-neighbour one of Algorithm 4.
 #pragma once
 
 #include "internal.cuh"
@@ -208,98 +207,81 @@ __device__ __forceinline__ float exact_f32_row(const float* qs, const DevIndex& 
     return warp_sum(acc);
 }
 
-// first unexpanded entry of T at or after `from` (sz if none), with the entry
-// itself (id as stored, distance) taken from the lane that loaded it
-__device__ __forceinline__ int find_next_entry(const float* Tk, const uint32_t* Ti, int sz,
-                                               int from, int lane, uint32_t& raw, float& d) {
-    for (int b = from; b < sz; b += 32) {
-        const int i = b + lane;
-        uint32_t v = EXP;
-        float kd = 0.f;
-        if (i < sz) {
-            v = Ti[i];
-            kd = Tk[i];
-        }
-        const unsigned m = __ballot_sync(FULLMASK, !(v & EXP));
-        if (m) {
-            const int src = __ffs(m) - 1;
-            raw = __shfl_sync(FULLMASK, v, src);
-            d = __shfl_sync(FULLMASK, kd, src);
-            return b + src;
-        }
-    }
-    return sz;
+// ---- The result list T: up to ef keys in shared memory, in no order.  An entry
+// is {distance bits, id word}: distances are not negative, so their bits order
+// as unsigned integers (a NaN last), and the word holds the id above its flags
+// (exp_bit: expanded; with codes also the degree tag in bit 0), so words order
+// as ids do.  Lane l owns the entries l, l + 32, ...  What a search asks of T --
+// the nearest unexpanded key, the largest key, the replacement of the largest
+// -- is one scan by all lanes, TSCAN entries of a lane requested together, and
+// two warp reductions (of the distances, then of the words that have it).
+// A sorted T needed a replay of the gate against a pool of its largest keys, then
+// a binary search and a shift of its tail per expansion.  Per expansion of the
+// 1M x 128 FP16-code search (2.8 admissions; cycles of a warp) pop, replay and
+// merge went from 333 + 957 + 1,365 to 567 + 900 + 122 unloaded and from 814 +
+// 1,374 + 1,852 to 1,143 + 1,624 + 164 at 24 warps per SM; 10,000 queries at ef
+// 140 from 3.34 to 3.04 ms.  The scans have no branches: with a conditional
+// update per entry one took 1,100 cycles instead of 560.
+constexpr int TSCAN = 5;   // 160 entries: one round for the usual ef
+
+__device__ __forceinline__ unsigned long long t_key(uint2 v) {
+    return (unsigned long long)v.x << 32 | v.y;
 }
 
-// Merge the sorted list A (ak / ai, na <= 32 NPL entries) into the sorted
-// T[0..tk): T[0..tk + na) afterwards (tk + na <= ef).  Each key of A finds its
-// rank in T by binary search; the entries of T above the smallest of those
-// ranks move up by the number of keys of A below them (the ranks at or below
-// their position), 32 at a time from the top; then the keys of A are written
-// at rank + index.  The scan cursor moves
-// back to the first position that changed.
-template <int NPL>
-__device__ __forceinline__ void t_merge(float* Tk, uint32_t* Ti, int tk, const float* ak,
-                                        const uint32_t* ai, int na, int ef, uint32_t idm,
-                                        int& cursor, int lane) {
-    int apt[NPL];         // rank of each key of A among T[0..tk)
-    float akd[NPL];
-    uint32_t aki[NPL];
+// Largest key of T[0..n) (n = |T| = ef); with REPLACE, after the entry with word
+// `out` has given way to `in`.
+template <bool REPLACE>
+__device__ __forceinline__ void t_largest(uint2* T, int n, uint32_t out, uint2 in, int lane,
+                                          uint32_t& D, uint32_t& W) {
+    unsigned long long m = 0ull;
+    for (int b = lane; b < n; b += 32 * TSCAN) {
+        uint2 v[TSCAN];
 #pragma unroll
-    for (int t = 0; t < NPL; ++t) {
-        const int k = lane + 32 * t;
-        apt[t] = 0;
-        akd[t] = 0.f;
-        aki[t] = 0u;
-        if (k < na) {
-            akd[t] = ak[k];
-            aki[t] = ai[k];
-            int lo = 0, hi = tk;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (key_lt(Tk[mid], Ti[mid] & idm, akd[t], aki[t] & idm)) lo = mid + 1;
-                else hi = mid;
-            }
-            apt[t] = lo;
-        }
-    }
-    const int pmin = __shfl_sync(FULLMASK, apt[0], 0);   // A is sorted
-    for (int top = tk - 1; top >= pmin; top -= 32) {
-        const int i = top - lane;
-        const bool act = i >= pmin;
-        float kd = 0.f;
-        uint32_t ki = 0;
-        if (act) {
-            kd = Tk[i];
-            ki = Ti[i];
-        }
-        // the keys of A below T[i] are those whose rank in T is at most i
-        int sh = 0;
-        if (na == 1) {
-            sh = act ? 1 : 0;
-        } else {
-            for (int k = 0; k < na; ++k) {
-                const int r = __shfl_sync(FULLMASK, k < 32 ? apt[0] : apt[NPL - 1], k & 31);
-                sh += act && r <= i;
-            }
-        }
-        __syncwarp();
-        if (act && sh) {
-            Tk[CK(i + sh, ef, 1014)] = kd;
-            Ti[i + sh] = ki;
-        }
-        __syncwarp();
-    }
+        for (int u = 0; u < TSCAN; ++u)
+            v[u] = b + 32 * u < n ? T[b + 32 * u] : make_uint2(0u, 0u);
 #pragma unroll
-    for (int t = 0; t < NPL; ++t) {
-        const int k = lane + 32 * t;
-        if (k < na) {
-            Tk[CK(apt[t] + k, ef, 1015)] = akd[t];
-            Ti[apt[t] + k] = aki[t];
+        for (int u = 0; u < TSCAN; ++u) {
+            unsigned long long k = t_key(v[u]);
+            if (REPLACE) {
+                const bool hit = v[u].y == out && b + 32 * u < n;   // ids are distinct: once
+                k = hit ? t_key(in) : k;
+                if (hit) T[b + 32 * u] = in;
+            }
+            m = k > m ? k : m;
         }
     }
     __syncwarp();
-    if (pmin < cursor) cursor = pmin;
+    const uint32_t md = (uint32_t)(m >> 32);
+    D = __reduce_max_sync(FULLMASK, md);
+    W = __reduce_max_sync(FULLMASK, md == D ? (uint32_t)m : 0u);
+}
+
+// Smallest key of T whose word has no bit of `flag`; sets `flag` there (the key is
+// expanded, or taken for the output) and returns it, false if there is none.
+__device__ __forceinline__ bool t_take(uint2* T, int n, uint32_t flag, int lane, uint32_t& D,
+                                       uint32_t& W) {
+    unsigned long long m = ~0ull;
+    int at = 0;
+    for (int b = lane; b < n; b += 32 * TSCAN) {
+        uint2 v[TSCAN];
+#pragma unroll
+        for (int u = 0; u < TSCAN; ++u)
+            v[u] = b + 32 * u < n ? T[b + 32 * u] : make_uint2(~0u, ~0u);
+#pragma unroll
+        for (int u = 0; u < TSCAN; ++u) {
+            const unsigned long long k = v[u].y & flag ? ~0ull : t_key(v[u]);
+            at = k < m ? b + 32 * u : at;
+            m = k < m ? k : m;
+        }
+    }
+    __syncwarp();
+    const uint32_t md = (uint32_t)(m >> 32);
+    D = __reduce_min_sync(FULLMASK, md);
+    const uint32_t c = md == D ? (uint32_t)m : ~0u;
+    W = __reduce_min_sync(FULLMASK, c);
+    if (W == ~0u) return false;
+    if (c == W) T[at].y = W | flag;
+    return true;
 }
 
 enum { V_SEEN = 0, V_NEW = 1, V_NEW_SPILL = 2, V_PENDING = 3 };
@@ -762,7 +744,7 @@ __device__ __forceinline__ void mlp_tile(const __nv_bfloat16* xt, int kp, const 
 
 // Cooperative form (OCC = COOP_OCC): one query per block, for batches too small
 // to fill the GPU with a warp per query.  Warp 0 runs the search as above; the
-// other warps wait at a named barrier for its commands (in meta[7]): a new
+// other warps wait at a named barrier for its commands (in meta[3]): a new
 // query to take into registers, a list of rows whose exact distances they
 // share, or the end.  A command is published before barrier 1 and its result
 // read after barrier 2, both over the whole block.
@@ -804,10 +786,15 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
     // bytes of half a code block (the slots 16 NPL .. of a centre are the other half)
     constexpr int HALF_BYTES = NPL * WKS * 512 / (W8 ? 2 : 1);
     constexpr int WNT = 2 * NPL;                            // tiles per node
-    // ids in T: FP16-code mode ids carry the tag TAG (the node has more than
-    // 16 NPL neighbours, so its code block's second half is needed) below EXP
+    // with codes, neighbour ids carry the tag TAG (the node has more than 16 NPL
+    // neighbours, so its code block's second half is needed)
     constexpr uint32_t TAG = 0x40000000u;
     constexpr uint32_t IDM = WB ? ~(EXP | TAG) : ~EXP;        // id without flags
+    // id words of T: the stored id rotated left, so that the tag (bit 0) and the
+    // expanded flag lie below the id
+    constexpr int WSH = WB ? 2 : 1;
+    constexpr uint32_t EXPW = WB ? 2u : 1u, TAGW = 1u;
+    auto word_of = [](uint32_t id) { return __funnelshift_l(id, id, WSH); };
     extern __shared__ __align__(16) unsigned char sm[];
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -826,14 +813,10 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
     float* es = reinterpret_cast<float*>(nbs + 32 * NPL);      // estimate of each slot
     float* xb = es + 32 * NPL;                                 // exact distance / t_hat
     int* lst = reinterpret_cast<int*>(xb + 32 * NPL);          // compacted slot lists
-    float* ak = reinterpret_cast<float*>(lst + 32 * NPL);      // admitted keys (sorted)
-    uint32_t* ai = reinterpret_cast<uint32_t*>(ak + 32 * NPL);
-    int* apos = reinterpret_cast<int*>(ai + 32 * NPL);         // slot of each admission
-    float* aub = reinterpret_cast<float*>(apos + 32 * NPL);    // ub after it
-    int* meta = reinterpret_cast<int*>(aub + 32 * NPL);        // replay results (8 ints)
-    float* Tk = reinterpret_cast<float*>(meta + 8);
-    uint32_t* Ti = reinterpret_cast<uint32_t*>(Tk + a.ef_cap);
-    uint32_t* hash = Ti + a.ef_cap;
+    int* meta = lst + 32 * NPL;                                // meta[3]: command to the helper warps
+    float* yo = reinterpret_cast<float*>(meta + 4);            // predictor outputs (MLP mode)
+    uint2* T = reinterpret_cast<uint2*>(yo + (MLP ? 32 * NPL : 0));
+    uint32_t* hash = reinterpret_cast<uint32_t*>(T + a.ef_cap);
     const int hwords = a.h16 ? a.H >> 1 : a.H;   // 32-bit words of the visited hash
     float* uq = reinterpret_cast<float*>(hash + hwords);
     // FP16 codes: the region holds u_q's B fragments, 16 KS packed words
@@ -861,7 +844,7 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
             QRegs<LP, VPL> q;
             for (;;) {
                 coop_bar(1);
-                const int cmd = meta[7];
+                const int cmd = meta[3];
                 if (cmd == COOP_EXIT) return;
                 if (cmd == COOP_QUERY) {
                     load_qregs<LP, G, VPL>(q, qs, nchunks, lane % G);
@@ -879,7 +862,7 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
         if (!COOP || nl <= ONE_PASS) {
             exact_list<LP, G, VPL, QST>(q, qs, ix, nbs, lst, nl, xb, lane, idm);
         } else {
-            if (lane == 0) meta[7] = nl;
+            if (lane == 0) meta[3] = nl;
             coop_bar(1);
             exact_list<LP, G, VPL, QST>(q, qs, ix, nbs, lst, nl, xb, lane, idm, 0, wpb);
             coop_bar(2);
@@ -902,7 +885,7 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
         QRegs<LP, VPL> q;
         if constexpr (!QST) load_qregs<LP, G, VPL>(q, qs, nchunks, lane % G);
         if constexpr (COOP) {
-            if (lane == 0) meta[7] = COOP_QUERY;
+            if (lane == 0) meta[3] = COOP_QUERY;
             coop_bar(1);
             coop_bar(2);   // the staged query may be overwritten after this
         }
@@ -926,8 +909,8 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
             }
             __syncwarp();
         }
-        int c_exp = 0, c_exa = 0, c_est = 0, c_skip = 0, c_exact = 0, c_adm = 0, c_up = 0,
-            c_gath = 0, c_half = 0;   // c_half: code-block halves read (FP16 codes)
+        int c_exa = 0, c_est = 0, c_skip = 0, c_adm = 0, c_up = 0, c_gath = 0,
+            c_half = 0;   // c_half: code-block halves read (FP16 codes)
         bool fail = false;
 
         // ---- a2: greedy descent through levels maxlevel..1 (exact distances)
@@ -985,8 +968,8 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
         for (int i = lane; i < hwords; i += 32) hash[i] = PAD;
         __syncwarp();
         if (lane == 0) {
-            Tk[0] = dcur;
-            Ti[0] = WB ? cur | TAG : cur;   // (its degree is not looked up: read both halves)
+            // (with codes: its degree is not looked up, both halves are read)
+            T[0] = make_uint2(__float_as_uint(dcur), word_of(WB ? cur | TAG : cur));
             if (a.h16) {   // the table is empty: distance 0, first slot
                 const uint32_t h = (cur * 0x9E3779B1u) & ((1u << (logNB + 15)) - 1u);
                 reinterpret_cast<uint16_t*>(hash)[8 * (h >> 15)] = (uint16_t)(h & 0x7FFFu);
@@ -995,23 +978,25 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
             }
         }
         __syncwarp();
-        int sz = 1, cursor = 0, hcount = 1, nspill = 0;
+        int sz = 1, hcount = 1, nspill = 0;
         bool spill_mode = false;
         int expansions = 0;
+        uint32_t ubd = 0u, ubw = 0u;   // largest key of T, valid while T is full
+        if (sz == ef) {
+            ubd = T[0].x;
+            ubw = T[0].y;
+        }
         while (!fail) {
-            uint32_t craw = 0u;
-            float dc = 0.f;
-            cursor = find_next_entry(Tk, Ti, sz, cursor, lane, craw, dc);
-            if (cursor >= sz) break;
+            uint32_t cd_bits, cw;
+            if (!t_take(T, sz, EXPW, lane, cd_bits, cw)) break;
             if (expansions >= a.max_expansions || nspill + 32 * NPL > a.spill_cap) {
                 fail = true;
                 break;
             }
-            (void)CK(cursor, ef, 1001);
-            const uint32_t c = craw & IDM;
-            const bool cfull = craw & TAG;   // FP16 codes: second half of the block needed
-            __syncwarp();
-            if (lane == 0) Ti[cursor] = craw | EXP;
+            if (cw == ubw) ubw |= EXPW;   // as stored
+            const float dc = __uint_as_float(cd_bits);
+            const uint32_t c = cw >> WSH;
+            const bool cfull = cw & TAGW;   // codes: second half of the block needed
             expansions++;
             const bool use_est = EST && expansions > a.warmup;
 
@@ -1147,7 +1132,7 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
 
             // a5: estimates of the new neighbours against ub at expansion start
             const bool full0 = sz == ef;
-            const float ub0 = full0 ? Tk[ef - 1] : INFINITY;
+            const float ub0 = full0 ? __uint_as_float(ubd) : INFINITY;
             float tr[NPL];          // distribution-matched cosine per slot
             int64_t hpos[NPL];      // harvest record of each slot (-1: none)
 #pragma unroll
@@ -1274,8 +1259,7 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
                 // within the margin mlp_delta * ub of the ub at the expansion start
                 // (every slot when mlp_delta < 0) gets the predictor.  Its feature
                 // rows go through the network 16 at a time (one m16 tile per
-                // round); outputs land in `ak` (free until the admission replay)
-                // at the slot's compact row.
+                // round); outputs land in `yo` at the slot's compact row.
                 if (use_est) {
                     int nunc = 0;
 #pragma unroll
@@ -1309,7 +1293,7 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
                         for (int i = rows * wpr + lane; i < 16 * wpr; i += 32) xw[i] = 0u;
                         __syncwarp();
                         mlp_tile(xt, ix.mlp_kp, ix.W1f, ix.W2f, ix.b1, ix.b2, ix.w3, ix.b3,
-                                 ak + base, lane);
+                                 yo + base, lane);
                         __syncwarp();
                     }
                 }
@@ -1328,7 +1312,7 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
                         // the fallback for a non-finite output), else the matched one
                         t = tr[s];
                         if (crow[s] >= 0) {
-                            const float y = ak[crow[s]];
+                            const float y = yo[crow[s]];
                             if (isfinite(y)) t = y + ix.mlp_eps;
                         }
                     } else if constexpr (BAL) {
@@ -1383,359 +1367,156 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
                 }
             }
 
-            // New neighbours met while T is below ef are admitted with no gate:
-            // the first ef - |T| of them in slot order are rank-sorted into
-            // ak / ai and merged at once.  The rest, met once T is full (all of
-            // them when it was full at the start), go through the gate replay.
+            // New neighbours met while T is below ef are admitted with no gate: the
+            // first ef - |T| of them in slot order are appended.  The rest, met once T
+            // is full (all of them when it was full at the start), go through the
+            // sequential gate.
             bool gate[NPL];
             bool replay = full0;
 #pragma unroll
             for (int s = 0; s < NPL; ++s) gate[s] = isnew[s];
             if (!full0) {
-                unsigned bnew[NPL], bfill[NPL];
+                const int room = ef - sz;
                 int nnew = 0;
 #pragma unroll
                 for (int s = 0; s < NPL; ++s) {
-                    bnew[s] = __ballot_sync(FULLMASK, isnew[s]);
-                    nnew += __popc(bnew[s]);
-                }
-                const int f = min(nnew, ef - sz);
-                bool fill[NPL];
-                int before = 0;
-#pragma unroll
-                for (int s = 0; s < NPL; ++s) {
-                    const int idx = before + __popc(bnew[s] & ltmask);
-                    fill[s] = isnew[s] && idx < f;
-                    gate[s] = isnew[s] && idx >= f;
-                    bfill[s] = __ballot_sync(FULLMASK, fill[s]);
-                    before += __popc(bnew[s]);
-                }
-#pragma unroll
-                for (int s = 0; s < NPL; ++s) {
-                    const float md = xb[s * 32 + lane];
-                    const uint32_t mi = nb[s];
-                    int rk = 0;
-#pragma unroll
-                    for (int s2 = 0; s2 < NPL; ++s2) {
-                        unsigned bits = bfill[s2];
-                        while (bits) {
-                            const int j = __ffs(bits) - 1;
-                            bits &= bits - 1;
-                            const int o = s2 * 32 + j;
-                            rk += key_lt(xb[o], nbs[o] & IDM, md, mi);
-                        }
-                    }
-                    if (fill[s]) {
-                        ak[rk] = md;
-                        ai[rk] = nbt[s];   // as stored in T
-                    }
+                    const unsigned bm = __ballot_sync(FULLMASK, isnew[s]);
+                    const int idx = nnew + __popc(bm & ltmask);
+                    gate[s] = isnew[s] && idx >= room;
+                    if (isnew[s] && idx < room)
+                        T[CK(sz + idx, ef, 1015)] =
+                            make_uint2(__float_as_uint(xb[s * 32 + lane]), word_of(nbt[s]));
+                    nnew += __popc(bm);
                 }
                 __syncwarp();
+                const int f = min(nnew, room);
                 c_exa += f;
-                c_exact += f;
                 c_adm += f;
-                if (f > 0) t_merge<NPL>(Tk, Ti, sz, ak, ai, f, ef, IDM, cursor, lane);
                 sz += f;
-                replay = nnew > f;   // T is full now and new neighbours remain
+                replay = nnew > room;   // T is full now and new neighbours remain
+                if (sz == ef) t_largest<false>(T, ef, 0u, make_uint2(0u, 0u), lane, ubd, ubw);
             }
             if (replay) {
-                // T is full and stays full.  Only neighbours evaluated exactly and
-                // below the starting ub can be admitted; replay the sequential gate
-                // over them with a running model of ub (top-ef of T and the admitted
-                // set A), then merge A into T once.
-                const float u0d = Tk[ef - 1];
-                const uint32_t u0i = Ti[ef - 1] & IDM;
-                unsigned cb[NPL], cskip[NPL];
+                // T is full and stays full.  Only neighbours evaluated exactly and below
+                // the starting ub can be admitted; they are taken in slot order, as
+                // the sequential scan meets them, against the running ub.
                 float xd[NPL];     // exact distance of each slot
                 float estv[NPL];   // estimate of each slot (read back: no register across the gathers)
-                int ncand = 0;
+                float myub[NPL];   // the running ub (distance) when the scan reaches each slot
+                unsigned cb[NPL];
+                uint32_t wd[NPL];
 #pragma unroll
                 for (int s = 0; s < NPL; ++s) {
                     const int o = s * 32 + lane;
                     xd[s] = xb[o];
                     estv[s] = es[o];
-                    const bool cand = gate[s] && needr[s] && key_lt(xd[s], nb[s], u0d, u0i);
-                    cb[s] = __ballot_sync(FULLMASK, cand);
-                    cskip[s] = 0u;
-                    ncand += __popc(cb[s]);
+                    wd[s] = word_of(nbt[s]);
+                    myub[s] = __uint_as_float(ubd);
+                    const uint32_t xbits = __float_as_uint(xd[s]);
+                    cb[s] = __ballot_sync(FULLMASK, gate[s] && needr[s] &&
+                                                        (xbits < ubd || (xbits == ubd && wd[s] < ubw)));
                 }
-                int tk, na, nadm;
-                float myub[NPL];   // the running ub (distance) when the scan reaches each slot
-                if (ncand == 0) {
-                    tk = ef;
-                    na = 0;
-                    nadm = 0;
 #pragma unroll
-                    for (int t = 0; t < NPL; ++t) myub[t] = u0d;
-                } else if (ncand == 1) {
-                    // The first candidate in slot order is always admitted (its
-                    // estimate and key are below the starting ub); it pushes out
-                    // T's last entry, and ub becomes the larger of it and T[ef - 2].
-                    int s1 = 0;
+                for (int s = 0; s < NPL; ++s) {
+                    unsigned bits = cb[s];
+                    while (bits) {
+                        const int jj = __ffs(bits) - 1;
+                        bits &= bits - 1;
+                        const float ce = __shfl_sync(FULLMASK, estv[s], jj);
+                        const uint32_t cd = __float_as_uint(__shfl_sync(FULLMASK, xd[s], jj));
+                        const uint32_t cword = __shfl_sync(FULLMASK, wd[s], jj);
+                        if (use_est && ce > __uint_as_float(ubd)) continue;
+                        if (!(cd < ubd || (cd == ubd && cword < ubw))) continue;
+                        // admitted: it takes the place of T's largest key
+                        t_largest<true>(T, ef, ubw, make_uint2(cd, cword), lane, ubd, ubw);
+                        c_adm++;
 #pragma unroll
-                    for (int s = NPL - 1; s >= 0; --s)
-                        if (cb[s]) s1 = s;
-                    float xs = xd[0];
-                    uint32_t ns = nbt[0];
-                    unsigned bs = cb[0];
-#pragma unroll
-                    for (int s = 1; s < NPL; ++s)
-                        if (s == s1) {
-                            xs = xd[s];
-                            ns = nbt[s];
-                            bs = cb[s];
-                        }
-                    const int jj = __ffs(bs) - 1;
-                    const int o1 = s1 * 32 + jj;
-                    const float cd = __shfl_sync(FULLMASK, xs, jj);
-                    const uint32_t craw2 = __shfl_sync(FULLMASK, ns, jj);   // as stored in T
-                    float ubd = cd;
-                    uint32_t ubi = craw2 & IDM;
-                    if (ef >= 2) {
-                        const float td = Tk[ef - 2];
-                        const uint32_t ti = Ti[ef - 2] & IDM;
-                        if (key_lt(ubd, ubi, td, ti)) {
-                            ubd = td;
-                            ubi = ti;
-                        }
-                    }
-#pragma unroll
-                    for (int t = 0; t < NPL; ++t) myub[t] = t * 32 + lane <= o1 ? u0d : ubd;
-                    tk = ef - 1;
-                    na = 1;
-                    nadm = 1;
-                    if (lane == 0) {
-                        ak[0] = cd;
-                        ai[0] = craw2;
-                    }
-                    __syncwarp();
-                } else if (ncand < 32) {
-                    // Warp-parallel replay.  After j admissions the top ef is the
-                    // ef smallest keys of T and the admitted set A, so ub is the
-                    // (j+1)-th largest key of T's tail and A: lane p holds the
-                    // p-th largest of them (the pool, 32 deep, enough for j < 32),
-                    // lane j the j-th admission (the log).  Candidates are taken
-                    // in slot order as the sequential scan meets them.
-                    float pd = lane < ef ? Tk[ef - 1 - lane] : -1.f;   // -1: below any distance
-                    uint32_t pi = lane < ef ? Ti[ef - 1 - lane] & IDM : 0u;
-                    float ld = 0.f;
-                    uint32_t li = 0u;
-                    float ubd = u0d;
-                    uint32_t ubi = u0i;
-                    int j = 0, prev = -1;
-#pragma unroll
-                    for (int s = 0; s < NPL; ++s) {
-                        unsigned bits = cb[s];
-                        unsigned skm = 0u;
-                        while (bits) {
-                            const int jj = __ffs(bits) - 1;
-                            bits &= bits - 1;
-                            const int o = s * 32 + jj;
-#pragma unroll
-                            for (int t = 0; t < NPL; ++t) {
-                                const int so = t * 32 + lane;
-                                if (so > prev && so <= o) myub[t] = ubd;
-                            }
-                            prev = o;
-                            const float ce = __shfl_sync(FULLMASK, estv[s], jj);
-                            const float cd = __shfl_sync(FULLMASK, xd[s], jj);
-                            const uint32_t craw2 = __shfl_sync(FULLMASK, nbt[s], jj);   // as stored in T
-                            const uint32_t cid = craw2 & IDM;
-                            if (use_est && ce > ubd) {
-                                skm |= 1u << jj;
-                                continue;
-                            }
-                            if (!key_lt(cd, cid, ubd, ubi)) continue;
-                            // admit: log it, insert it into the descending pool
-                            if (lane == j) {
-                                ld = cd;
-                                li = craw2;
-                            }
-                            const int pos = __popc(__ballot_sync(FULLMASK, key_lt(cd, cid, pd, pi)));
-                            const float sd = __shfl_up_sync(FULLMASK, pd, 1);
-                            const uint32_t si = __shfl_up_sync(FULLMASK, pi, 1);
-                            if (lane > pos) {
-                                pd = sd;
-                                pi = si;
-                            } else if (lane == pos) {
-                                pd = cd;
-                                pi = cid;
-                            }
-                            ++j;
-                            ubd = __shfl_sync(FULLMASK, pd, j);
-                            ubi = __shfl_sync(FULLMASK, pi, j);
-                        }
-                        cskip[s] = skm;
-                    }
-#pragma unroll
-                    for (int t = 0; t < NPL; ++t)
-                        if (t * 32 + lane > prev) myub[t] = ubd;
-                    nadm = j;
-                    // the j largest keys left the top ef; an admitted key stays iff
-                    // it is below the smallest of them, pool[j - 1]
-                    const float thd = __shfl_sync(FULLMASK, pd, j > 0 ? j - 1 : 0);
-                    const uint32_t thi = __shfl_sync(FULLMASK, pi, j > 0 ? j - 1 : 0);
-                    const bool kept = lane < j && key_lt(ld, li & IDM, thd, thi);
-                    const unsigned bk = __ballot_sync(FULLMASK, kept);
-                    na = __popc(bk);
-                    tk = ef - na;
-                    // the kept admissions, ascending, into ak / ai for the merge
-                    int rk = 0;
-                    for (int t = 0; t < j; ++t) {
-                        const float od = __shfl_sync(FULLMASK, ld, t);
-                        const uint32_t oi = __shfl_sync(FULLMASK, li, t);
-                        rk += ((bk >> t) & 1u) && key_lt(od, oi & IDM, ld, li & IDM);
-                    }
-                    if (kept) {
-                        ak[rk] = ld;
-                        ai[rk] = li;
-                    }
-                    __syncwarp();
-                } else {
-                    // 32 or more candidates: the serial replay on lane 0, results
-                    // through shared memory
-                    if (lane == 0) {
-                        float ubd = u0d;
-                        uint32_t ubi = u0i;
-                        int tk = ef, na = 0, nadm = 0;
-#pragma unroll
-                        for (int s = 0; s < NPL; ++s) {
-                            unsigned bits = cb[s];
-                            unsigned skm = 0u;
-                            while (bits) {
-                                const int j = __ffs(bits) - 1;
-                                bits &= bits - 1;
-                                const int o = s * 32 + j;
-                                if (use_est && es[o] > ubd) {
-                                    skm |= 1u << j;
-                                    continue;
-                                }
-                                const float d = xb[CK(o, 32 * NPL, 1008)];
-                                const uint32_t idt = nbs[o];   // as stored in T
-                                const uint32_t id = idt & IDM;
-                                if (!key_lt(d, id, ubd, ubi)) continue;
-                                // the current worst of the top ef leaves it
-                                if (tk == 0 ||
-                                    (na > 0 && key_lt(Tk[CK(tk - 1, ef, 1009)], Ti[tk - 1] & IDM,
-                                                      ak[CK(na - 1, 32 * NPL, 1010)], ai[na - 1] & IDM)))
-                                    na--;
-                                else
-                                    tk--;
-                                // insert (d, id) into the sorted admitted list
-                                int p = na;
-                                while (p > 0 && key_lt(d, id, ak[p - 1], ai[p - 1] & IDM)) {
-                                    ak[CK(p, 32 * NPL, 1011)] = ak[p - 1];
-                                    ai[p] = ai[p - 1];
-                                    --p;
-                                }
-                                ak[CK(p, 32 * NPL, 1012)] = d;
-                                ai[p] = idt;
-                                na++;
-                                // new ub: the larger of T[tk-1] and max(A)
-                                ubd = ak[na - 1];
-                                ubi = ai[na - 1] & IDM;
-                                if (tk > 0 && key_lt(ubd, ubi, Tk[tk - 1], Ti[tk - 1] & IDM)) {
-                                    ubd = Tk[tk - 1];
-                                    ubi = Ti[tk - 1] & IDM;
-                                }
-                                apos[CK(nadm, 32 * NPL, 1013)] = o;
-                                aub[nadm] = ubd;
-                                nadm++;
-                            }
-                            meta[3 + s] = (int)skm;
-                        }
-                        meta[0] = tk;
-                        meta[1] = na;
-                        meta[2] = nadm;
-                    }
-                    __syncwarp();
-                    tk = meta[0];
-                    na = meta[1];
-                    nadm = meta[2];
-#pragma unroll
-                    for (int s = 0; s < NPL; ++s) {
-                        cskip[s] = (unsigned)meta[3 + s];
-                        const int o = s * 32 + lane;
-                        float ubt = u0d;
-                        for (int k = 0; k < nadm; ++k)
-                            if (apos[k] < o) ubt = aub[k];
-                        myub[s] = ubt;
+                        for (int t = 0; t < NPL; ++t)
+                            if (t * 32 + lane > s * 32 + jj) myub[t] = __uint_as_float(ubd);
                     }
                 }
                 // counters of every new neighbour under the sequential semantics
 #pragma unroll
                 for (int s = 0; s < NPL; ++s) {
-                    bool skipped = false;
-                    if (gate[s]) {
-                        if ((cb[s] >> lane) & 1u) skipped = (cskip[s] >> lane) & 1u;
-                        else if (use_est) skipped = estv[s] > myub[s];
-                    }
                     const int nnew = __popc(__ballot_sync(FULLMASK, gate[s]));
-                    const int nsk = __popc(__ballot_sync(FULLMASK, skipped));
                     c_exa += nnew;
-                    if (use_est) c_est += nnew;
-                    c_skip += nsk;
-                    c_exact += nnew - nsk;
+                    if (use_est) {
+                        c_est += nnew;
+                        c_skip += __popc(__ballot_sync(FULLMASK, gate[s] && estv[s] > myub[s]));
+                    }
                 }
-                c_adm += nadm;
-                // merge A (sorted, na entries) into T[0..tk) -> T[0..ef)
-                if (na > 0) t_merge<NPL>(Tk, Ti, tk, ak, ai, na, ef, IDM, cursor, lane);
             }
             __syncwarp();
         }
-        c_exp = expansions;
 
-        // ---- LP: re-rank the head of T with FP32 rows
+        // ---- the head of T in order: its R smallest keys
+        const int R = min(sz, LP ? max(K, a.rerank) : K);
+        for (int i = lane; i < sz; i += 32) T[i].y &= ~EXPW;   // now: taken for the output
+        __syncwarp();
         if constexpr (LP) {
-            const int R = min(sz, max(K, a.rerank));
-            float* rk = reinterpret_cast<float*>(hash);
-            uint32_t* ri = hash + a.ef_cap;   // the plan keeps 2 ef_cap words in the table
+            // re-rank with FP32 rows; the plan keeps 2 ef_cap words in the table
+            uint2* hd = reinterpret_cast<uint2*>(hash);
             for (int i = 0; i < R; ++i) {
-                const float d = exact_f32_row(qs, ix, Ti[i] & IDM, lane);
-                if (lane == 0) Tk[i] = d;
+                uint32_t d, w;
+                t_take(T, sz, EXPW, lane, d, w);
+                const float x = exact_f32_row(qs, ix, w >> WSH, lane);
+                if (lane == 0) hd[i] = make_uint2(__float_as_uint(x), w >> WSH);
             }
             __syncwarp();
             for (int i = lane; i < R; i += 32) {
-                const float d = Tk[i];
-                const uint32_t id = Ti[i] & IDM;
+                const uint2 e = hd[i];
                 int rank = 0;
-                for (int j = 0; j < R; ++j) rank += key_lt(Tk[j], Ti[j] & IDM, d, id);
-                rk[rank] = d;
-                ri[rank] = id;
-            }
-            __syncwarp();
-            for (int i = lane; i < R; i += 32) {
-                Tk[i] = rk[i];
-                Ti[i] = ri[i];
+                for (int j = 0; j < R; ++j) {
+                    const uint2 o = hd[j];
+                    rank += o.x < e.x || (o.x == e.x && o.y < e.y);
+                }
+                if (rank < K) {
+                    a.out_ids[ooff + rank] = (int64_t)e.y;
+                    a.out_d[ooff + rank] = __uint_as_float(e.x);
+                }
             }
             __syncwarp();
         }
 
         // ---- a7: output
-        for (int k = lane; k < K; k += 32) {
-            a.out_ids[ooff + k] = k < sz ? (int64_t)(Ti[k] & IDM) : (int64_t)-1;
-            a.out_d[ooff + k] = k < sz ? Tk[k] : INFINITY;
+        for (int k0 = 0; k0 < K; k0 += 32) {
+            uint32_t od = 0x7F800000u;   // +inf: no result
+            int64_t oi = -1;
+            if constexpr (!LP)
+                for (int k = k0; k < min(k0 + 32, R); ++k) {
+                    uint32_t d, w;
+                    t_take(T, sz, EXPW, lane, d, w);
+                    if (lane == k - k0) {
+                        od = d;
+                        oi = (int64_t)(w >> WSH);
+                    }
+                }
+            const int k = k0 + lane;
+            if (k < K && (!LP || k >= R)) {
+                a.out_ids[ooff + k] = oi;
+                a.out_d[ooff + k] = __uint_as_float(od);
+            }
         }
         for (int i = lane; i < nspill; i += 32) bitmap[spl[i] >> 5] = 0u;
         if (lane == 0) {
             if (fail) atomicOr(a.err, (int)FINGER_ERR_LIMIT);
             unsigned long long* g = a.cnt;
-            atomicAdd(g + 0, (unsigned long long)c_exp);
+            atomicAdd(g + 0, (unsigned long long)expansions);
             atomicAdd(g + 1, (unsigned long long)c_exa);
             atomicAdd(g + 2, (unsigned long long)c_est);
             atomicAdd(g + 3, (unsigned long long)c_skip);
-            atomicAdd(g + 4, (unsigned long long)c_exact);
+            atomicAdd(g + 4, (unsigned long long)(c_exa - c_skip));
             atomicAdd(g + 5, (unsigned long long)c_adm);
             atomicAdd(g + 6, (unsigned long long)c_up);
             atomicAdd(g + 7, (unsigned long long)c_gath);
             if (WB) atomicAdd(g + 8, (unsigned long long)c_half * HALF_BYTES);
             if (a.cnt_q) {
                 int32_t* cq = a.cnt_q + (size_t)qi * 8;
-                cq[0] = c_exp;
+                cq[0] = expansions;
                 cq[1] = c_exa;
                 cq[2] = c_est;
                 cq[3] = c_skip;
-                cq[4] = c_exact;
+                cq[4] = c_exa - c_skip;
                 cq[5] = c_adm;
                 cq[6] = c_up;
                 cq[7] = c_gath;
@@ -1744,7 +1525,7 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
         __syncwarp();
     }
     if constexpr (COOP) {
-        if (lane == 0) meta[7] = COOP_EXIT;
+        if (lane == 0) meta[3] = COOP_EXIT;
         coop_bar(1);
     }
 }
