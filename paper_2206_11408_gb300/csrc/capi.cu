@@ -70,12 +70,11 @@ int search_uq_len(const DevIndex& ix, int mode) {
     return code_mode(mode) ? std::max(r_pad, 16 * ix.hks) : r_pad;
 }
 
-int search_smem_per_warp(const DevIndex& ix, int mode, int ef_cap, int H, int NPL, int h16) {
+int search_smem_per_warp(const DevIndex& ix, int mode, int ef_cap, int H, int NPL, int h16,
+                         bool own_qs) {
     const int r_pad = ix.r4 * 4;
     const int uq_len = search_uq_len(ix, mode);
     const int qs_len = mode == FINGER_MODE_FINGER_LP ? ix.m8 * 8 : ix.m4 * 4;
-    // the code modes keep the staged query in a region of its own
-    const bool own_qs = code_mode(mode);
     const int qs_bytes = own_qs ? 4 * ((qs_len + 3) & ~3) : 0;
     const int tile = mode == FINGER_MODE_FINGER_MLP ? 2 * 16 * (ix.mlp_kp + MLP_PAD) : 0;
     const int yo = mode == FINGER_MODE_FINGER_MLP ? 4 * 32 * NPL : 0;   // predictor outputs
@@ -244,8 +243,11 @@ finger_status make_plan(finger_index* ix, int mode, int ef_max, int64_t nq, Sear
     p->NPL = ix->deg0 > 32 ? 2 : 1;
     p->ef_cap = (ef_max + 3) & ~3;
     if (H <= 0) H = pow2ceil(std::min(std::max(16 * ef_max, 512), 2048));
+    // the code modes, and every mode with long rows, keep the staged query in a
+    // region of its own; else it is staged in the hash region
+    const bool own_qs = code_mode(mode) || p->VPL >= LONG_VPL;
     if (mode == FINGER_MODE_FINGER_LP) H = std::max(H, pow2ceil(2 * p->ef_cap));
-    else H = std::max(H, pow2ceil(ix->m_pad));   // the query is staged in the hash region
+    else H = std::max(H, pow2ceil(ix->m_pad));
     p->H = H;
     // 16-bit visited slots: ids must fit the bucket index plus 15 bits
     // (n <= 4096 H), and what reuses the table's H / 2 words must fit there:
@@ -254,13 +256,12 @@ finger_status make_plan(finger_index* ix, int mode, int ef_max, int64_t nq, Sear
     p->h16 = ix->visited_bits != 32 && ix->n <= 4096 * (int64_t)H &&
              (mode == FINGER_MODE_FINGER_LP ? H >= 4 * p->ef_cap : H >= 2 * ix->m_pad);
     p->wpb = wpb;
-    p->smem_per_warp = search_smem_per_warp(d, mode, p->ef_cap, p->H, p->NPL, p->h16);
+    p->smem_per_warp = search_smem_per_warp(d, mode, p->ef_cap, p->H, p->NPL, p->h16, own_qs);
     p->blk_smem = 0;
     p->occ = occ_force;
     if (plan_smem(*p) > 227 * 1024) return FINGER_ERR_UNSUPPORTED;
-    // the kernel variant with the most resident blocks that shared memory admits:
-    // 8 blocks (64 registers, plain mode), 6 (80 registers, plain, FP32 FINGER,
-    // LP and FP16 codes), else 5 (96 registers)
+    // the variant with the most resident blocks that shared memory admits, among
+    // those the mode and shape have (has_variant in search_impl.cuh)
     int bps = 0;
     p->occ = 5;
     if (occ_force > 0) {
@@ -306,27 +307,24 @@ finger_status make_plan(finger_index* ix, int mode, int ef_max, int64_t nq, Sear
 // warps per SM, so that is 8 warps for up to 2 queries per SM, 4 for up to 4, 2
 // for up to 8 (fewer where shared memory limits the blocks).  Measured per
 // launch, one warp per query against the rule's pick:
-//   m = 960 FP16 codes, ef 300: 5.16 -> 2.49 ms at 304 queries, 5.91 -> 3.09
-//   at 608, 6.05 -> 3.79 at 1,216; plain 7.68 -> 2.01, 8.82 -> 2.60, 9.01 -> 3.39
-//   m = 128 FP16 codes, ef 140: 0.90 -> 0.83 ms at 304, 0.90 -> 0.86 at 608, but
-//   0.94 -> 0.97 at 1,216; plain, ef 122: 0.91 -> 0.57, 0.93 -> 0.63, 1.01 -> 0.85
-// Larger batches lose with short rows (m = 128 FP16 codes, 2,000 queries: 0.99
-// -> 1.64 ms).  Rows above 2 KB take a warp several load rounds each, so two
-// warps per query stay ahead there (2,000 / 4,000 / 10,000 queries: 7.5 -> 5.5,
-// 10.1 -> 8.5, 15.7 -> 15.8 ms; plain 11.4 -> 5.1, 12.4 -> 7.8, 22.3 -> 15.5).
+//   m = 960 FP16 codes, ef 300: 3.13 -> 1.90 ms at 304 queries, 3.62 -> 2.45 at
+//   608, 3.75 -> 3.15 at 1,216; plain 3.58 -> 2.18 at 608, 3.74 -> 3.00 at 1,216
+//   m = 128 FP16 codes, ef 140: 0.71 -> 0.62 ms at 304, 0.71 -> 0.65 at 608;
+//   plain, ef 122: 0.61 -> 0.46 at 608, 0.67 -> 0.62 at 1,216
+// Beyond one wave it loses (m = 960, 1,500 queries: 4.46 -> 4.62 ms; m = 128,
+// 1,500: 0.80 -> 1.23), and 2 warps bring the code modes nothing with short rows,
+// whose few survivors fit one warp's pass (m = 128, 1,216 queries: 0.767 ->
+// 0.777 ms; m = 100 LP 1.26 -> 1.33).
 void make_coop_plan(finger_index* ix, int ef_max, int64_t nq, SearchPlan* p) {
-    const bool long_rows = p->G == 32 && p->VPL >= 8;
-    const bool code_short = code_mode(p->mode) && !long_rows;
-    for (int W = COOP_MAX_WARPS; W >= 2; W >>= 1) {
-        if (W == 2 && code_short) return;
-        const bool last = W == 2 && long_rows;
-        if (nq > (int64_t)ix->num_sms * (2 * COOP_MAX_WARPS / W) && !last) continue;
+    const int narrowest = code_mode(p->mode) && p->G < 32 ? 4 : 2;
+    for (int W = COOP_MAX_WARPS; W >= narrowest; W >>= 1) {
+        if (nq > (int64_t)ix->num_sms * (2 * COOP_MAX_WARPS / W)) continue;
         SearchPlan t;
         if (make_plan(ix, p->mode, ef_max, nq, &t, W, p->H, COOP_OCC, p->shape) != FINGER_OK) {
             cudaGetLastError();
             return;
         }
-        if (last || nq <= (int64_t)ix->num_sms * t.bps) {
+        if (nq <= (int64_t)ix->num_sms * t.bps) {
             *p = t;
             return;
         }

@@ -121,6 +121,9 @@ __host__ __device__ constexpr int rows_in_flight(int G, int VPL) {
     return (32 / G) * rows_per_group(VPL);
 }
 
+// chunks per lane from which every mode keeps the staged query in shared memory
+constexpr int LONG_VPL = 8;
+
 struct SearchPlan {
     int mode;
     int G, VPL, NPL;
@@ -150,7 +153,8 @@ inline int64_t plan_slots(const SearchPlan& p) {
 // kernels / launchers (search.cu)
 cudaError_t launch_search(const DevIndex& ix, const SearchArgs& a, const SearchPlan& p,
                           cudaStream_t s);
-int search_smem_per_warp(const DevIndex& ix, int mode, int ef_cap, int H, int NPL, int h16);
+int search_smem_per_warp(const DevIndex& ix, int mode, int ef_cap, int H, int NPL, int h16,
+                         bool own_qs);
 cudaError_t search_occupancy(const DevIndex& ix, const SearchPlan& p, int* blocks_per_sm);
 void choose_groups(int nchunks, int* G, int* VPL);
 

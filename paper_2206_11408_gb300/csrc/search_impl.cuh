@@ -35,6 +35,8 @@
 // exactly the per-neighbour one of Algorithm 4.
 #pragma once
 
+#include <type_traits>
+
 #include "internal.cuh"
 
 namespace fg {
@@ -95,77 +97,83 @@ __device__ __forceinline__ void bf16x8(const uint4& x, float* f) {
     }
 }
 
-// partial sum of (q - x)^2 over this lane's chunks of row `id`
-template <bool LP, int G, int VPL>
-__device__ __forceinline__ float row_partial(const QRegs<LP, VPL>& q, const DevIndex& ix,
-                                             uint32_t id, int kin) {
-    float acc = 0.f;
-    if constexpr (!LP) {
-        const float4* row = ix.X + (size_t)id * ix.m4;
-        float4 x[VPL];
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-            const int ch = kin + G * v;
-            x[v] = ch < ix.m4 ? __ldg(row + ch) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-            float d;
-            d = q.v[v][0] - x[v].x; acc = fmaf(d, d, acc);
-            d = q.v[v][1] - x[v].y; acc = fmaf(d, d, acc);
-            d = q.v[v][2] - x[v].z; acc = fmaf(d, d, acc);
-            d = q.v[v][3] - x[v].w; acc = fmaf(d, d, acc);
-        }
-    } else {
-        const uint4* row = ix.Xh + (size_t)id * ix.m8;
-        uint4 x[VPL];
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-            const int ch = kin + G * v;
-            x[v] = ch < ix.m8 ? __ldg(row + ch) : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-            float f[8];
-            bf16x8(x[v], f);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float d = q.v[v][e] - f[e];
-                acc = fmaf(d, d, acc);
-            }
-        }
-    }
-    return acc;
-}
-
-// exact distances of the rows nbs[lst[i]], i < nlist, into xb[lst[i]].  With
-// QS the lane's query chunks are read from the staged query qs (shared
-// memory) for this call only instead of living in registers for the whole
-// search (the FP16-code mode, whose code block needs the registers).
-// wq of W warps take the rows in turn, a pass of RPW rows each (a lone warp: 0
-// of 1); every row's sum is formed the same way whichever warp takes it.
+// exact distances of the rows nbs[lst[i]], i < nlist, into xb[lst[i]]: groups
+// of G lanes per row, VPL 16-byte chunks per lane, U rows per group and pass.
+// All loads of a pass are issued before the first product: with the row's
+// validity as a condition around its whole sum, each row group waited for its
+// own loads in turn (a pass of 8 rows of 512 bytes took 4,000 cycles unloaded).
+// With QS the query chunks are read from the staged query qs (shared memory) as
+// they are used instead of living in registers (the code modes, whose code
+// block needs the registers).  wq of W warps take the rows in turn, a pass of
+// RPW rows each (a lone warp: 0 of 1); every row's sum is formed the same way
+// whichever warp takes it.
 template <bool LP, int G, int VPL, bool QS = false>
-__device__ __forceinline__ void exact_list(const QRegs<LP, VPL>& qr, const float* qs,
+__device__ __forceinline__ void exact_list(const QRegs<LP, VPL>& q, const float* qs,
                                            const DevIndex& ix, const uint32_t* nbs,
                                            const int* lst, int nlist, float* xb, int lane,
                                            uint32_t idm = 0xFFFFFFFFu, int wq = 0, int W = 1) {
-    QRegs<LP, VPL> qt;
-    if constexpr (QS) load_qregs<LP, G, VPL>(qt, qs, LP ? ix.m8 : ix.m4, lane % G);
-    const QRegs<LP, VPL>& q = QS ? qt : qr;
     constexpr int RPW = 32 / G;
     constexpr int U = rows_per_group(VPL);   // rows per group in flight
+    constexpr int E = LP ? 8 : 4;            // elements per chunk
+    using Chunk = std::conditional_t<LP, uint4, float4>;
     const int grp = lane / G, kin = lane % G;
+    const int nch = LP ? ix.m8 : ix.m4;
+    const Chunk* X;
+    if constexpr (LP) X = ix.Xh;
+    else X = ix.X;
     for (int base = wq * RPW; base < nlist; base += U * RPW * W) {
         int o[U];
-        float p[U];
+        Chunk x[U][VPL];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int i = base + u * RPW * W + grp;
             o[u] = i < nlist ? lst[i] : -1;
-        }
+            const uint32_t id = (uint32_t)CK(nbs[CK(max(o[u], 0), 64, 1018)] & idm, ix.n, 1019);
+            const Chunk* row = X + (size_t)id * nch;
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            p[u] = o[u] >= 0 ? row_partial<LP, G, VPL>(q, ix, (uint32_t)CK(nbs[CK(o[u], 64, 1018)] & idm, ix.n, 1019), kin) : 0.f;
+            for (int v = 0; v < VPL; ++v) {
+                const int ch = kin + G * v;
+                x[u][v] = o[u] >= 0 && ch < nch ? __ldg(row + ch) : Chunk{};
+            }
+        }
+        float p[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) p[u] = 0.f;
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+            float qv[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) qv[e] = q.v[v][e];
+            if constexpr (QS) {
+                const int ch = kin + G * v;
+#pragma unroll
+                for (int e = 0; e < E; e += 4) {
+                    const float4 y = ch < nch ? *reinterpret_cast<const float4*>(qs + ch * E + e)
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+                    qv[e] = y.x;
+                    qv[e + 1] = y.y;
+                    qv[e + 2] = y.z;
+                    qv[e + 3] = y.w;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                float f[E];
+                if constexpr (LP) {
+                    bf16x8(x[u][v], f);
+                } else {
+                    f[0] = x[u][v].x;
+                    f[1] = x[u][v].y;
+                    f[2] = x[u][v].z;
+                    f[3] = x[u][v].w;
+                }
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const float d = qv[e] - f[e];
+                    p[u] = fmaf(d, d, p[u]);
+                }
+            }
+        }
 #pragma unroll
         for (int off = G / 2; off > 0; off >>= 1)
 #pragma unroll
@@ -823,10 +831,10 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
     const int uq_len = WB ? max(r_pad, 16 * WKS) : r_pad;
     float* pq = uq + uq_len;
     // the query staging buffer is only read before the visited hash is cleared,
-    // so outside the LP mode (which re-reads it for the FP32 re-rank) and the
-    // FP16-code mode (whose exact distances read it) it lives inside the hash
-    // region (the plan keeps its words >= m_pad)
-    constexpr bool QSM = LP || WB;   // query kept in its own region
+    // so outside the code modes and long rows (whose exact distances read it, and
+    // LP's re-rank) it lives inside the hash region (the plan keeps its words >=
+    // m_pad)
+    constexpr bool QSM = WB || VPL >= LONG_VPL;   // query kept in its own region
     float* qs = QSM ? pq + r_pad : reinterpret_cast<float*>(hash);
     __nv_bfloat16* xt = reinterpret_cast<__nv_bfloat16*>(QSM ? qs + ((qs_len + 3) & ~3) : pq + r_pad);   // predictor input tile
     if (FG_CHECKED) g_chk_err = a.err;   // same value from every thread
@@ -834,10 +842,16 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
     uint32_t* bitmap = a.bitmap + slot * a.words;
     uint32_t* spl = a.spill + slot * a.spill_cap;
     const int logNB = 31 - __clz(a.H >> (a.h16 ? 3 : 2));   // buckets of the visited hash
-    // the lane's query chunks stay in registers, except where the code block needs
-    // them (80 registers); the cooperative form has 128
-    constexpr bool QST = WB && !COOP;
+    // the lane's query chunks stay in registers, except where the code block or a
+    // long row's own chunks need them (80 registers); the cooperative form has 128
+    constexpr bool QST = QSM && !COOP;
     constexpr int ONE_PASS = rows_in_flight(G, VPL);   // rows one warp requests at once
+    // L2 prefetch of the survivors' rows as soon as the gate has passed them, ahead
+    // of the list and its passes: 1M x 128 plain 2.94 -> 2.66 ms, FP16 codes 3.09
+    // -> 2.96, m = 960 7.05 -> 6.60 (rows beyond the first pass only: 2.76, 3.05,
+    // 6.65).  Rows of at most 256 bytes do without (m = 100 BF16 3.62 -> 3.53 ms,
+    // m = 64 0.673 -> 0.657); helper warps prefetch their own.
+    constexpr bool PREFETCH = !COOP && G * VPL * 16 > 256;
 
     if constexpr (COOP) {
         if (wib != 0) {
@@ -1338,7 +1352,7 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
                 bool need = isnew[s] && (!use_est || !full0 || !(est > ub0));
                 if (HARV && hpos[s] >= 0) need = true;   // the record needs the exact distance
                 needr[s] = need;
-                if (!COOP && need) prefetch_row<LP>(ix, nb[s]);   // (helpers prefetch theirs)
+                if (PREFETCH && need) prefetch_row<LP>(ix, nb[s]);
                 es[s * 32 + lane] = est;
                 const unsigned bm = __ballot_sync(FULLMASK, need);
                 if (need) lst[CK(nl + __popc(bm & ltmask), 32 * NPL, 1017)] = s * 32 + lane;
@@ -1530,13 +1544,26 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
     }
 }
 
-// instantiate and dispatch one mode over the (G, VPL, NPL) variants and the
-// resident-block target: COOP_OCC (search_coop_*.cu) one block per query, else
-// 5 blocks of 4 warps (96 registers) everywhere, 6 (80
-// registers) for the plain, FINGER, LP and FP16/FP8-code modes, 8 (64 registers)
-// for the plain mode.  The FINGER modes keep their gathers in flight in
-// registers and are fastest at 6 (the FP16-code mode measured slower at 7,
-// where it spills); plain search at 8.
+// Instantiate and dispatch one mode over the (G, VPL, NPL) variants and the
+// resident-block target OCC: COOP_OCC (search_coop_*.cu) one query per block;
+// else blocks of 4 warps per SM, which sets the registers: 5 blocks (96)
+// everywhere, 6 (80) in all but the predictor and harvest modes, 8 (64) for
+// plain search and FP8 codes.  A pass of exact rows needs 16 VPL registers for
+// its loads in flight and a code block 32, so
+//   * 64 registers serve one chunk per lane only (rows of at most 64 floats:
+//     10,000 x 64 plain 519 us against 540 at 80); with two, 1M x 128 plain
+//     took 2.87 ms against 2.65 at 80 registers and 2.75 at 96;
+//   * code modes with more than 32 links (two slots per lane) spill at 80:
+//     m = 100, 48 links, FP16 codes 3.24 ms against 3.08 at 96, LP 3.68 against
+//     3.59; with 32 links 80 registers win (1M x 128 FP16 codes 2.97 against
+//     3.29, plain as above).
+template <int MODE, int OCC>
+constexpr bool has_variant(int VPL, int NPL) {
+    const bool codes = MODE == MODE_F16_K2 || MODE == MODE_F16_K4 || MODE == MODE_LP_K2 ||
+                       MODE == MODE_LP_K4 || MODE == MODE_F8_K2 || MODE == MODE_F8_K4;
+    return OCC == 8 ? VPL == 1 && !(codes && NPL > 1) : OCC == 6 ? !(codes && NPL > 1) : true;
+}
+
 #define LP_MODE(m) ((m) == MODE_LP_K2 || (m) == MODE_LP_K4 || (m) == MODE_F8_K2 || (m) == MODE_F8_K4)
 
 template <int MODE, int OCC>
@@ -1545,6 +1572,7 @@ cudaError_t launch_occ(const DevIndex& ix, const SearchArgs& a, const SearchPlan
     const int smem = plan_smem(p);
     const dim3 grid(p.blocks), block(p.wpb * 32);
 #define FG_CASE(G_, V_, N_)                                                                    \
+    if constexpr (has_variant<MODE, OCC>(V_, N_))                                              \
     if (p.G == G_ && p.VPL == V_ && p.NPL == N_) {                                           \
         auto k = k_search<MODE, G_, V_, N_, OCC>;                                              \
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); \
@@ -1566,6 +1594,7 @@ template <int MODE, int OCC>
 cudaError_t occupancy_occ(const SearchPlan& p, int* blocks) {
     const int smem = plan_smem(p);
 #define FG_CASE(G_, V_, N_)                                                                    \
+    if constexpr (has_variant<MODE, OCC>(V_, N_))                                              \
     if (p.G == G_ && p.VPL == V_ && p.NPL == N_) {                                           \
         auto k = k_search<MODE, G_, V_, N_, OCC>;                                              \
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); \
