@@ -5,28 +5,34 @@
 // accumulators in tensor memory) with each FP32 operand split into a BF16 high
 // part and a BF16 low part: q.x ~ qh.xh + qh.xl + ql.xh (the dropped ql.xl and
 // the rounding of the parts are ~2^-17 of |q||x|).  Every query row keeps the
-// K' smallest approximate distances of its base segment; a second kernel then
-// recomputes the candidates' distances exactly in FP32 (sum of (q - x)^2) and
-// returns the K best by (distance, id), so the result is the exact kNN unless
-// more than K' - K rows lie within the approximation error of the K-th
-// distance.
+// K' smallest approximate distances of its share of the base; a second kernel
+// takes the K' smallest of all shares, recomputes their distances exactly in
+// FP32 (sum of (q - x)^2) and returns the K best by (distance, id), so the
+// result is the exact kNN unless more than K' - K rows lie within the
+// approximation error of the K-th distance.
 //
 // k_knn_tc is persistent (one CTA per SM) and warp-specialised:
-//   warp 0     TMA producer: 64-column (128-byte, SWIZZLE_128B) chunks of the
-//              query tile (hi, lo) and the base tile (hi, lo) into a 2-stage ring
+//   warp 0     TMA producer: the query tile (hi, lo), resident in shared memory
+//              for the whole job where m <= 128, and 64-column (128-byte,
+//              SWIZZLE_128B) chunks of the base tiles (hi, lo) into a ring;
+//              longer rows stream the query's chunks through the ring as well
 //   warp 1     MMA issuer (one elected lane): 3 products x 4 K-steps per chunk
 //              into one of two 128x128 FP32 accumulators in tensor memory
 //   warps 2-5  epilogue: tcgen05.ld of the accumulator (thread = query row),
-//              distances and their per-row minimum against the row's K'-th
-//              distance; the few rows with a smaller one are transposed
-//              through shared memory and their new candidates inserted into
-//              the row's sorted K' list by the whole warp (ballot for the
-//              position, shuffle for the shift); the accumulator is handed
-//              back through an mbarrier
-// Work items are (query tile of 128, segment of base tiles), so small query
-// batches still fill the GPU.  Every mbarrier wait is bounded: on a timeout the
-// kernel raises an error flag, every role leaves its loop, and tensor memory is
-// released.
+//              distances and their minimum against the row's K'-th distance;
+//              where some row of the warp has a smaller one, every thread
+//              appends its own to its row's pending buffer
+// A row's K' candidates are (distance, id) pairs in shared memory, in eight
+// groups whose largest keys its thread holds in registers; once some row of a
+// warp has more than 16 pending, all 32 rows insert theirs side by side, a thread
+// per row (replace the largest key, find its group's next, then the row's).  A
+// warp-wide insertion of one candidate into one row's sorted list took 260 cycles
+// and bounded the launch: the causal candidate search over 200k x 128 rows spent
+// 145 ms there; now 35 ms (an insertion for 32 rows at once takes 500 cycles).
+//
+// Work is dealt out in items of one query tile and one base segment: contiguous
+// segments for a kNN launch, base tiles s, s + nseg, ... for the causal one.  Every mbarrier wait is bounded: on a timeout the kernel raises an
+// error flag, every role leaves its loop, and tensor memory is released.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
@@ -43,33 +49,69 @@ namespace {
 constexpr int TQ = 128;                      // query rows per tile (MMA M)
 constexpr int TB = 128;                      // base rows per tile (MMA N)
 constexpr int KCH = 64;                      // K elements per chunk (128 bytes of BF16)
-constexpr int STAGES = 2;
 constexpr int PART = TQ * 128;               // one 128-row x 128-byte operand part: 16 KB
-constexpr int STAGE_BYTES = 4 * PART;        // qh, ql, xh, xl
+constexpr int MAX_STAGES = 4;
+constexpr int PEND = 32;                     // pending candidates per row
+constexpr int QRES_CHUNKS = 2;               // query tiles up to this many chunks stay resident
 constexpr int TC_THREADS = 192;
 constexpr long WAIT_TRIES = 1L << 21;
+
+using u64 = unsigned long long;
+// candidate key: distance bits mapped to unsigned order, then the id (a kept
+// distance is finite).  NO_KEY and above: none
+constexpr u64 NO_KEY = 0xFF800000FFFFFFFFull;
+
+__device__ __forceinline__ uint32_t ord_of(float d) {
+    const uint32_t b = __float_as_uint(d);
+    return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
+}
+__device__ __forceinline__ float dist_of(u64 k) {
+    const uint32_t o = (uint32_t)(k >> 32);
+    return __uint_as_float(o ^ (o & 0x80000000u ? 0x80000000u : 0xFFFFFFFFu));
+}
 
 struct TcArgs {
     int64_t nq, n;
     int nchunk;           // ceil(m / 64)
     int nbt;              // base tiles
-    int nseg;             // base segments per query tile; segment s holds the base
-                          // tiles s, s + nseg, s + 2 nseg, ... (interleaved)
+    int nseg;             // segments of the base: contiguous, or (causal) the tiles s,
+                          // s + nseg, ...
     int nqt;              // query tiles
     int causal;           // 1: queries are the base rows, row i sees base rows < i
+    int stages;
     const float* qn;      // ||q||^2 (FP32), nq
     const float* xn;      // ||x||^2 (FP32), n
-    int32_t* cand;        // nq x nseg x KP candidate ids (-1 = none)
-    float* cand_d;        // optional: their approximate distances
+    u64* keys;            // nq x nseg x KP candidate keys
+    uint32_t* bound;      // optional: per row, the smallest K'-th distance of its finished
+                          // segments (ord_of), 0xFFFFFFFF before the first
     int* err;             // device status word (FINGER_ERR_LIMIT on a wait timeout)
 };
 
-// work item -> (query tile, segment): the largest causal items first
-__device__ __forceinline__ void item_of(const TcArgs& a, int item, int& qt, int& seg, int& bt_end) {
-    qt = a.causal ? a.nqt - 1 - item / a.nseg : item / a.nseg;
-    seg = item % a.nseg;
-    bt_end = a.causal ? min(a.nbt, qt + 1) : a.nbt;
-}
+// a CTA's jobs, the same sequence for every role: (query tile, segment) items
+struct Jobs {
+    const TcArgs& a;
+    int at;
+    __device__ __forceinline__ explicit Jobs(const TcArgs& a_) : a(a_), at(blockIdx.x) {}
+    // query tile, base tiles b0, b0 + step, ... < b1, segment
+    __device__ __forceinline__ bool next(int& qt, int& b0, int& b1, int& step, int& seg) {
+        if (at >= a.nqt * a.nseg) return false;
+        if (a.causal) {   // the largest items first
+            qt = a.nqt - 1 - at / a.nseg;
+            seg = at % a.nseg;
+            b0 = seg;
+            b1 = min(a.nbt, qt + 1);
+            step = a.nseg;
+        } else {          // the query tiles of one segment next to each other
+            qt = at % a.nqt;
+            seg = at / a.nqt;
+            b0 = (int)((int64_t)a.nbt * seg / a.nseg);
+            b1 = (int)((int64_t)a.nbt * (seg + 1) / a.nseg);
+            step = 1;
+        }
+        at += gridDim.x;
+        return true;
+    }
+};
 
 __device__ __forceinline__ uint32_t s32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -118,8 +160,9 @@ __device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap* map, int
         : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-    uint32_t r[32];
+// 32 columns of this thread's tensor-memory lane; the registers hold them after
+// tmem_wait32, which takes them as operands so that no use moves ahead of it
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
         "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
@@ -129,36 +172,116 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
           "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
           "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+__device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
+                   "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
+                   "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]),
+                   "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]),
+                   "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]));
 }
 
+// (qn + xa) - 2 ra, (qn + xb) - 2 rb, each rounded as its scalar form is
+__device__ __forceinline__ void dist2(float qn, float xa, float xb, uint32_t ra, uint32_t rb,
+                                      float& va, float& vb) {
+    asm("{\n .reg .b64 q, x, r, n;\n mov.b64 q, {%2, %2};\n mov.b64 x, {%3, %4};\n"
+        " mov.b64 r, {%5, %6};\n mov.b64 n, {%7, %7};\n add.rn.f32x2 x, q, x;\n"
+        " fma.rn.f32x2 x, n, r, x;\n mov.b64 {%0, %1}, x;\n}\n"
+        : "=f"(va), "=f"(vb)
+        : "f"(qn), "f"(xa), "f"(xb), "r"(ra), "r"(rb), "f"(-2.f));
+}
+
+// Candidates of one row: slot i is dist[128 i] (ord_of bits) and id[128 i], group g
+// holds the slots g GS .. g GS + GS - 1; gm: the groups' largest distances, gs:
+// their places (4 bits each).  The choices go by distance alone, one 32-bit
+// maximum per step; equal ones are told apart by id on a path of their own.
 template <int KP>
+struct RowTop {
+    static constexpr int GS = KP / 8;
+    uint32_t *dist, *id;
+    uint32_t gm[8], root, gs;
+    int g;   // group of the root
+
+    __device__ __forceinline__ uint32_t* id_at(int grp, int place) const {
+        return id + 128 * (GS * grp + place);
+    }
+    __device__ __forceinline__ uint32_t place_of(int grp) const { return (gs >> (4 * grp)) & 15u; }
+    __device__ __forceinline__ uint32_t root_id() const { return *id_at(g, place_of(g)); }
+    __device__ __forceinline__ void clear() {
+        for (int i = 0; i < KP; ++i) {
+            dist[128 * i] = 0xFFFFFFFFu - i;   // above +inf, and distinct
+            id[128 * i] = 0xFFFFFFFFu;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) gm[i] = 0xFFFFFFFFu - i * GS;
+        gs = 0u;
+        root = 0xFFFFFFFFu;
+        g = 0;
+    }
+    // the largest key gives way to (d, i), which is smaller
+    __device__ __forceinline__ void insert(uint32_t d, uint32_t i) {
+        const int at = 128 * (GS * g + (int)place_of(g));
+        dist[at] = d;
+        id[at] = i;
+        const uint32_t* grp = dist + 128 * GS * g;
+        uint32_t k[GS], m = 0u, same = 0u;
+#pragma unroll
+        for (int j = 0; j < GS; ++j) k[j] = grp[128 * j];
+#pragma unroll
+        for (int j = 0; j < GS; ++j) m = max(m, k[j]);
+#pragma unroll
+        for (int j = 0; j < GS; ++j) same |= k[j] == m ? 1u << j : 0u;
+        int p = __ffs(same) - 1;
+        for (same &= same - 1; same; same &= same - 1) {   // equal distances: the larger id
+            const int o = __ffs(same) - 1;
+            if (*id_at(g, o) > *id_at(g, p)) p = o;
+        }
+        gs = (gs & ~(15u << (4 * g))) | ((uint32_t)p << (4 * g));
+        root = 0u;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            gm[j] = j == g ? m : gm[j];
+            root = max(root, gm[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) same |= gm[j] == root ? 1u << j : 0u;
+        g = __ffs(same) - 1;
+        for (same &= same - 1; same; same &= same - 1) {
+            const int o = __ffs(same) - 1;
+            if (*id_at(o, place_of(o)) > root_id()) g = o;
+        }
+    }
+};
+
+template <int KP, bool QRES>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_knn_tc(const __grid_constant__ CUtensorMap tqh, const __grid_constant__ CUtensorMap tql,
              const __grid_constant__ CUtensorMap txh, const __grid_constant__ CUtensorMap txl,
              TcArgs a) {
     static_assert(KP == 32 || KP == 64, "candidate lists of 32 or 64");
+    constexpr int STAGE_BYTES = QRES ? 2 * PART : 4 * PART;        // [qh, ql,] xh, xl
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* stages = sm;                                   // STAGES x 64 KB
-    float* Ld = reinterpret_cast<float*>(sm + STAGES * STAGE_BYTES);   // 128 x KP (row-major)
-    int32_t* Li = reinterpret_cast<int32_t*>(Ld + KP * TQ);
-    float* Bs = reinterpret_cast<float*>(Li + KP * TQ);                // 4 x 32 x 33
-    uint64_t* bars = reinterpret_cast<uint64_t*>(Bs + 4 * 32 * 33);   // full[2] empty[2] accf[2] acce[2]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 8);
+    unsigned char* qres = sm;                                      // nchunk x (qh, ql)
+    unsigned char* stages = sm + (QRES ? a.nchunk * 2 * PART : 0);
+    uint32_t* lists = reinterpret_cast<uint32_t*>(stages + (size_t)a.stages * STAGE_BYTES);
+    // lists: KP x 128 distances, then ids; PEND x 128 pending (distance, id)
+    uint2* pend = reinterpret_cast<uint2*>(lists + 2 * KP * TQ);
+    float* xns = reinterpret_cast<float*>(pend + PEND * TQ);                        // 4 x 64 norms
+    uint64_t* bars = reinterpret_cast<uint64_t*>(xns + 4 * 64);
+    // full[4] empty[4] accf[2] acce[2] qfull qempty
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_STAGES + 6);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t full0 = s32(bars), empty0 = s32(bars + 2), accf0 = s32(bars + 4),
-                   acce0 = s32(bars + 6);
+    const uint32_t full0 = s32(bars), empty0 = s32(bars + MAX_STAGES),
+                   accf0 = s32(bars + 2 * MAX_STAGES), acce0 = accf0 + 16, qfull = accf0 + 32,
+                   qempty = accf0 + 40;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < 2; ++i) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8 * i));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(empty0 + 8 * i));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(accf0 + 8 * i));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 128;" ::"r"(acce0 + 8 * i));
+        for (int i = 0; i < 2 * MAX_STAGES + 6; ++i) {
+            const int count = i == 2 * MAX_STAGES + 2 || i == 2 * MAX_STAGES + 3 ? 128 : 1;   // acce
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full0 + 8 * i), "r"(count));
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -172,28 +295,45 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
-    const int items = a.nqt * a.nseg;
+    Jobs jobs(a);
+    int qt, b0, b1, step, seg;
 
     if (warp == 0) {
         if (lane == 0) {
-            uint32_t it = 0;
-            for (int item = blockIdx.x; item < items && !*abort_flag; item += gridDim.x) {
-                int qt, seg, bt_end;
-                item_of(a, item, qt, seg, bt_end);
-                for (int bt = seg; bt < bt_end && !*abort_flag; bt += a.nseg)
-                    for (int c = 0; c < a.nchunk; ++c, ++it) {
-                        const int s = it % STAGES;
-                        const uint32_t ph = (it / STAGES) & 1u;
-                        if (!wait_bar(empty0 + 8 * s, ph ^ 1u, abort_flag, a.err)) break;
+            uint32_t s = 0, ph = 1u, job = 0;   // ring slot and its parity for `empty`
+            while (!*abort_flag && jobs.next(qt, b0, b1, step, seg)) {
+                if (b0 >= b1) continue;
+                if (QRES) {
+                    if (!wait_bar(qempty, (job & 1u) ^ 1u, abort_flag, a.err)) break;
+                    ++job;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(qfull),
+                                 "r"(a.nchunk * 2 * PART)
+                                 : "memory");
+                    for (int c = 0; c < a.nchunk; ++c) {
+                        const uint32_t dst = s32(qres + (size_t)c * 2 * PART);
+                        tma_2d(dst, &tqh, c * KCH, qt * TQ, qfull);
+                        tma_2d(dst + PART, &tql, c * KCH, qt * TQ, qfull);
+                    }
+                }
+                for (int bt = b0; bt < b1 && !*abort_flag; bt += step)
+                    for (int c = 0; c < a.nchunk; ++c) {
+                        if (!wait_bar(empty0 + 8 * s, ph, abort_flag, a.err)) break;
                         const uint32_t fb = full0 + 8 * s;
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
                                      "r"(STAGE_BYTES)
                                      : "memory");
-                        const uint32_t dst = s32(stages + (size_t)s * STAGE_BYTES);
-                        tma_2d(dst, &tqh, c * KCH, qt * TQ, fb);
-                        tma_2d(dst + PART, &tql, c * KCH, qt * TQ, fb);
-                        tma_2d(dst + 2 * PART, &txh, c * KCH, bt * TB, fb);
-                        tma_2d(dst + 3 * PART, &txl, c * KCH, bt * TB, fb);
+                        uint32_t dst = s32(stages + (size_t)s * STAGE_BYTES);
+                        if (!QRES) {
+                            tma_2d(dst, &tqh, c * KCH, qt * TQ, fb);
+                            tma_2d(dst + PART, &tql, c * KCH, qt * TQ, fb);
+                            dst += 2 * PART;
+                        }
+                        tma_2d(dst, &txh, c * KCH, bt * TB, fb);
+                        tma_2d(dst + PART, &txl, c * KCH, bt * TB, fb);
+                        if (++s == (uint32_t)a.stages) {
+                            s = 0;
+                            ph ^= 1u;
+                        }
                     }
             }
         }
@@ -202,26 +342,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             // D F32, A BF16, B BF16, K-major A and B, N = 128, M = 128
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TB >> 3) << 17) |
                                    ((uint32_t)(TQ >> 4) << 24);
-            uint32_t it = 0, tile = 0;
-            for (int item = blockIdx.x; item < items && !*abort_flag; item += gridDim.x) {
-                int qt, seg, bt_end;
-                item_of(a, item, qt, seg, bt_end);
-                for (int bt = seg; bt < bt_end && !*abort_flag; bt += a.nseg, ++tile) {
+            uint32_t s = 0, ph = 0u, job = 0, tile = 0;
+            while (!*abort_flag && jobs.next(qt, b0, b1, step, seg)) {
+                if (b0 >= b1) continue;
+                if (QRES) {
+                    if (!wait_bar(qfull, job & 1u, abort_flag, a.err)) break;
+                    ++job;
+                }
+                for (int bt = b0; bt < b1 && !*abort_flag; bt += step, ++tile) {
                     const uint32_t b = tile & 1u, tph = (tile >> 1) & 1u;
                     if (!wait_bar(acce0 + 8 * b, tph ^ 1u, abort_flag, a.err)) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t d = tmem + b * TB;
-                    for (int c = 0; c < a.nchunk; ++c, ++it) {
-                        const int s = it % STAGES;
-                        const uint32_t ph = (it / STAGES) & 1u;
+                    for (int c = 0; c < a.nchunk; ++c) {
                         if (!wait_bar(full0 + 8 * s, ph, abort_flag, a.err)) break;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t base = s32(stages + (size_t)s * STAGE_BYTES);
+                        const uint32_t st = s32(stages + (size_t)s * STAGE_BYTES);
+                        const uint32_t qb = QRES ? s32(qres + (size_t)c * 2 * PART) : st;
+                        const uint32_t xb = QRES ? st : st + 2 * PART;
 #pragma unroll
                         for (int k = 0; k < KCH / 16; ++k) {
-                            const uint64_t qh = sdesc(base + 32 * k), ql = sdesc(base + PART + 32 * k);
-                            const uint64_t xh = sdesc(base + 2 * PART + 32 * k),
-                                           xl = sdesc(base + 3 * PART + 32 * k);
+                            const uint64_t qh = sdesc(qb + 32 * k), ql = sdesc(qb + PART + 32 * k);
+                            const uint64_t xh = sdesc(xb + 32 * k), xl = sdesc(xb + PART + 32 * k);
                             mma_bf16_tc(d, qh, xh, idesc, (c | k) != 0);
                             mma_bf16_tc(d, qh, xl, idesc, 1u);
                             mma_bf16_tc(d, ql, xh, idesc, 1u);
@@ -230,151 +372,151 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                             "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                                 empty0 + 8 * s)
                             : "memory");
+                        if (++s == (uint32_t)a.stages) {
+                            s = 0;
+                            ph ^= 1u;
+                        }
                     }
                     asm volatile(
                         "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                             accf0 + 8 * b)
                         : "memory");
                 }
+                if (QRES)   // the job's products have read the query tile
+                    asm volatile(
+                        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                            qempty)
+                        : "memory");
             }
         }
     } else {
         // epilogue: warp w owns the query rows 32 (w % 4) + lane of every tile
-        // (the tensor-memory lanes it may read).  Per 32-column block a thread
-        // forms its row's 32 distances and their minimum; only rows whose
-        // minimum beats their K'-th distance go on, through a transpose in
-        // shared memory, to a warp-wide insertion into the row's sorted list.
+        // (the tensor-memory lanes it may read), thread = row
         const int quarter = warp & 3;
         const int row = 32 * quarter + lane;
-        float* B = Bs + (warp - 2) * 32 * 33;               // 32 x 32 transpose, padded
-        float* Lw = Ld + (size_t)quarter * 32 * KP;          // this warp's 32 lists, row-major
-        int32_t* Lwi = Li + (size_t)quarter * 32 * KP;
+        RowTop<KP> top;
+        top.dist = lists + row;
+        top.id = lists + KP * TQ + row;
+        uint2* pr = pend + row;
+        float* xs = xns + 64 * quarter;
         uint32_t tile = 0;
-        for (int item = blockIdx.x; item < items && !*abort_flag; item += gridDim.x) {
-            int qt, seg, bt_end;
-            item_of(a, item, qt, seg, bt_end);
+        bool stop = false;   // a wait timed out (the same in all lanes: they vote below)
+        while (!stop && jobs.next(qt, b0, b1, step, seg)) {
             const int64_t q0 = (int64_t)qt * TQ;
             const int64_t qi = q0 + row;
             const int64_t id_end = a.causal ? min(qi, a.n) : a.n;   // ids below this count
             const int64_t lim = a.causal ? min(q0, a.n) : a.n;      // smallest id_end of the tile
             const float qn = qi < a.nq ? a.qn[qi] : 0.f;
-            float thr = qi < a.nq ? INFINITY : -INFINITY;            // K'-th distance of the row
-            for (int k = lane; k < 32 * KP; k += 32) {
-                Lw[k] = INFINITY;
-                Lwi[k] = -1;
-            }
-            __syncwarp();
-            for (int bt = seg; bt < bt_end; bt += a.nseg, ++tile) {
+            // only distances below thr count: the row's K'-th here, and from the start
+            // what the row's finished segments say (their K'-th smallest is no
+            // smaller than the whole base's; equal distances still count, by id)
+            uint32_t bound = 0xFF800000u;
+            if (a.bound && qi < a.nq) bound = min(bound, *(volatile uint32_t*)(a.bound + qi));
+            const float cap = bound < 0xFF800000u ? dist_of((u64)(bound + 1u) << 32) : INFINITY;
+            float thr = qi < a.nq ? cap : -INFINITY;
+            int cnt = 0;                                    // pending candidates of the row
+            top.clear();
+            auto flush = [&]() {
+                const int most = __reduce_max_sync(0xffffffffu, cnt);
+                for (int p = 0; p < most; ++p) {
+                    if (p >= cnt) continue;
+                    const uint2 e = pr[128 * p];
+                    const uint32_t d = ord_of(__uint_as_float(e.x));
+                    if (d < top.root || (d == top.root && e.y < top.root_id())) top.insert(d, e.y);
+                }
+                cnt = 0;
+                // (a list that is not full: its root is a NaN's bits, and cap stays)
+                if (qi < a.nq) thr = fminf(cap, dist_of((u64)top.root << 32));
+            };
+            // a tile's 128 base norms, four per lane, requested two tiles ahead: behind
+            // the base tiles' own traffic a load takes over 1,000 cycles (half a tile
+            // ahead the epilogue waited for them, 8.3 ms of a launch of 10.9)
+            auto norms = [&](int bt) {
+                const int64_t id = (int64_t)bt * TB + 4 * lane;
+                if (id + 4 <= a.n) return __ldg(reinterpret_cast<const float4*>(a.xn + id));
+                return make_float4(id < a.n ? __ldg(a.xn + id) : 0.f,
+                                   id + 1 < a.n ? __ldg(a.xn + id + 1) : 0.f,
+                                   id + 2 < a.n ? __ldg(a.xn + id + 2) : 0.f, 0.f);
+            };
+            float4 xnow, x1 = norms(b0), x2 = norms(b0 + step);
+            for (int bt = b0; bt < b1; bt += step, ++tile) {
                 const uint32_t b = tile & 1u, tph = (tile >> 1) & 1u;
-                if (!wait_bar(accf0 + 8 * b, tph, abort_flag, a.err)) break;
+                xnow = x1;
+                x1 = x2;
+                x2 = norms(bt + 2 * step);
+                stop = !__all_sync(0xffffffffu, wait_bar(accf0 + 8 * b, tph, abort_flag, a.err));
+                if (stop) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t tbase = tmem + ((uint32_t)(32 * quarter) << 16) + b * TB;
                 const bool masked = (int64_t)(bt + 1) * TB > lim;
-                for (int c0 = 0; c0 < TB; c0 += 32) {
+                uint32_t r[32];
+                tmem_ld32(tbase, r);
+                // one warp per scheduler: 32 columns per step for independent work, and
+                // a loop that fits the instruction cache (unrolled over the tile the
+                // launch took 1.5x)
+#pragma unroll 1
+                for (int c = 0; c < TB; c += 32) {
+                    const int64_t id0 = (int64_t)bt * TB + c;
+                    if (!(c & 63)) {   // half a tile's norms
+                        __syncwarp();
+                        if (lane >> 4 == c >> 6) reinterpret_cast<float4*>(xs)[lane & 15] = xnow;
+                        __syncwarp();
+                    }
+                    float4 x[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        x[j] = reinterpret_cast<const float4*>(xs + (c & 32))[j];
+                    tmem_wait32(r);
                     float v[32];
-                    tmem_ld32(tbase + c0, v);
-                    const int64_t id0 = (int64_t)bt * TB + c0;
-                    if (!masked) {
-                        const float4* x4 = reinterpret_cast<const float4*>(a.xn + id0);
 #pragma unroll
-                        for (int j4 = 0; j4 < 8; ++j4) {
-                            const float4 x = __ldg(x4 + j4);
-                            v[4 * j4] = fmaf(-2.f, v[4 * j4], qn + x.x);
-                            v[4 * j4 + 1] = fmaf(-2.f, v[4 * j4 + 1], qn + x.y);
-                            v[4 * j4 + 2] = fmaf(-2.f, v[4 * j4 + 2], qn + x.z);
-                            v[4 * j4 + 3] = fmaf(-2.f, v[4 * j4 + 3], qn + x.w);
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const int64_t id = id0 + j;
-                            v[j] = id < id_end ? fmaf(-2.f, v[j], qn + __ldg(a.xn + id)) : INFINITY;
-                        }
+                    for (int j = 0; j < 8; ++j) {
+                        dist2(qn, x[j].x, x[j].y, r[4 * j], r[4 * j + 1], v[4 * j], v[4 * j + 1]);
+                        dist2(qn, x[j].z, x[j].w, r[4 * j + 2], r[4 * j + 3], v[4 * j + 2], v[4 * j + 3]);
                     }
-                    float mn = v[0];
+                    if (masked) {   // (norms() fills the last tile's padding with 0)
 #pragma unroll
-                    for (int j = 1; j < 32; ++j) mn = fminf(mn, v[j]);
-                    unsigned rows = __ballot_sync(0xffffffffu, mn < thr);
-                    if (!rows) continue;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) B[j * 33 + lane] = v[j];
-                    __syncwarp();
-                    while (rows) {
-                        const int r = __ffs(rows) - 1;
-                        rows &= rows - 1;
-                        float t = __shfl_sync(0xffffffffu, thr, r);
-                        const float dj = B[lane * 33 + r];           // column lane of row r
-                        unsigned hit = __ballot_sync(0xffffffffu, dj < t);
-                        float* Lr = Lw + r * KP;
-                        int32_t* Lir = Lwi + r * KP;
-                        float d0 = Lr[lane], d1 = INFINITY;
-                        int32_t i0 = Lir[lane], i1 = -1;
-                        if (KP == 64) {
-                            d1 = Lr[lane + 32];
-                            i1 = Lir[lane + 32];
-                        }
-                        while (hit) {
-                            const int c = __ffs(hit) - 1;
-                            hit &= hit - 1;
-                            const float cd = __shfl_sync(0xffffffffu, dj, c);
-                            if (!(cd < t)) continue;
-                            const int32_t cid = (int32_t)(id0 + c);
-                            // ids grow along the scan, so equal distances already
-                            // in the list come first: position = #entries <= cd
-                            int pos = __popc(__ballot_sync(0xffffffffu, d0 <= cd));
-                            if (KP == 64) pos += __popc(__ballot_sync(0xffffffffu, d1 <= cd));
-                            const float u0 = __shfl_up_sync(0xffffffffu, d0, 1);
-                            const int32_t ui0 = __shfl_up_sync(0xffffffffu, i0, 1);
-                            if (KP == 64) {
-                                float u1 = __shfl_up_sync(0xffffffffu, d1, 1);
-                                int32_t ui1 = __shfl_up_sync(0xffffffffu, i1, 1);
-                                const float t31 = __shfl_sync(0xffffffffu, d0, 31);
-                                const int32_t ti31 = __shfl_sync(0xffffffffu, i0, 31);
-                                if (lane == 0) {
-                                    u1 = t31;
-                                    ui1 = ti31;
-                                }
-                                if (lane + 32 > pos) {
-                                    d1 = u1;
-                                    i1 = ui1;
-                                } else if (lane + 32 == pos) {
-                                    d1 = cd;
-                                    i1 = cid;
-                                }
-                            }
-                            if (lane > pos) {
-                                d0 = u0;
-                                i0 = ui0;
-                            } else if (lane == pos) {
-                                d0 = cd;
-                                i0 = cid;
-                            }
-                            t = __shfl_sync(0xffffffffu, KP == 64 ? d1 : d0, 31);
-                        }
-                        Lr[lane] = d0;
-                        Lir[lane] = i0;
-                        if (KP == 64) {
-                            Lr[lane + 32] = d1;
-                            Lir[lane + 32] = i1;
-                        }
-                        if (lane == r) thr = t;
+                        for (int j = 0; j < 32; ++j) v[j] = id0 + j < id_end ? v[j] : INFINITY;
                     }
-                    __syncwarp();
+                    if (c + 32 < TB) tmem_ld32(tbase + c + 32, r);   // behind the checks
+                    float mn[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float t[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            t[j] = fminf(fminf(v[16 * h + j], v[16 * h + 4 + j]),
+                                         fminf(v[16 * h + 8 + j], v[16 * h + 12 + j]));
+                        mn[h] = fminf(fminf(t[0], t[1]), fminf(t[2], t[3]));
+                    }
+                    if (!__any_sync(0xffffffffu, fminf(mn[0], mn[1]) < thr)) continue;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (!__any_sync(0xffffffffu, mn[h] < thr)) continue;
+                        // append (at most 16 pending here, 32 afterwards).  Ids grow along the
+                        // scan, so an equal distance already listed comes first.
+                        uint2* w = pr + 128 * cnt;
+#pragma unroll
+                        for (int j = 16 * h; j < 16 * h + 16; ++j) {
+                            const bool hit = v[j] < thr;
+                            if (hit) *w = make_uint2(__float_as_uint(v[j]), (uint32_t)id0 + j);
+                            w += hit ? 128 : 0;
+                        }
+                        cnt = (int)(w - pr) >> 7;
+                        if (__any_sync(0xffffffffu, cnt > PEND - 16)) flush();
+                    }
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acce0 + 8 * b) : "memory");
             }
-            __syncwarp();
-            for (int r = 0; r < 32; ++r) {
-                const int64_t qr = q0 + 32 * quarter + r;
-                if (qr >= a.nq) break;
-                const size_t o = ((size_t)qr * a.nseg + seg) * KP;
-                for (int k = lane; k < KP; k += 32) {
-                    a.cand[o + k] = Lwi[r * KP + k];
-                    if (a.cand_d) a.cand_d[o + k] = Lw[r * KP + k];
-                }
+            flush();
+            if (qi < a.nq) {
+                if (a.bound) atomicMin(a.bound + qi, top.root);
+                u64* out = a.keys + ((size_t)qi * a.nseg + seg) * KP;
+                for (int k = 0; k < KP; k += 2)
+                    *reinterpret_cast<uint4*>(out + k) =
+                        make_uint4(top.id[128 * k], top.dist[128 * k], top.id[128 * (k + 1)],
+                                   top.dist[128 * (k + 1)]);
             }
-            __syncwarp();
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -403,101 +545,180 @@ __global__ void k_split_bf16(const float* __restrict__ X, int64_t rows, int m, i
     if (norm2 && lane == 0) norm2[w] = acc;
 }
 
-// exact FP32 distances of every query's candidates and the K best by
-// (distance, id); one warp per query
-__global__ void k_rerank(const float4* __restrict__ X, int m4, const float* __restrict__ Q, int m,
-                         int64_t nq, const int32_t* __restrict__ cand, int nc, int K,
-                         int64_t* out_ids, float* out_d) {
-    extern __shared__ float rr_s[];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
-    if (q >= nq) return;
-    float* cd = rr_s + (size_t)wib * 2 * nc;
-    int32_t* ci = reinterpret_cast<int32_t*>(cd + nc);
-    const float* qr = Q + (size_t)q * m;
-    for (int i = 0; i < nc; ++i) {
-        const int32_t id = cand[(size_t)q * nc + i];
-        float acc = 0.f;
-        if (id >= 0) {
-            const float4* xr = X + (size_t)id * m4;
-            for (int k = lane; k < m4; k += 32) {
-                const float4 x = __ldg(xr + k);
-                const int e = 4 * k;
-                float dlt;
-                if (e < m) { dlt = qr[e] - x.x; acc = fmaf(dlt, dlt, acc); }
-                if (e + 1 < m) { dlt = qr[e + 1] - x.y; acc = fmaf(dlt, dlt, acc); }
-                if (e + 2 < m) { dlt = qr[e + 2] - x.z; acc = fmaf(dlt, dlt, acc); }
-                if (e + 3 < m) { dlt = qr[e + 3] - x.w; acc = fmaf(dlt, dlt, acc); }
-            }
+__device__ __forceinline__ u64 warp_min(u64 k) {
+    const uint32_t hi = __reduce_min_sync(0xffffffffu, (uint32_t)(k >> 32));
+    const uint32_t lo =
+        __reduce_min_sync(0xffffffffu, (uint32_t)(k >> 32) == hi ? (uint32_t)k : 0xFFFFFFFFu);
+    return (u64)hi << 32 | lo;
+}
+
+// The R smallest of a warp's 32 E distinct keys (E per lane, destroyed), ascending,
+// into out[0..R); NO_KEY where there are fewer
+template <int E>
+__device__ __forceinline__ void warp_smallest(u64 (&k)[E], int R, u64* out, int lane) {
+    for (int r = 0; r < R; ++r) {
+        u64 m = k[0];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        for (int j = 1; j < E; ++j) m = k[j] < m ? k[j] : m;
+        m = warp_min(m);
+        if (m >= NO_KEY) {
+            for (int i = r + lane; i < R; i += 32) out[i] = NO_KEY;
+            break;
         }
-        if (lane == 0) {
-            cd[i] = id >= 0 ? acc : INFINITY;
-            ci[i] = id;
-        }
+#pragma unroll
+        for (int j = 0; j < E; ++j) k[j] = k[j] == m ? NO_KEY : k[j];
+        if (lane == 0) out[r] = m;
     }
     __syncwarp();
-    // rank of every candidate among the valid ones by (distance, id)
-    for (int i = lane; i < nc; i += 32) {
-        const float di = cd[i];
-        const int32_t ii = ci[i];
-        if (ii < 0) continue;
+}
+
+// Final step of a kNN launch: the KP smallest approximate keys of a query's lists,
+// their exact FP32 distances, the K best by (distance, id).  W warps per query
+// (E keys per lane: 32 E W >= the query's keys); with W = 1 four queries per block.
+template <int W, int E>
+__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
+    k_rerank(const float4* __restrict__ X, int m4, const float* __restrict__ Q, int m, int64_t nq,
+             const u64* __restrict__ keys, int nc, int KP, int K, int64_t* out_ids, float* out_d) {
+    constexpr int QPB = W == 1 ? 4 : 1;
+    __shared__ u64 sel_s[QPB][64];
+    __shared__ u64 part_s[W == 1 ? 1 : W * 64];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int64_t q = W == 1 ? (int64_t)blockIdx.x * 4 + wib : (int64_t)blockIdx.x;
+    const int wq = W == 1 ? 0 : wib;
+    if (q >= nq) return;
+    u64* sel = sel_s[W == 1 ? wib : 0];
+    const u64* kr = keys + (size_t)q * nc;
+    u64 k[E];
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        const int c = (j * W + wq) * 32 + lane;
+        k[j] = c < nc ? kr[c] : NO_KEY;
+    }
+    if constexpr (W == 1) {
+        warp_smallest<E>(k, KP, sel, lane);
+    } else {
+        warp_smallest<E>(k, KP, part_s + wq * KP, lane);
+        __syncthreads();
+        if (wq == 0) {
+            u64 k2[2 * W];
+#pragma unroll
+            for (int j = 0; j < 2 * W; ++j)
+                k2[j] = 32 * j + lane < W * KP ? part_s[32 * j + lane] : NO_KEY;
+            warp_smallest<2 * W>(k2, KP, sel, lane);
+        }
+        __syncthreads();
+    }
+    // exact distances, four rows in flight per warp; each key gets its exact distance
+    const float* qr = Q + (size_t)q * m;
+    constexpr int U = 4;
+    for (int i = wq * U; i < KP; i += W * U) {
+        uint32_t id[U];
+        float acc[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            id[u] = (uint32_t)sel[i + u];
+            acc[u] = 0.f;
+        }
+        for (int c = lane; c < m4; c += 32) {
+            float4 x[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                x[u] = (int32_t)id[u] >= 0 ? __ldg(X + (size_t)id[u] * m4 + c)
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+            const int e = 4 * c;
+            float qv[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) qv[t] = e + t < m ? qr[e + t] : 0.f;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                float dlt;
+                dlt = qv[0] - x[u].x; acc[u] = fmaf(dlt, dlt, acc[u]);
+                dlt = qv[1] - x[u].y; acc[u] = fmaf(dlt, dlt, acc[u]);
+                dlt = qv[2] - x[u].z; acc[u] = fmaf(dlt, dlt, acc[u]);
+                dlt = qv[3] - x[u].w; acc[u] = fmaf(dlt, dlt, acc[u]);
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < U; ++u) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+        __syncwarp();
+        if (lane < U && (int32_t)(uint32_t)sel[i + lane] >= 0) {
+            const float d = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
+            sel[i + lane] = (u64)ord_of(d) << 32 | (uint32_t)sel[i + lane];
+        }
+    }
+    if constexpr (W == 1) __syncwarp();
+    else __syncthreads();
+    if (wq != 0) return;
+    for (int i = lane; i < KP; i += 32) {
+        const u64 ki = sel[i];
         int rank = 0;
-        for (int j = 0; j < nc; ++j) {
-            const int32_t ij = ci[j];
-            if (ij < 0) continue;
-            rank += cd[j] < di || (cd[j] == di && ij < ii);
+        for (int j = 0; j < KP; ++j) {
+            const u64 kj = sel[j];
+            rank += kj < ki || (kj == ki && j < i);   // (only NO_KEYs are equal)
         }
         if (rank < K) {
-            out_ids[(size_t)q * K + rank] = ii;
-            out_d[(size_t)q * K + rank] = di;
+            const bool ok = (int32_t)(uint32_t)ki >= 0;
+            out_ids[(size_t)q * K + rank] = ok ? (int64_t)(uint32_t)ki : (int64_t)-1;
+            out_d[(size_t)q * K + rank] = ok ? dist_of(ki) : INFINITY;
         }
-    }
-    __syncwarp();
-    // pad when fewer than K valid candidates
-    int valid = 0;
-    for (int j = lane; j < nc; j += 32) valid += ci[j] >= 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) valid += __shfl_xor_sync(0xffffffffu, valid, o);
-    for (int k = valid + lane; k < K; k += 32) {
-        out_ids[(size_t)q * K + k] = -1;
-        out_d[(size_t)q * K + k] = INFINITY;
     }
 }
 
-// Merge of the segments' candidate lists by approximate distance: the K
-// smallest (distance, id) of every row, int64 ids (-1 padded); one warp per row
-__global__ void k_merge_topk(const int32_t* __restrict__ cand, const float* __restrict__ cand_d,
-                             int64_t rows, int nc, int K, int64_t* out_ids, float* out_d) {
-    const int lane = threadIdx.x & 31;
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= rows) return;
-    const int32_t* ci = cand + (size_t)w * nc;
-    const float* cd = cand_d + (size_t)w * nc;
-    int valid = 0;
-    for (int i = lane; i < nc; i += 32) {
-        const int32_t ii = ci[i];
-        if (ii < 0) continue;
-        valid++;
-        const float di = cd[i];
-        int rank = 0;
-        for (int j = 0; j < nc; ++j) {
-            const int32_t ij = ci[j];
-            if (ij < 0) continue;
-            const float dj = cd[j];
-            rank += dj < di || (dj == di && ij < ii);
-        }
-        if (rank < K) {
-            out_ids[(size_t)w * K + rank] = ii;
-            out_d[(size_t)w * K + rank] = di;
+// ascending bitonic sort of a warp's 32 E keys; lane l holds places E l .. E l + E - 1
+template <int E>
+__device__ __forceinline__ void warp_sort(u64 (&k)[E], int lane) {
+#pragma unroll
+    for (int size = 2; size <= 32 * E; size <<= 1) {
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            if (stride >= E) {   // between lanes
+                const int ls = stride / E;
+                const bool up = (lane & (size / E)) == 0;
+                const bool low = (lane & ls) == 0;
+#pragma unroll
+                for (int j = 0; j < E; ++j) {
+                    const u64 o = __shfl_xor_sync(0xffffffffu, k[j], ls);
+                    k[j] = (up == low) == (o < k[j]) ? o : k[j];
+                }
+            } else {   // within the lane
+#pragma unroll
+                for (int j = 0; j < E; ++j)
+                    if (!(j & stride)) {
+                        const bool up = size < E ? (j & size) == 0 : (lane & (size / E)) == 0;
+                        const u64 x = k[j], y = k[j | stride];
+                        const bool sw = up == (y < x);
+                        k[j] = sw ? y : x;
+                        k[j | stride] = sw ? x : y;
+                    }
+            }
         }
     }
+}
+
+// The K smallest keys of every row's 512 candidates, ascending, as int64 ids (-1
+// padded) and approximate distances; one warp per row sorts them in registers
+// (ranking every candidate against all others took 20 ms for 200k rows)
+__global__ void __launch_bounds__(128) k_merge_topk(const u64* __restrict__ keys, int64_t rows,
+                                                    int K, int64_t* out_ids, float* out_d) {
+    constexpr int E = 16;
+    __shared__ u64 s[4][32 * (E + 1)];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int64_t w = (int64_t)blockIdx.x * 4 + wib;
+    if (w >= rows) return;
+    u64 k[E];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) valid += __shfl_xor_sync(0xffffffffu, valid, o);
-    for (int k = valid + lane; k < K; k += 32) {
-        out_ids[(size_t)w * K + k] = -1;
-        out_d[(size_t)w * K + k] = INFINITY;
+    for (int j = 0; j < E; ++j) k[j] = keys[(size_t)w * 32 * E + 32 * j + lane];
+    warp_sort<E>(k, lane);
+#pragma unroll
+    for (int j = 0; j < E; ++j) s[wib][lane * (E + 1) + j] = k[j];
+    __syncwarp();
+    for (int i = lane; i < K; i += 32) {
+        const u64 x = s[wib][i / E * (E + 1) + i % E];
+        const bool ok = (int32_t)(uint32_t)x >= 0;
+        out_ids[(size_t)w * K + i] = ok ? (int64_t)(uint32_t)x : (int64_t)-1;
+        out_d[(size_t)w * K + i] = ok ? dist_of(x) : INFINITY;
     }
 }
 
@@ -527,18 +748,19 @@ bool make_map(CUtensorMap* map, const void* base, int64_t rows, int m, int ms) {
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int KP>
-size_t tc_smem() {
-    return 1024 + (size_t)STAGES * STAGE_BYTES + (size_t)KP * TQ * 8 + 4 * 32 * 33 * 4 + 8 * 8 + 16;
-}
-
-template <int KP>
+// ring stages that the shared memory beside the heaps, pending buffers and a
+// resident query tile holds (at least two: 224 KB at KP = 64)
+template <int KP, bool QRES>
 cudaError_t run_tc(const CUtensorMap* maps, TcArgs a, int grid, cudaStream_t s) {
-    const size_t smem = tc_smem<KP>();
-    cudaError_t e = cudaFuncSetAttribute(k_knn_tc<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const size_t fixed = 1024 + (size_t)(KP + PEND) * TQ * 8 + 4 * 64 * 4 + 8 * (2 * MAX_STAGES + 6) +
+                         16 + (QRES ? (size_t)a.nchunk * 2 * PART : 0);
+    const size_t stage = (QRES ? 2 : 4) * PART;
+    a.stages = (int)std::min<size_t>(MAX_STAGES, (227 * 1024 - fixed) / stage);
+    const size_t smem = fixed + a.stages * stage;
+    cudaError_t e = cudaFuncSetAttribute(k_knn_tc<KP, QRES>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_knn_tc<KP><<<grid, TC_THREADS, smem, s>>>(maps[0], maps[1], maps[2], maps[3], a);
+    k_knn_tc<KP, QRES><<<grid, TC_THREADS, smem, s>>>(maps[0], maps[1], maps[2], maps[3], a);
     return cudaGetLastError();
 }
 
@@ -569,15 +791,15 @@ cudaError_t ensure_split(finger_index* ix, cudaStream_t s) {
 
 // one launch of k_knn_tc over nq query rows (BF16 parts qh/ql) against the base
 cudaError_t run_items(finger_index* ix, const __nv_bfloat16* qh, const __nv_bfloat16* ql,
-                      const float* qn, int64_t nq, int KP, int nseg, bool causal, int32_t* cand,
-                      float* cand_d, cudaStream_t s) {
+                      const float* qn, int64_t nq, int KP, int nseg, bool causal, u64* keys,
+                      uint32_t* bound, cudaStream_t s) {
     const int m = ix->m, ms = (m + 7) & ~7;
     const int64_t n = ix->n;
     CUtensorMap maps[4];
     if (!make_map(&maps[0], qh, nq, m, ms) || !make_map(&maps[1], ql, nq, m, ms) ||
         !make_map(&maps[2], ix->xs_hi, n, m, ms) || !make_map(&maps[3], ix->xs_lo, n, m, ms))
         return cudaErrorInvalidValue;
-    TcArgs a;
+    TcArgs a{};
     a.nq = nq;
     a.n = n;
     a.nchunk = (m + KCH - 1) / KCH;
@@ -587,11 +809,39 @@ cudaError_t run_items(finger_index* ix, const __nv_bfloat16* qh, const __nv_bflo
     a.causal = causal ? 1 : 0;
     a.qn = qn;
     a.xn = ix->xnorm2;
-    a.cand = cand;
-    a.cand_d = cand_d;
+    a.keys = keys;
+    a.bound = bound;
     a.err = ix->err;
     const int grid = (int)std::min<int64_t>(ix->num_sms, (int64_t)a.nqt * nseg);
-    return KP == 32 ? run_tc<32>(maps, a, grid, s) : run_tc<64>(maps, a, grid, s);
+    const bool res = a.nchunk <= QRES_CHUNKS;
+    if (KP == 32) return res ? run_tc<32, true>(maps, a, grid, s) : run_tc<32, false>(maps, a, grid, s);
+    return res ? run_tc<64, true>(maps, a, grid, s) : run_tc<64, false>(maps, a, grid, s);
+}
+
+// Base segments of a kNN launch.  The items (query tile, segment) are dealt to one
+// CTA per SM in waves, segment by segment, so the CTAs of a wave scan the same rows
+// at the same time: a segment of at most 48 MB of BF16 parts stays in L2 for
+// them.  (One equal range of the (query tile, base tile) sequence per CTA balances
+// without waves, but each CTA then scans rows of its own and DRAM bounds it: 10,000
+// queries x 1M x 128 took 11.6 ms.)  From there the smallest count whose last
+// wave costs at most 3 %, or the best of the next 32; each segment adds a list of
+// K' per row to fill and to merge.
+int base_segments(const finger_index* ix, int nqt, int nbt) {
+    const int64_t bytes = (int64_t)nbt * TB * ((ix->m + 7) & ~7) * 4;
+    const int lo = (int)std::min<int64_t>(nbt, std::max<int64_t>(bytes / (48 << 20), 1));
+    const int64_t G = ix->num_sms;
+    int best = lo;
+    double best_eff = 0;
+    for (int S = lo; S <= std::min<int64_t>(nbt, std::max<int64_t>(lo + 32, (G + nqt - 1) / nqt)); ++S) {
+        const int64_t items = (int64_t)nqt * S;
+        const double eff = (double)items / ((items + G - 1) / G * G);
+        if (eff > best_eff + 0.002) {
+            best_eff = eff;
+            best = S;
+        }
+        if (best_eff >= 0.97) break;
+    }
+    return best;
 }
 
 }  // namespace
@@ -606,41 +856,46 @@ cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, i
     const int KP = K <= 16 ? 32 : 64;
     const int nqt = (int)((nq + TQ - 1) / TQ);
     const int nbt = (int)((n + TB - 1) / TB);
-    // enough (query tile, base segment) items for two per SM, at most 64
-    // segments; any segmentation is exact here because K <= KP
-    const int nseg = std::max(1, std::min({nbt, 64, (2 * ix->num_sms + nqt - 1) / nqt}));
+    const int nseg = base_segments(ix, nqt, nbt);   // any is exact here: K <= KP
     const int nc = nseg * KP;
     __nv_bfloat16 *qh = nullptr, *ql = nullptr;
     float* qn = nullptr;
-    int32_t* cand = nullptr;
-    if (cudaMallocAsync(&qh, sizeof(__nv_bfloat16) * (size_t)nq * ms, s) != cudaSuccess ||
+    u64* keys = nullptr;
+    uint32_t* bound = nullptr;
+    if (cudaMallocAsync(&bound, sizeof(uint32_t) * (size_t)nq, s) != cudaSuccess ||
+        cudaMallocAsync(&qh, sizeof(__nv_bfloat16) * (size_t)nq * ms, s) != cudaSuccess ||
         cudaMallocAsync(&ql, sizeof(__nv_bfloat16) * (size_t)nq * ms, s) != cudaSuccess ||
         cudaMallocAsync(&qn, sizeof(float) * (size_t)nq, s) != cudaSuccess ||
-        cudaMallocAsync(&cand, sizeof(int32_t) * (size_t)nq * nc, s) != cudaSuccess) {
+        cudaMallocAsync(&keys, sizeof(u64) * (size_t)nq * nc, s) != cudaSuccess) {
         e = cudaErrorMemoryAllocation;
         goto done;
     }
+    if ((e = cudaMemsetAsync(bound, 0xFF, sizeof(uint32_t) * (size_t)nq, s)) != cudaSuccess) goto done;
     k_split_bf16<<<(unsigned)((nq * 32 + 255) / 256), 256, 0, s>>>(Q, nq, m, m, ms, qh, ql, qn);
     if ((e = cudaGetLastError()) != cudaSuccess) goto done;
-    if ((e = run_items(ix, qh, ql, qn, nq, KP, nseg, false, cand, nullptr, s)) != cudaSuccess)
+    if ((e = run_items(ix, qh, ql, qn, nq, KP, nseg, false, keys, bound, s)) != cudaSuccess)
         goto done;
     {
-        const int wpb = nc > 1024 ? 1 : 4;
-        const size_t smem = (size_t)wpb * 2 * nc * sizeof(float);
-        if (smem > 48 * 1024 &&
-            (e = cudaFuncSetAttribute(k_rerank, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem)) != cudaSuccess)
-            goto done;
-        k_rerank<<<(unsigned)((nq + wpb - 1) / wpb), 32 * wpb, smem, s>>>(
-            reinterpret_cast<const float4*>(ix->X), ix->m4, Q, m, nq, cand, nc, K, out_ids, out_d);
-        e = cudaGetLastError();
+        const float4* X = reinterpret_cast<const float4*>(ix->X);
+        // a query tile's lists: a few for large batches, up to one per SM for small ones
+#define FG_RERANK(W_, E_)                                                                        \
+    k_rerank<W_, E_><<<(unsigned)(W_ == 1 ? (nq + 3) / 4 : nq), W_ == 1 ? 128 : 32 * W_, 0, s>>>( \
+        X, ix->m4, Q, m, nq, keys, nc, KP, K, out_ids, out_d)
+        if (nc <= 32 * 4) FG_RERANK(1, 4);
+        else if (nc <= 32 * 16) FG_RERANK(1, 16);
+        else if (nc <= 8 * 32 * 16) FG_RERANK(8, 16);
+        else if (nc <= 16 * 32 * 32) FG_RERANK(16, 32);
+        else e = cudaErrorInvalidValue;   // (more than 256 SMs)
+#undef FG_RERANK
+        if (e == cudaSuccess) e = cudaGetLastError();
     }
 done:
     // stream-ordered frees: the temporaries live until the kernels above finish
     if (qh) cudaFreeAsync(qh, s);
     if (ql) cudaFreeAsync(ql, s);
     if (qn) cudaFreeAsync(qn, s);
-    if (cand) cudaFreeAsync(cand, s);
+    if (bound) cudaFreeAsync(bound, s);
+    if (keys) cudaFreeAsync(keys, s);
     return e;
 }
 
@@ -659,23 +914,18 @@ cudaError_t launch_knn_tc_causal(finger_index* ix, int K, int64_t* out_ids, floa
     cudaError_t e = ensure_split(ix, s);
     if (e != cudaSuccess) return e;
     constexpr int KP = 64, NSEG = 8;
-    const int nc = NSEG * KP;
-    int32_t* cand = nullptr;
-    float* cand_d = nullptr;
-    if (cudaMallocAsync(&cand, sizeof(int32_t) * (size_t)n * nc, s) != cudaSuccess ||
-        cudaMallocAsync(&cand_d, sizeof(float) * (size_t)n * nc, s) != cudaSuccess) {
+    u64* keys = nullptr;
+    if (cudaMallocAsync(&keys, sizeof(u64) * (size_t)n * NSEG * KP, s) != cudaSuccess) {
         e = cudaErrorMemoryAllocation;
         goto done;
     }
-    if ((e = run_items(ix, ix->xs_hi, ix->xs_lo, ix->xnorm2, n, KP, NSEG, true, cand, cand_d, s)) !=
+    if ((e = run_items(ix, ix->xs_hi, ix->xs_lo, ix->xnorm2, n, KP, NSEG, true, keys, nullptr, s)) !=
         cudaSuccess)
         goto done;
-    k_merge_topk<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(cand, cand_d, n, nc, K, out_ids,
-                                                                 out_d);
+    k_merge_topk<<<(unsigned)((n + 3) / 4), 128, 0, s>>>(keys, n, K, out_ids, out_d);
     e = cudaGetLastError();
 done:
-    if (cand) cudaFreeAsync(cand, s);
-    if (cand_d) cudaFreeAsync(cand_d, s);
+    if (keys) cudaFreeAsync(keys, s);
     return e;
 }
 

@@ -1,0 +1,36 @@
+"""Candidate lists, segments and merges of the tensor-core kNN at their edges.
+
+Rows and queries are small integers, so distances are exact in BF16 split products
+and in FP32 and many are equal: ids and distances must be exactly the K smallest
+(distance, id) keys.  Sizes: around a tile (128 rows), fewer rows than K or than the
+32 / 64 kept, queries around a query tile, one chunk of columns, two (the largest
+resident query tile) and three."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("m", [3, 64, 65, 128, 129])
+@pytest.mark.parametrize("n", [5, 127, 128, 129, 1000, 20011])
+def test_exact_keys_with_ties(n, m):
+    import torch
+
+    import paper_2206_11408_gb300 as fg
+
+    rng = np.random.default_rng(n + m)
+    X = rng.integers(0, 4, (n, m)).astype(np.float32)
+    Q = rng.integers(0, 4, (300, m)).astype(np.float32)
+    D = ((Q[:, None].astype(np.int64) - X[None, :2000].astype(np.int64)) ** 2).sum(-1) if n <= 2000 else \
+        (Q ** 2).sum(1).astype(np.int64)[:, None] + (X ** 2).sum(1).astype(np.int64)[None] - 2 * (Q @ X.T).astype(np.int64)
+    order = np.argsort(D * (1 << 20) + np.arange(n)[None], axis=1, kind="stable")
+    ix = fg.Index(X)
+    for nq in (1, 127, 129, 300):
+        for K in (1, 10, 16, 17, 40):
+            ids, d = ix.knn(torch.from_numpy(Q[:nq]).cuda(), K)
+            ix.sync()
+            k = min(K, n)
+            assert np.array_equal(ids.cpu().numpy()[:, :k], order[:nq, :k])
+            assert np.array_equal(d.cpu().numpy()[:, :k], np.take_along_axis(D[:nq], order[:nq, :k], 1))
+            assert (ids.cpu().numpy()[:, k:] == -1).all() and np.isinf(d.cpu().numpy()[:, k:]).all()
+    ix.close()
