@@ -834,8 +834,7 @@ finger_status finger_knn(finger_index* ix, const float* queries, int64_t nq, int
     if (K <= knn_tc_max_k())
         e = launch_knn_tc(ix, queries, nq, K, out_ids, out_dists, (cudaStream_t)stream);
     else
-        e = launch_knn(reinterpret_cast<const float4*>(ix->X), ix->n, ix->m4, queries, ix->m, ix->m,
-                       nq, K, false, nullptr, out_ids, out_dists, (cudaStream_t)stream);
+        e = launch_knn_big(ix, queries, nq, K, out_ids, out_dists, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? FINGER_ERR_OOM : FINGER_ERR_CUDA;

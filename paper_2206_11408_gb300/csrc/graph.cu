@@ -280,6 +280,8 @@ finger_status build_layer(finger_index* ix, const int32_t* d_nodes, int64_t cnt,
     }
     if (tensor && causal && !d_nodes)   // layer 0: causal candidates on the tensor cores
         CK(launch_knn_tc_causal(ix, kk, cid, cd, s));
+    else if (tensor && causal)          // an upper layer
+        CK(launch_knn_layer(ix, Xl, cnt, kk, d_nodes, cid, cd, s));
     else
         CK(launch_knn(d_nodes ? Xl : reinterpret_cast<const float4*>(ix->X), cnt, m4,
                       d_nodes ? reinterpret_cast<const float*>(Xl) : ix->X, (int64_t)m4 * 4,
@@ -415,7 +417,7 @@ finger_status build_graph(finger_index* ix, const finger_graph_params* p, cudaSt
             // upper layers are small: offer up to 256 exact candidates so that the
             // selection sees beyond a node's own cluster and keeps long links
             status = build_layer(ix, d_nodes, cnt, (int)std::min<int64_t>(cnt - 1, 256), M, M,
-                                 up_adj, M, d_rows, d_cmap, causal, false, s);
+                                 up_adj, M, d_rows, d_cmap, causal, p->fp32_candidates == 0, s);
             if (status != FINGER_OK) goto done;
         }
     }

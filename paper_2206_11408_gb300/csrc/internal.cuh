@@ -161,12 +161,17 @@ void choose_groups(int nchunks, int* G, int* VPL);
 // brute force (knn.cu); causal: query row i sees base rows < i only
 cudaError_t launch_knn(const float4* Xb, int64_t nb, int m4, const float* Q, int64_t q_stride,
                        int q_m, int64_t nq, int K, bool exclude_self, const int32_t* remap,
-                       int64_t* out_ids, float* out_d, cudaStream_t s, bool causal = false);
+                       int64_t* out_ids, float* out_d, cudaStream_t s, bool causal = false,
+                       const int32_t* only = nullptr);
 size_t knn_smem(int K);
 // tensor-core exact kNN (knn_tc.cu): K <= knn_tc_max_k()
 int knn_tc_max_k();
 cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, int64_t* out_ids,
                           float* out_d, cudaStream_t s);
+cudaError_t launch_knn_big(finger_index* ix, const float* Q, int64_t nq, int K, int64_t* out_ids,
+                           float* out_d, cudaStream_t s);
+cudaError_t launch_knn_layer(finger_index* ix, const float4* X, int64_t cnt, int K,
+                             const int32_t* remap, int64_t* out_ids, float* out_d, cudaStream_t s);
 cudaError_t launch_knn_tc_causal(finger_index* ix, int K, int64_t* out_ids, float* out_d,
                                  cudaStream_t s);
 

@@ -27,7 +27,8 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
                                             const float* __restrict__ Q, int64_t q_stride,
                                             int q_m, int64_t nq, int K, int exclude_self,
                                             int causal, const int32_t* __restrict__ remap,
-                                            int64_t* out_ids, float* out_d) {
+                                            int64_t* out_ids, float* out_d,
+                                            const int32_t* __restrict__ only) {
     extern __shared__ __align__(16) unsigned char sm[];
     float* Qs = reinterpret_cast<float*>(sm);          // KC x QB
     float* Xs = Qs + KC * QB;                          // KC x XB
@@ -39,9 +40,13 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
     float* thr_d = reinterpret_cast<float*>(li + QB * K);
     int* thr_i = reinterpret_cast<int*>(thr_d + QB);
     int* lsz = thr_i + QB;
+    __shared__ int64_t qid[QB];   // query of each of the block's rows (-1: none)
 
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t q0 = (int64_t)blockIdx.x * QB;
+    // `only`: the queries only[1 .. only[0]] instead of all nq
+    if (only) nq = only[0];
+    if (q0 >= nq) return;
     const int tq = t >> 5;     // 0..7 -> queries tq*4 .. +4
     const int tx = t & 31;     // 0..31 -> rows tx*4 .. +4
     for (int i = t; i < QB; i += NT) {
@@ -49,9 +54,16 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
         lsz[i] = 0;
         thr_d[i] = INFINITY;
         thr_i[i] = 0x7fffffff;
+        qid[i] = q0 + i >= nq ? -1 : only ? (int64_t)only[1 + q0 + i] : q0 + i;
     }
+    __syncthreads();
     const int m = m4 * 4;
-    const int64_t x_end = causal ? (q0 + QB < nb ? q0 + QB : nb) : nb;
+    int64_t x_end = nb;
+    if (causal) {
+        x_end = 0;
+        for (int i = 0; i < QB; ++i) x_end = max(x_end, qid[i]);   // rows below the last query
+        x_end = min(x_end, nb);
+    }
     for (int64_t x0 = 0; x0 < x_end; x0 += XB) {
         float acc[4][4];
 #pragma unroll
@@ -63,9 +75,9 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
             // stage Q chunk (transposed): QB x KC
             for (int i = t; i < QB * KC; i += NT) {
                 const int qq = i / KC, kk = i % KC;
-                const int64_t gq = q0 + qq;
+                const int64_t gq = qid[qq];
                 const int gk = k0 + kk;
-                Qs[kk * QB + qq] = (gq < nq && gk < q_m) ? Q[gq * q_stride + gk] : 0.f;
+                Qs[kk * QB + qq] = (gq >= 0 && gk < q_m) ? Q[gq * q_stride + gk] : 0.f;
             }
             // stage X chunk (transposed): XB rows x KC dims
             {
@@ -103,8 +115,8 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
             const int qq = tq * 4 + a;
-            const int64_t gq = q0 + qq;
-            if (gq >= nq) continue;
+            const int64_t gq = qid[qq];
+            if (gq < 0) continue;
             const int64_t self = exclude_self ? (remap ? (int64_t)remap[gq] : gq) : -1;
             const float td = thr_d[qq];
             const int ti = thr_i[qq];
@@ -173,8 +185,8 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
     }
     for (int i = t; i < QB * K; i += NT) {
         const int qq = i / K, k = i % K;
-        const int64_t gq = q0 + qq;
-        if (gq >= nq) continue;
+        const int64_t gq = qid[qq];
+        if (gq < 0) continue;
         const bool ok = k < lsz[qq];
         out_ids[gq * K + k] = ok ? (int64_t)li[qq * K + k] : (int64_t)-1;
         out_d[gq * K + k] = ok ? ld[qq * K + k] : INFINITY;
@@ -190,11 +202,12 @@ size_t knn_smem(int K) {
 
 // Q: nq rows with stride q_stride floats of which the first q_m are read (the
 // rest count as 0, matching the zero padding of the base rows).  remap (optional) maps base row -> id
-// reported (and query row -> its own id for exclusion).
+// reported (and query row -> its own id for exclusion).  only (optional, device): a
+// count and that many query rows, the only ones done.
 cudaError_t launch_knn(const float4* Xb, int64_t nb, int m4, const float* Q, int64_t q_stride,
                        int q_m, int64_t nq, int K, bool exclude_self,
                        const int32_t* remap, int64_t* out_ids, float* out_d, cudaStream_t s,
-                       bool causal) {
+                       bool causal, const int32_t* only) {
     if (nq == 0) return cudaSuccess;
     const size_t smem = knn_smem(K);
     cudaError_t e = cudaFuncSetAttribute(k_knn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -202,7 +215,7 @@ cudaError_t launch_knn(const float4* Xb, int64_t nb, int m4, const float* Q, int
     if (e != cudaSuccess) return e;
     const int64_t grid = (nq + QB - 1) / QB;
     k_knn<<<(unsigned)grid, NT, smem, s>>>(Xb, nb, m4, Q, q_stride, q_m, nq, K, exclude_self ? 1 : 0,
-                                           causal ? 1 : 0, remap, out_ids, out_d);
+                                           causal ? 1 : 0, remap, out_ids, out_d, only);
     return cudaGetLastError();
 }
 

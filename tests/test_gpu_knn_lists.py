@@ -34,3 +34,30 @@ def test_exact_keys_with_ties(n, m):
             assert np.array_equal(d.cpu().numpy()[:, :k], np.take_along_axis(D[:nq], order[:nq, :k], 1))
             assert (ids.cpu().numpy()[:, k:] == -1).all() and np.isinf(d.cpu().numpy()[:, k:]).all()
     ix.close()
+
+
+@pytest.mark.parametrize("m", [24, 130])
+@pytest.mark.parametrize("n", [4095, 4096, 20011])
+@pytest.mark.parametrize("clustered", [False, True])
+def test_large_k(n, m, clustered):
+    """K > 40: lists of 64 per segment merged, and the queries whose neighbours fill one
+    segment's list (rows in runs of 300 copies of a few points) done again."""
+    import torch
+
+    import paper_2206_11408_gb300 as fg
+
+    rng = np.random.default_rng(n + m)
+    X = rng.integers(0, 5, (n, m)).astype(np.float32)
+    if clustered:
+        X = X[np.arange(n) // 300 * 300] + rng.integers(0, 2, (n, m)) * (np.arange(m) < 3)
+        X = X.astype(np.float32)
+    Q = X[rng.integers(0, n, 130)] + rng.integers(0, 2, (130, m)).astype(np.float32)
+    D = (Q ** 2).sum(1).astype(np.int64)[:, None] + (X ** 2).sum(1).astype(np.int64)[None] - 2 * (Q @ X.T).astype(np.int64)
+    order = np.argsort(D * (1 << 20) + np.arange(n)[None], axis=1, kind="stable")
+    ix = fg.Index(X)
+    for nq, K in ((1, 41), (130, 100), (33, 256)):
+        ids, d = ix.knn(torch.from_numpy(Q[:nq]).cuda(), K)
+        ix.sync()
+        assert np.array_equal(ids.cpu().numpy(), order[:nq, :K])
+        assert np.array_equal(d.cpu().numpy(), np.take_along_axis(D[:nq], order[:nq, :K], 1))
+    ix.close()
