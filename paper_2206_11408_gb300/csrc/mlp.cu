@@ -9,14 +9,19 @@
 // weights, hidden-layer inputs rounded to BF16, FP32 accumulation), with the
 // roundings passed straight through in the backward pass.
 //
-// Kernels (one mini-batch of B rows per step):
-//   k_quant     BF16-rounded copies of the master weights
-//   k_fwd       thread per row: x~, h1~ = bf16(relu(W1 x~ + b1)), h2 = relu(W2 h1~ + b2),
-//               y = w3 . h2 + b3, residual y - t
-//   k_bwd       thread per row: dy = 2 (y - t) / B, dz2 = dy w3 [h2 > 0],
-//               dz1 = W2^T dz2 [h1 > 0]
-//   k_wgrad     thread per weight: sums of dz1 x~, dz2 h1~, dy h2 over the batch
-//   k_adam      Adam on the FP32 masters
+// Kernels, two per mini-batch of B rows:
+//   k_rows      a block per 32 rows, lane = row, warp = 8 of the 64 units of a layer:
+//               x~, h1~ = bf16(relu(W1 x~ + b1)), h2 = relu(W2 h1~ + b2),
+//               y = w3 . h2 + b3; training also dy = 2 (y - t) / B,
+//               dz2 = dy w3 [h2 > 0], dz1 = W2^T dz2 [h1 > 0] and the squared errors
+//   k_weights   thread per weight: sums of dz1 x~, dz2 h1~, dy h2 over the batch (a
+//               bias is the weight of a constant 1), then Adam on the FP32 master
+// Every sum runs in a fixed order (units, inputs and rows ascending).  Weights are
+// rounded to BF16 as they are read.  Between the two kernels a quantity is stored
+// unit-major (one row of B values per unit), so that both sides move 16 bytes per
+// lane.  A step of 4,096 rows with r = 24 took 500 us as six kernels (the weight
+// sums alone over 400: 48 blocks of strided loads); the sums' chain of B dependent
+// FMAs (8.5 us) bounds it now.
 #include <math.h>
 #include <string.h>
 
@@ -55,109 +60,214 @@ struct Off {
 
 __device__ __forceinline__ float bf(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
-__global__ void k_quant(const float* w, int64_t n, int64_t b1, int64_t W2, int64_t b2, int64_t w3,
-                        int64_t b3, float* q) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const bool is_bias = (i >= b1 && i < W2) || (i >= b2 && i < w3) || i == b3;
-    q[i] = is_bias ? w[i] : bf(w[i]);
-}
+constexpr int RB = 32;        // rows per block of k_rows
+constexpr int RT = 256;       // its threads: a warp per 8 units
+constexpr int WTJ = 8, WTK = 16, WTB = 128;   // weights per block of k_weights, rows per stage
+constexpr int WLD = WTB + 4;  // its row stride in shared memory (conflict-free 16-byte reads)
 
-// forward: rows idx[0..B) of X (N x nf); stores x~ (B x nf), h1~ (B x H), h2 (B x H), res (B)
-__global__ void k_fwd(const float* wq, int nf, const float* X, const float* T, const int64_t* idx,
-                      int B, float* xs, float* h1s, float* h2s, float* res, float* y_out) {
-    extern __shared__ float sw[];
+size_t rows_smem(int nf) { return sizeof(float) * ((size_t)nf * (HID + RB) + 2 * HID * HID + 3 * HID * RB + 2 * HID + 4 * HID); }
+
+// per-unit arrays of a batch: nf, 64, 64, 64, 64 and 1 rows of Bp values
+struct Batch {
+    float *x, *h1, *h2, *dz1, *dz2, *dy;
+    int64_t Bp;
+};
+
+// rows idx[0 .. B) (or 0 .. B - 1) of X (N x nf).  g.x == nullptr: forward only.
+__global__ void __launch_bounds__(RT) k_rows(const float* __restrict__ w, int nf,
+                                             const float* __restrict__ X, const float* __restrict__ T,
+                                             const int64_t* __restrict__ idx, int B, Batch g,
+                                             float* res, float* y_out, double* sq) {
+    extern __shared__ __align__(16) float sw[];
+    float* W1t = sw;                       // nf x 64: W1 transposed
+    float* W2t = W1t + nf * HID;           // 64 x 64: W2 transposed
+    float* W2s = W2t + HID * HID;          // 64 x 64: W2
+    float* xs = W2s + HID * HID;           // nf x 32
+    float* h1 = xs + nf * RB;              // 64 x 32
+    float* h2 = h1 + HID * RB;             // 64 x 32
+    float* dz = h2 + HID * RB;             // 64 x 32
+    float* w3 = dz + HID * RB;             // 64
+    float* dyv = w3 + HID;                 // 32
     const Off o(nf);
-    const int64_t nw = wcount(nf);
-    for (int64_t i = threadIdx.x; i < nw; i += blockDim.x) sw[i] = wq[i];
+    const int t = threadIdx.x, lane = t & 31, u0 = (t >> 5) * 8;
+    const bool train = g.x != nullptr;
+    for (int i = t; i < HID * nf; i += RT) W1t[(i % nf) * HID + i / nf] = bf(w[o.W1 + i]);
+    for (int i = t; i < HID * HID; i += RT) {
+        const float v = bf(w[o.W2 + i]);
+        W2s[i] = v;
+        W2t[(i % HID) * HID + i / HID] = v;
+    }
+    if (t < HID) w3[t] = bf(w[o.w3 + t]);
+    const int b = blockIdx.x * RB + lane;
+    for (int i = t; i < RB * nf; i += RT) {   // consecutive threads: consecutive features of a row
+        const int r = i / nf, f = i % nf, br = blockIdx.x * RB + r;
+        xs[f * RB + r] = br < B ? bf(X[(idx ? idx[br] : (int64_t)br) * nf + f]) : 0.f;
+    }
     __syncthreads();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const int64_t row = idx ? idx[b] : b;
-    float x[96];
-    for (int i = 0; i < nf; ++i) {
-        x[i] = bf(X[row * nf + i]);
-        if (xs) xs[(int64_t)b * nf + i] = x[i];
-    }
-    float z2[HID];
-    for (int k = 0; k < HID; ++k) z2[k] = sw[o.b2 + k];
-    for (int j = 0; j < HID; ++j) {
-        float z = sw[o.b1 + j];
-        for (int i = 0; i < nf; ++i) z = fmaf(sw[o.W1 + (int64_t)j * nf + i], x[i], z);
-        const float h = bf(fmaxf(z, 0.f));
-        if (h1s) h1s[(int64_t)b * HID + j] = h;
-        for (int k = 0; k < HID; ++k) z2[k] = fmaf(sw[o.W2 + k * HID + j], h, z2[k]);
-    }
-    float y = sw[o.b3];
-    for (int k = 0; k < HID; ++k) {
-        const float h2 = fmaxf(z2[k], 0.f);
-        if (h2s) h2s[(int64_t)b * HID + k] = h2;
-        y = fmaf(sw[o.w3 + k], h2, y);
-    }
-    if (res) res[b] = y - (T ? T[row] : 0.f);
-    if (y_out) y_out[b] = y;
-}
+    if (train && b < B)
+        for (int f = t >> 5; f < nf; f += RT / 32) g.x[f * g.Bp + b] = xs[f * RB + lane];
 
-__global__ void k_bwd(const float* wq, int nf, const float* h1s, const float* h2s, const float* res,
-                      int B, float* dys, float* dz1s, float* dz2s) {
-    extern __shared__ float sw[];
-    const Off o(nf);
-    for (int64_t i = threadIdx.x; i < HID * HID; i += blockDim.x) sw[i] = wq[o.W2 + i];
-    for (int i = threadIdx.x; i < HID; i += blockDim.x) sw[HID * HID + i] = wq[o.w3 + i];
+    // out[u0 .. u0 + 7][lane] = init + sum over i of M[i][u] v[i][lane], i ascending
+    auto layer = [&](const float* M, const float* v, int n, float (&z)[8]) {
+#pragma unroll 4
+        for (int i = 0; i < n; ++i) {
+            const float a = v[i * RB + lane];
+            const float4 m0 = *reinterpret_cast<const float4*>(M + i * HID + u0);
+            const float4 m1 = *reinterpret_cast<const float4*>(M + i * HID + u0 + 4);
+            z[0] = fmaf(m0.x, a, z[0]);
+            z[1] = fmaf(m0.y, a, z[1]);
+            z[2] = fmaf(m0.z, a, z[2]);
+            z[3] = fmaf(m0.w, a, z[3]);
+            z[4] = fmaf(m1.x, a, z[4]);
+            z[5] = fmaf(m1.y, a, z[5]);
+            z[6] = fmaf(m1.z, a, z[6]);
+            z[7] = fmaf(m1.w, a, z[7]);
+        }
+    };
+    float z[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) z[q] = w[o.b1 + u0 + q];
+    layer(W1t, xs, nf, z);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const float h = bf(fmaxf(z[q], 0.f));
+        h1[(u0 + q) * RB + lane] = h;
+        if (train && b < B) g.h1[(u0 + q) * g.Bp + b] = h;
+        z[q] = w[o.b2 + u0 + q];
+    }
     __syncthreads();
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const float dy = 2.f * res[b] / (float)B;
-    dys[b] = dy;
-    float dz2[HID];
-    for (int k = 0; k < HID; ++k) {
-        dz2[k] = h2s[(int64_t)b * HID + k] > 0.f ? dy * sw[HID * HID + k] : 0.f;
-        dz2s[(int64_t)b * HID + k] = dz2[k];
+    layer(W2t, h1, HID, z);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const float h = fmaxf(z[q], 0.f);
+        h2[(u0 + q) * RB + lane] = h;
+        if (train && b < B) g.h2[(u0 + q) * g.Bp + b] = h;
     }
-    for (int j = 0; j < HID; ++j) {
-        float s = 0.f;
-        for (int k = 0; k < HID; ++k) s = fmaf(sw[k * HID + j], dz2[k], s);
-        dz1s[(int64_t)b * HID + j] = h1s[(int64_t)b * HID + j] > 0.f ? s : 0.f;
+    __syncthreads();
+    if (t < 32) {
+        float y = w[o.b3];
+#pragma unroll 8
+        for (int k = 0; k < HID; ++k) y = fmaf(w3[k], h2[k * RB + lane], y);
+        float e = 0.f;
+        if (b < B) {
+            if (y_out) y_out[b] = y;
+            e = y - (T ? T[idx ? idx[b] : (int64_t)b] : 0.f);
+            if (res) res[b] = e;
+        }
+        if (train) {
+            const float dy = 2.f * e / (float)B;
+            dyv[lane] = dy;
+            if (b < B) g.dy[b] = dy;
+            double a = (double)e * e;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+            if (lane == 0) atomicAdd(sq, a);
+        }
     }
+    if (!train) return;
+    __syncthreads();
+    const float dy = dyv[lane];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int k = u0 + q;
+        const float d = h2[k * RB + lane] > 0.f ? dy * w3[k] : 0.f;
+        dz[k * RB + lane] = d;
+        if (b < B) g.dz2[k * g.Bp + b] = d;
+        z[q] = 0.f;
+    }
+    __syncthreads();
+    layer(W2s, dz, HID, z);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        if (b < B) g.dz1[(u0 + q) * g.Bp + b] = h1[(u0 + q) * RB + lane] > 0.f ? z[q] : 0.f;
 }
 
-// one thread per weight: gradient summed over the batch
-__global__ void k_wgrad(int nf, int B, const float* xs, const float* h1s, const float* h2s,
-                        const float* dys, const float* dz1s, const float* dz2s, float* g) {
-    const Off o(nf);
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= wcount(nf)) return;
-    float s = 0.f;
-    if (i < o.b1) {
-        const int j = (int)(i / nf), k = (int)(i % nf);
-        for (int b = 0; b < B; ++b) s = fmaf(dz1s[(int64_t)b * HID + j], xs[(int64_t)b * nf + k], s);
-    } else if (i < o.W2) {
-        const int j = (int)(i - o.b1);
-        for (int b = 0; b < B; ++b) s += dz1s[(int64_t)b * HID + j];
-    } else if (i < o.b2) {
-        const int k = (int)((i - o.W2) / HID), j = (int)((i - o.W2) % HID);
-        for (int b = 0; b < B; ++b) s = fmaf(dz2s[(int64_t)b * HID + k], h1s[(int64_t)b * HID + j], s);
-    } else if (i < o.w3) {
-        const int k = (int)(i - o.b2);
-        for (int b = 0; b < B; ++b) s += dz2s[(int64_t)b * HID + k];
-    } else if (i < o.b3) {
-        const int k = (int)(i - o.w3);
-        for (int b = 0; b < B; ++b) s = fmaf(dys[b], h2s[(int64_t)b * HID + k], s);
-    } else {
-        for (int b = 0; b < B; ++b) s += dys[b];
-    }
-    g[i] = s;
-}
-
-__global__ void k_adam(float* w, const float* g, float* m, float* v, int64_t n, float lr, float b1,
-                       float b2, float c1, float c2) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
+__device__ __forceinline__ void adam(float* w, float* m, float* v, int64_t i, float gi, float lr,
+                                     float b1, float b2, float c1, float c2) {
     m[i] = b1 * m[i] + (1.f - b1) * gi;
     v[i] = b2 * v[i] + (1.f - b2) * gi * gi;
     const float mh = m[i] / c1, vh = v[i] / c2;
     w[i] -= lr * mh / (sqrtf(vh) + 1e-8f);
+}
+
+// One weight per thread: its gradient summed over the batch's rows in order, written to
+// `grad` (when not null) and applied by Adam (when w is not null).  Blocks of 8 x 16
+// weights of the three outer products dz1 x [x~, 1], dz2 x [h1~, 1], dy x [h2, 1]; their 24
+// rows of values pass through shared memory 128 batch rows at a time.
+__global__ void __launch_bounds__(WTJ * WTK)
+    k_weights(int nf, int B, Batch g, float* grad, float* w, float* m, float* v, float lr, float b1,
+              float b2, float c1, float c2) {
+    __shared__ __align__(16) float s[2][WTJ + WTK][WLD];
+    const Off o(nf);
+    const int n1 = (nf + 1 + WTK - 1) / WTK, n2 = (HID + 1 + WTK - 1) / WTK;
+    int blk = blockIdx.x;
+    const float *A, *C;   // rows of the outer product's sides
+    int nj = HID, nk = HID;
+    int64_t wb, bb;
+    if (blk < n1 * (HID / WTJ)) {
+        A = g.dz1;
+        C = g.x;
+        nk = nf;
+        wb = o.W1;
+        bb = o.b1;
+    } else if ((blk -= n1 * (HID / WTJ)) < n2 * (HID / WTJ)) {
+        A = g.dz2;
+        C = g.h1;
+        wb = o.W2;
+        bb = o.b2;
+    } else {
+        blk -= n2 * (HID / WTJ);
+        A = g.dy;
+        C = g.h2;
+        nj = 1;
+        wb = o.w3;
+        bb = o.b3;
+    }
+    const int nt = nk == nf && A == g.dz1 ? n1 : n2;
+    const int j0 = blk / nt * WTJ, k0 = blk % nt * WTK;
+    const int t = threadIdx.x, jj = t / WTK, kk = t % WTK;
+    const int j = j0 + jj, k = k0 + kk;
+    // 16-byte asynchronous copies; rows that do not exist and values past B read as 0
+    auto stage = [&](int st, int lo) {
+        for (int i = t; i < (WTJ + WTK) * (WTB / 4); i += WTJ * WTK) {
+            const int r = i / (WTB / 4), c = i % (WTB / 4) * 4;
+            const bool side = r < WTJ;
+            const int row = side ? j0 + r : k0 + r - WTJ;
+            const bool ok = row < (side ? nj : nk) && lo + c < B;
+            const float* src = ok ? (side ? A : C) + (size_t)row * g.Bp + lo + c : A;
+            const int bytes = ok ? min(16, 4 * (B - lo - c)) : 0;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(&s[st][r][c])),
+                         "l"(src), "r"(bytes));
+        }
+        asm volatile("cp.async.commit_group;");
+    };
+    float acc = 0.f;
+    const bool bias = k == nk;
+    stage(0, 0);
+    for (int lo = 0, st = 0; lo < B; lo += WTB, st ^= 1) {
+        if (lo + WTB < B) stage(st ^ 1, lo + WTB);
+        else asm volatile("cp.async.commit_group;");
+        asm volatile("cp.async.wait_group 1;");
+        __syncthreads();
+        const float* a = s[st][jj];
+        const float* c = s[st][WTJ + kk];
+#pragma unroll 8
+        for (int i = 0; i < WTB; i += 4) {
+            const float4 x = *reinterpret_cast<const float4*>(a + i);
+            float4 y = *reinterpret_cast<const float4*>(c + i);
+            if (bias) y = make_float4(1.f, 1.f, 1.f, 1.f);
+            acc = fmaf(x.x, y.x, acc);
+            acc = fmaf(x.y, y.y, acc);
+            acc = fmaf(x.z, y.z, acc);
+            acc = fmaf(x.w, y.w, acc);
+        }
+        __syncthreads();
+    }
+    if (j >= nj || k > nk) return;
+    const int64_t i = bias ? bb + j : wb + (int64_t)j * nk + k;
+    if (grad) grad[i] = acc;
+    if (w) adam(w, m, v, i, acc, lr, b1, b2, c1, c2);
 }
 
 __global__ void k_abs_sum(const float* res, int n, double* out) {
@@ -165,20 +275,6 @@ __global__ void k_abs_sum(const float* res, int n, double* out) {
     double a = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         a += fabs((double)res[i]);
-    s[threadIdx.x] = a;
-    __syncthreads();
-    for (int k = 128; k > 0; k >>= 1) {
-        if ((int)threadIdx.x < k) s[threadIdx.x] += s[threadIdx.x + k];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(out, s[0]);
-}
-
-__global__ void k_sq_sum(const float* res, int n, double* out) {
-    __shared__ double s[256];
-    double a = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        a += (double)res[i] * res[i];
     s[threadIdx.x] = a;
     __syncthreads();
     for (int k = 128; k > 0; k >>= 1) {
@@ -202,16 +298,32 @@ struct Buf {
     }
 };
 
-cudaError_t fwd_bwd(const float* wq, int nf, const float* X, const float* T, const int64_t* idx,
-                    int B, float* xs, float* h1s, float* h2s, float* res, float* dys, float* dz1s,
-                    float* dz2s, float* g, cudaStream_t s) {
-    const size_t smw = sizeof(float) * wcount(nf);
-    cudaFuncSetAttribute(k_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw);
-    k_fwd<<<(B + 127) / 128, 128, smw, s>>>(wq, nf, X, T, idx, B, xs, h1s, h2s, res, nullptr);
-    const size_t smb = sizeof(float) * (HID * HID + HID);
-    k_bwd<<<(B + 127) / 128, 128, smb, s>>>(wq, nf, h1s, h2s, res, B, dys, dz1s, dz2s);
-    const int64_t nw = wcount(nf);
-    k_wgrad<<<(unsigned)((nw + 127) / 128), 128, 0, s>>>(nf, B, xs, h1s, h2s, dys, dz1s, dz2s, g);
+bool get_batch(Buf& buf, int nf, int64_t B, Batch* g) {
+    g->Bp = (B + 3) & ~int64_t(3);
+    g->x = buf.get<float>((size_t)g->Bp * nf);
+    g->h1 = buf.get<float>((size_t)g->Bp * HID);
+    g->h2 = buf.get<float>((size_t)g->Bp * HID);
+    g->dz1 = buf.get<float>((size_t)g->Bp * HID);
+    g->dz2 = buf.get<float>((size_t)g->Bp * HID);
+    g->dy = buf.get<float>((size_t)g->Bp);
+    return g->x && g->h1 && g->h2 && g->dz1 && g->dz2 && g->dy;
+}
+
+cudaError_t run_rows(const float* w, int nf, const float* X, const float* T, const int64_t* idx,
+                     int B, const Batch& g, float* res, float* y, double* sq, cudaStream_t s) {
+    const size_t smem = rows_smem(nf);
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_rows<<<(B + RB - 1) / RB, RT, smem, s>>>(w, nf, X, T, idx, B, g, res, y, sq);
+    return cudaGetLastError();
+}
+
+cudaError_t run_weights(int nf, int B, const Batch& g, float* grad, float* w, float* m, float* v,
+                        float lr, float b1, float b2, float c1, float c2, cudaStream_t s) {
+    const int n1 = (nf + 1 + WTK - 1) / WTK, n2 = (HID + 1 + WTK - 1) / WTK;
+    k_weights<<<(n1 + n2) * (HID / WTJ) + n2, WTJ * WTK, 0, s>>>(nf, B, g, grad, w, m, v, lr, b1, b2,
+                                                                c1, c2);
     return cudaGetLastError();
 }
 
@@ -377,28 +489,19 @@ finger_status finger_mlp_loss_grad(finger_index* ix, int nf, const float* weight
     const int64_t nw = wcount(nf);
     Buf buf;
     float* w = buf.get<float>(nw);
-    float* wq = buf.get<float>(nw);
     float* g = buf.get<float>(nw);
-    float* xs = buf.get<float>((size_t)B * nf);
-    float* h1s = buf.get<float>((size_t)B * HID);
-    float* h2s = buf.get<float>((size_t)B * HID);
-    float* res = buf.get<float>(B);
-    float* dys = buf.get<float>(B);
-    float* dz1s = buf.get<float>((size_t)B * HID);
-    float* dz2s = buf.get<float>((size_t)B * HID);
     double* acc = buf.get<double>(1);
+    Batch bt;
     finger_status st = FINGER_OK;
-    if (!w || !wq || !g || !xs || !h1s || !h2s || !res || !dys || !dz1s || !dz2s || !acc) {
+    if (!w || !g || !acc || !get_batch(buf, nf, B, &bt)) {
         st = FINGER_ERR_OOM;
     } else {
-        const Off o(nf);
         double h = 0;
         bool ok = cudaMemcpyAsync(w, weights, nw * 4, cudaMemcpyHostToDevice, s) == cudaSuccess;
-        k_quant<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(w, nw, o.b1, o.W2, o.b2, o.w3, o.b3, wq);
-        ok = ok && fwd_bwd(wq, nf, feat, target, nullptr, B, xs, h1s, h2s, res, dys, dz1s, dz2s, g,
-                           s) == cudaSuccess;
         ok = ok && cudaMemsetAsync(acc, 0, 8, s) == cudaSuccess;
-        k_sq_sum<<<64, 256, 0, s>>>(res, B, acc);
+        ok = ok && run_rows(w, nf, feat, target, nullptr, B, bt, nullptr, nullptr, acc, s) == cudaSuccess;
+        ok = ok && run_weights(nf, B, bt, g, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, 1.f, 1.f, s) ==
+                       cudaSuccess;
         ok = ok && cudaMemcpyAsync(grad, g, nw * 4, cudaMemcpyDeviceToHost, s) == cudaSuccess;
         ok = ok && cudaMemcpyAsync(&h, acc, 8, cudaMemcpyDeviceToHost, s) == cudaSuccess;
         ok = ok && cudaStreamSynchronize(s) == cudaSuccess;
@@ -423,20 +526,15 @@ finger_status finger_mlp_predict(finger_index* ix, const float* feat, int64_t n,
     cudaStream_t s = (cudaStream_t)stream;
     Buf buf;
     float* w = buf.get<float>(nw);
-    float* wq = buf.get<float>(nw);
     finger_status st = FINGER_OK;
-    if (!w || !wq) {
+    if (!w) {
         st = FINGER_ERR_OOM;
     } else {
-        const Off o(nf);
         bool ok = cudaMemcpyAsync(w, ix->h_mlp.data(), nw * 4, cudaMemcpyHostToDevice, s) == cudaSuccess;
-        k_quant<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(w, nw, o.b1, o.W2, o.b2, o.w3, o.b3, wq);
-        const size_t smw = sizeof(float) * nw;
-        cudaFuncSetAttribute(k_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw);
         for (int64_t lo = 0; lo < n && ok; lo += 1 << 20) {
             const int B = (int)std::min<int64_t>(n - lo, 1 << 20);
-            k_fwd<<<(B + 127) / 128, 128, smw, s>>>(wq, nf, feat + lo * nf, nullptr, nullptr, B,
-                                                    nullptr, nullptr, nullptr, nullptr, out + lo);
+            ok = run_rows(w, nf, feat + lo * nf, nullptr, nullptr, B, Batch{}, nullptr, out + lo, nullptr,
+                          s) == cudaSuccess;
         }
         ok = ok && cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess;
         if (!ok) st = FINGER_ERR_CUDA;
@@ -462,21 +560,13 @@ finger_status finger_train_predictor(finger_index* ix, const finger_train_params
     const int B = p->batch;
     Buf buf;
     float* w = buf.get<float>(nw);
-    float* wq = buf.get<float>(nw);
-    float* g = buf.get<float>(nw);
     float* m1 = buf.get<float>(nw);
     float* m2 = buf.get<float>(nw);
-    float* xs = buf.get<float>((size_t)B * nf);
-    float* h1s = buf.get<float>((size_t)B * HID);
-    float* h2s = buf.get<float>((size_t)B * HID);
     float* res = buf.get<float>(B);
-    float* dys = buf.get<float>(B);
-    float* dz1s = buf.get<float>((size_t)B * HID);
-    float* dz2s = buf.get<float>((size_t)B * HID);
     int64_t* idx = buf.get<int64_t>((size_t)p->n_train);
     double* acc = buf.get<double>(1);
-    if (!w || !wq || !g || !m1 || !m2 || !xs || !h1s || !h2s || !res || !dys || !dz1s || !dz2s ||
-        !idx || !acc) {
+    Batch bt;
+    if (!w || !m1 || !m2 || !res || !idx || !acc || !get_batch(buf, nf, B, &bt)) {
         cudaSetDevice(prev);
         return FINGER_ERR_OOM;
     }
@@ -495,21 +585,21 @@ finger_status finger_train_predictor(finger_index* ix, const finger_train_params
     std::iota(perm.begin(), perm.end(), 0);
     int64_t step = 0;
     const float b1 = 0.9f, b2 = 0.999f;
+    std::shuffle(perm.begin(), perm.end(), rng);
     for (int ep = 0; ep < p->epochs && ok; ++ep) {
-        std::shuffle(perm.begin(), perm.end(), rng);
         ok = cudaMemcpyAsync(idx, perm.data(), perm.size() * 8, cudaMemcpyHostToDevice, s) == cudaSuccess &&
              cudaStreamSynchronize(s) == cudaSuccess;
         double sq = 0;
         ok = ok && cudaMemsetAsync(acc, 0, 8, s) == cudaSuccess;
         for (int64_t lo = 0; lo + B <= p->n_train && ok; lo += B) {
             step++;
-            k_quant<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(w, nw, o.b1, o.W2, o.b2, o.w3, o.b3, wq);
-            ok = fwd_bwd(wq, nf, p->feat, p->target, idx + lo, B, xs, h1s, h2s, res, dys, dz1s,
-                         dz2s, g, s) == cudaSuccess;
-            k_sq_sum<<<16, 256, 0, s>>>(res, B, acc);
             const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-            k_adam<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(w, g, m1, m2, nw, p->lr, b1, b2, c1, c2);
+            ok = run_rows(w, nf, p->feat, p->target, idx + lo, B, bt, nullptr, nullptr, acc, s) ==
+                     cudaSuccess &&
+                 run_weights(nf, B, bt, nullptr, w, m1, m2, p->lr, b1, b2, c1, c2, s) == cudaSuccess;
         }
+        // the next epoch's order while this one runs
+        if (ep + 1 < p->epochs) std::shuffle(perm.begin(), perm.end(), rng);
         ok = ok && cudaMemcpyAsync(&sq, acc, 8, cudaMemcpyDeviceToHost, s) == cudaSuccess &&
              cudaStreamSynchronize(s) == cudaSuccess;
         if (losses) losses[ep] = (float)(sq / std::max<int64_t>(1, (p->n_train / B) * B));
@@ -517,16 +607,12 @@ finger_status finger_train_predictor(finger_index* ix, const finger_train_params
     // eps' = mean |prediction - target| on the held-out rows (inference semantics)
     float eps = 0.f;
     if (ok) {
-        k_quant<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(w, nw, o.b1, o.W2, o.b2, o.w3, o.b3, wq);
         ok = cudaMemsetAsync(acc, 0, 8, s) == cudaSuccess;
         const int64_t v0 = p->n_train, nv = p->n_val;
-        const size_t smw = sizeof(float) * nw;
-        cudaFuncSetAttribute(k_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw);
         for (int64_t lo = 0; lo < nv && ok; lo += B) {
             const int nb = (int)std::min<int64_t>(B, nv - lo);
-            k_fwd<<<(nb + 127) / 128, 128, smw, s>>>(wq, nf, p->feat + (v0 + lo) * nf,
-                                                     p->target + v0 + lo, nullptr, nb, nullptr,
-                                                     nullptr, nullptr, res, nullptr);
+            ok = run_rows(w, nf, p->feat + (v0 + lo) * nf, p->target + v0 + lo, nullptr, nb, Batch{}, res,
+                          nullptr, nullptr, s) == cudaSuccess;
             k_abs_sum<<<16, 256, 0, s>>>(res, nb, acc);
         }
         double sa = 0;
