@@ -12,16 +12,19 @@
 // approximation error of the K-th distance.
 //
 // k_knn_tc is persistent (one CTA per SM) and warp-specialised:
-//   warp 0     TMA producer: the query tile (hi, lo), resident in shared memory
-//              for the whole job where m <= 128, and 64-column (128-byte,
-//              SWIZZLE_128B) chunks of the base tiles (hi, lo) into a ring;
-//              longer rows stream the query's chunks through the ring as well
+//   warp 0     TMA producer: 64-column (128-byte, SWIZZLE_128B) chunks of the base
+//              tiles (hi, lo) into a ring; rows above 128 dimensions stream the
+//              query tile's chunks through it as well
 //   warp 1     MMA issuer (one elected lane): 3 products x 4 K-steps per chunk
-//              into one of two 128x128 FP32 accumulators in tensor memory
+//              into one of two 128x128 FP32 accumulators in tensor memory.  Up to
+//              128 dimensions the query tile is the A operand from tensor memory: with
+//              both operands in shared memory a 128 x 128 x 16 product reads all the
+//              128 bytes per cycle it gives, and the epilogue's own accesses starve
 //   warps 2-5  epilogue: tcgen05.ld of the accumulator (thread = query row),
 //              distances and their minimum against the row's K'-th distance;
 //              where some row of the warp has a smaller one, every thread
-//              appends its own to its row's pending buffer
+//              appends its own to its row's pending buffer; they also load the
+//              query tiles
 // A row's K' candidates are (distance, id) pairs in shared memory, in eight
 // groups whose largest keys its thread holds in registers; once some row of a
 // warp has more than 16 pending, all 32 rows insert theirs side by side, a thread
@@ -50,7 +53,7 @@ constexpr int TQ = 128;                      // query rows per tile (MMA M)
 constexpr int TB = 128;                      // base rows per tile (MMA N)
 constexpr int KCH = 64;                      // K elements per chunk (128 bytes of BF16)
 constexpr int PART = TQ * 128;               // one 128-row x 128-byte operand part: 16 KB
-constexpr int MAX_STAGES = 4;
+constexpr int MAX_STAGES = 5;
 constexpr int PEND = 32;                     // pending candidates per row
 constexpr int QRES_CHUNKS = 2;               // query tiles up to this many chunks stay resident
 constexpr int TC_THREADS = 192;
@@ -79,6 +82,8 @@ struct TcArgs {
     int nqt;              // query tiles
     int causal;           // 1: queries are the base rows, row i sees base rows < i
     int stages;
+    const __nv_bfloat16 *qh, *ql;   // the queries' BF16 parts, row stride ms
+    int ms;
     const float* qn;      // ||q||^2 (FP32), nq
     const float* xn;      // ||x||^2 (FP32), n
     u64* keys;            // nq x nseg x KP candidate keys
@@ -117,6 +122,14 @@ __device__ __forceinline__ uint32_t s32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// true in one lane of the (converged) warp, always the same one
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
 // bounded parity wait; false (and the abort flag raised) on timeout
 __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                          int* err) {
@@ -151,6 +164,15 @@ __device__ __forceinline__ void mma_bf16_tc(uint32_t tmem, uint64_t ad, uint64_t
         "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate));
 }
 
+// the same with A (128 rows, one per lane, two BF16 of K per column) in tensor memory
+__device__ __forceinline__ void mma_bf16_ts(uint32_t tmem, uint32_t at, uint64_t bd, uint32_t idesc,
+                                            uint32_t accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem),
+        "r"(at), "l"(bd), "r"(idesc), "r"(accumulate));
+}
+
 __device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
                                        uint32_t bar) {
     asm volatile(
@@ -180,6 +202,19 @@ __device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32]) {
                    "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]),
                    "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]),
                    "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]));
+}
+
+// 32 columns of this thread's tensor-memory lane from registers (wait::st ends it)
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+        "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]),
+        "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]),
+        "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]),
+        "r"(r[29]), "r"(r[30]), "r"(r[31])
+        : "memory");
 }
 
 // (qn + xa) - 2 ra, (qn + xb) - 2 rb, each rounded as its scalar form is
@@ -260,133 +295,141 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
              const __grid_constant__ CUtensorMap txh, const __grid_constant__ CUtensorMap txl,
              TcArgs a) {
     static_assert(KP == 32 || KP == 64, "candidate lists of 32 or 64");
-    constexpr int STAGE_BYTES = QRES ? 2 * PART : 4 * PART;        // [qh, ql,] xh, xl
+    // tensor memory: two 128-column accumulators, then two query tiles of 2 x 64 columns
+    constexpr int TMEM_COLS = QRES ? 512 : 256, QCOL = 2 * TB, QBUF = 128;
+    constexpr int XOFF = QRES ? 0 : 2 * PART;                      // a stage: [qh, ql,] xh, xl
+    constexpr int STAGE_BYTES = XOFF + 2 * PART;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* qres = sm;                                      // nchunk x (qh, ql)
-    unsigned char* stages = sm + (QRES ? a.nchunk * 2 * PART : 0);
+    unsigned char* stages = sm;
     uint32_t* lists = reinterpret_cast<uint32_t*>(stages + (size_t)a.stages * STAGE_BYTES);
     // lists: KP x 128 distances, then ids; PEND x 128 pending (distance, id)
     uint2* pend = reinterpret_cast<uint2*>(lists + 2 * KP * TQ);
     float* xns = reinterpret_cast<float*>(pend + PEND * TQ);                        // 4 x 64 norms
     uint64_t* bars = reinterpret_cast<uint64_t*>(xns + 4 * 64);
-    // full[4] empty[4] accf[2] acce[2] qfull qempty
+    // full[], empty[], accf[2], acce[2], qfull[2]
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_STAGES + 6);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const uint32_t ring = s32(stages);
     const uint32_t full0 = s32(bars), empty0 = s32(bars + MAX_STAGES),
-                   accf0 = s32(bars + 2 * MAX_STAGES), acce0 = accf0 + 16, qfull = accf0 + 32,
-                   qempty = accf0 + 40;
+                   accf0 = s32(bars + 2 * MAX_STAGES), acce0 = accf0 + 16, qfull0 = accf0 + 32;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2 * MAX_STAGES + 6; ++i) {
-            const int count = i == 2 * MAX_STAGES + 2 || i == 2 * MAX_STAGES + 3 ? 128 : 1;   // acce
+            const int count = i >= 2 * MAX_STAGES + 2 ? 128 : 1;   // acce, qfull: the epilogue
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full0 + 8 * i), "r"(count));
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(
-            s32(tmem_slot)));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         s32(tmem_slot)),
+                     "n"(TMEM_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     Jobs jobs(a);
     int qt, b0, b1, step, seg;
 
+    // The producer and the MMA warp run their loops whole, with one elected lane for
+    // the asynchronous instructions only: descriptors, barriers and coordinates then
+    // stay in uniform registers, where those instructions take them.  (On one
+    // lane alone the issue of a tile's products took 1,800 cycles for 1,400 of work.)
+    const bool leader = elect_one();
+    auto wait_all = [&](uint32_t bar, uint32_t parity) {
+        return __all_sync(0xffffffffu, wait_bar(bar, parity, abort_flag, a.err)) != 0;
+    };
     if (warp == 0) {
-        if (lane == 0) {
-            uint32_t s = 0, ph = 1u, job = 0;   // ring slot and its parity for `empty`
-            while (!*abort_flag && jobs.next(qt, b0, b1, step, seg)) {
-                if (b0 >= b1) continue;
-                if (QRES) {
-                    if (!wait_bar(qempty, (job & 1u) ^ 1u, abort_flag, a.err)) break;
-                    ++job;
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(qfull),
-                                 "r"(a.nchunk * 2 * PART)
-                                 : "memory");
-                    for (int c = 0; c < a.nchunk; ++c) {
-                        const uint32_t dst = s32(qres + (size_t)c * 2 * PART);
-                        tma_2d(dst, &tqh, c * KCH, qt * TQ, qfull);
-                        tma_2d(dst + PART, &tql, c * KCH, qt * TQ, qfull);
-                    }
-                }
-                for (int bt = b0; bt < b1 && !*abort_flag; bt += step)
-                    for (int c = 0; c < a.nchunk; ++c) {
-                        if (!wait_bar(empty0 + 8 * s, ph, abort_flag, a.err)) break;
-                        const uint32_t fb = full0 + 8 * s;
+        uint32_t s = 0, ph = 1u;   // ring slot and its parity for `empty`
+        bool ok = true;
+        while (ok && jobs.next(qt, b0, b1, step, seg))
+            for (int bt = b0; ok && bt < b1; bt += step)
+                for (int c = 0; c < a.nchunk; ++c) {
+                    ok = wait_all(empty0 + 8 * s, ph);
+                    if (!ok) break;
+                    const uint32_t fb = full0 + 8 * s;
+                    const uint32_t dst = ring + s * STAGE_BYTES;
+                    if (leader) {
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
                                      "r"(STAGE_BYTES)
                                      : "memory");
-                        uint32_t dst = s32(stages + (size_t)s * STAGE_BYTES);
                         if (!QRES) {
                             tma_2d(dst, &tqh, c * KCH, qt * TQ, fb);
                             tma_2d(dst + PART, &tql, c * KCH, qt * TQ, fb);
-                            dst += 2 * PART;
                         }
-                        tma_2d(dst, &txh, c * KCH, bt * TB, fb);
-                        tma_2d(dst + PART, &txl, c * KCH, bt * TB, fb);
-                        if (++s == (uint32_t)a.stages) {
-                            s = 0;
-                            ph ^= 1u;
-                        }
+                        tma_2d(dst + XOFF, &txh, c * KCH, bt * TB, fb);
+                        tma_2d(dst + XOFF + PART, &txl, c * KCH, bt * TB, fb);
                     }
-            }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            // D F32, A BF16, B BF16, K-major A and B, N = 128, M = 128
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TB >> 3) << 17) |
-                                   ((uint32_t)(TQ >> 4) << 24);
-            uint32_t s = 0, ph = 0u, job = 0, tile = 0;
-            while (!*abort_flag && jobs.next(qt, b0, b1, step, seg)) {
-                if (b0 >= b1) continue;
-                if (QRES) {
-                    if (!wait_bar(qfull, job & 1u, abort_flag, a.err)) break;
-                    ++job;
+                    __syncwarp();
+                    if (++s == (uint32_t)a.stages) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
-                for (int bt = b0; bt < b1 && !*abort_flag; bt += step, ++tile) {
-                    const uint32_t b = tile & 1u, tph = (tile >> 1) & 1u;
-                    if (!wait_bar(acce0 + 8 * b, tph ^ 1u, abort_flag, a.err)) break;
+    } else if (warp == 1) {
+        // D F32, A BF16, B BF16, K-major A and B, N = 128, M = 128
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TB >> 3) << 17) |
+                               ((uint32_t)(TQ >> 4) << 24);
+        uint32_t s = 0, ph = 0u, job = 0, tile = 0;
+        bool ok = true;
+        while (ok && jobs.next(qt, b0, b1, step, seg)) {
+            if (b0 >= b1) continue;
+            uint32_t qt0 = 0;
+            if (QRES) {
+                ok = wait_all(qfull0 + 8 * (job & 1u), (job >> 1) & 1u);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                qt0 = tmem + QCOL + (job & 1u) * QBUF;
+                ++job;
+            }
+            for (int bt = b0; ok && bt < b1; bt += step, ++tile) {
+                const uint32_t b = tile & 1u, tph = (tile >> 1) & 1u;
+                ok = wait_all(acce0 + 8 * b, tph ^ 1u);
+                if (!ok) break;
+                const uint32_t d = tmem + b * TB;
+                for (int c = 0; c < a.nchunk; ++c) {
+                    ok = wait_all(full0 + 8 * s, ph);
+                    if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t d = tmem + b * TB;
-                    for (int c = 0; c < a.nchunk; ++c) {
-                        if (!wait_bar(full0 + 8 * s, ph, abort_flag, a.err)) break;
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t st = s32(stages + (size_t)s * STAGE_BYTES);
-                        const uint32_t qb = QRES ? s32(qres + (size_t)c * 2 * PART) : st;
-                        const uint32_t xb = QRES ? st : st + 2 * PART;
+                    const uint32_t st = ring + s * STAGE_BYTES;
+                    const uint64_t xd = sdesc(st + XOFF), qd = sdesc(st);   // + 2 per 32 bytes
+                    if (leader) {
 #pragma unroll
                         for (int k = 0; k < KCH / 16; ++k) {
-                            const uint64_t qh = sdesc(qb + 32 * k), ql = sdesc(qb + PART + 32 * k);
-                            const uint64_t xh = sdesc(xb + 32 * k), xl = sdesc(xb + PART + 32 * k);
-                            mma_bf16_tc(d, qh, xh, idesc, (c | k) != 0);
-                            mma_bf16_tc(d, qh, xl, idesc, 1u);
-                            mma_bf16_tc(d, ql, xh, idesc, 1u);
+                            const uint64_t xh = xd + 2 * k, xl = xd + (PART >> 4) + 2 * k;
+                            if constexpr (QRES) {   // 8 columns per K step; low parts from column 64
+                                const uint32_t qh = qt0 + (KCH / 2) * c + 8 * k, ql = qh + 64;
+                                mma_bf16_ts(d, qh, xh, idesc, (c | k) != 0);
+                                mma_bf16_ts(d, qh, xl, idesc, 1u);
+                                mma_bf16_ts(d, ql, xh, idesc, 1u);
+                            } else {
+                                const uint64_t qh = qd + 2 * k, ql = qd + (PART >> 4) + 2 * k;
+                                mma_bf16_tc(d, qh, xh, idesc, (c | k) != 0);
+                                mma_bf16_tc(d, qh, xl, idesc, 1u);
+                                mma_bf16_tc(d, ql, xh, idesc, 1u);
+                            }
                         }
                         asm volatile(
                             "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                                 empty0 + 8 * s)
                             : "memory");
-                        if (++s == (uint32_t)a.stages) {
-                            s = 0;
-                            ph ^= 1u;
-                        }
+                        if (c + 1 == a.nchunk)
+                            asm volatile(
+                                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                    accf0 + 8 * b)
+                                : "memory");
                     }
-                    asm volatile(
-                        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                            accf0 + 8 * b)
-                        : "memory");
+                    __syncwarp();
+                    if (++s == (uint32_t)a.stages) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
                 }
-                if (QRES)   // the job's products have read the query tile
-                    asm volatile(
-                        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                            qempty)
-                        : "memory");
             }
         }
     } else {
@@ -401,7 +444,46 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         float* xs = xns + 64 * quarter;
         uint32_t tile = 0;
         bool stop = false;   // a wait timed out (the same in all lanes: they vote below)
+        // Query tile of the next job that has tiles into tensor memory: this thread's row
+        // (zeros beyond the rows and columns there are).  Two buffers: a job's tile
+        // goes in while the job before it runs, when the one before that is done (its
+        // last accumulator has been waited for).
+        Jobs ahead(a);
+        uint32_t loaded = 0;
+        auto load_queries = [&]() {
+            int nqt_, f0, f1, fs, fseg;
+            do {
+                if (!ahead.next(nqt_, f0, f1, fs, fseg)) return;
+            } while (f0 >= f1);
+            const int64_t qr = (int64_t)nqt_ * TQ + row;
+            const uint32_t at = tmem + ((uint32_t)(32 * quarter) << 16) + QCOL + (loaded & 1u) * QBUF;
+#pragma unroll 1
+            for (int part = 0; part < 2; ++part)
+#pragma unroll 1
+                for (int c = 0; c < a.nchunk; ++c) {
+                    const uint4* src =
+                        reinterpret_cast<const uint4*>((part ? a.ql : a.qh) + qr * a.ms) + 8 * c;
+                    uint32_t r[32];
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) {
+                        const uint4 v = qr < a.nq && c * KCH + 8 * p < a.ms ? __ldg(src + p)
+                                                                           : make_uint4(0u, 0u, 0u, 0u);
+                        r[4 * p] = v.x;
+                        r[4 * p + 1] = v.y;
+                        r[4 * p + 2] = v.z;
+                        r[4 * p + 3] = v.w;
+                    }
+                    tmem_st32(at + 64 * part + (KCH / 2) * c, r);
+                }
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(qfull0 + 8 * (loaded & 1u))
+                         : "memory");
+            ++loaded;
+        };
+        if (QRES) load_queries();
         while (!stop && jobs.next(qt, b0, b1, step, seg)) {
+            if (QRES && b0 < b1) load_queries();   // the next job's
             const int64_t q0 = (int64_t)qt * TQ;
             const int64_t qi = q0 + row;
             const int64_t id_end = a.causal ? min(qi, a.n) : a.n;   // ids below this count
@@ -444,6 +526,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 xnow = x1;
                 x1 = x2;
                 x2 = norms(bt + 2 * step);
+                // norms of 32 columns, read ahead of the accumulator's load: behind it in
+                // the same queue they took 250 cycles a step
+                float4 x[8];
+                auto put = [&](int half) {   // half a tile's norms into shared memory
+                    __syncwarp();
+                    if (lane >> 4 == half) reinterpret_cast<float4*>(xs)[lane & 15] = xnow;
+                    __syncwarp();
+                };
+                auto get = [&](int c) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) x[j] = reinterpret_cast<const float4*>(xs + (c & 32))[j];
+                };
+                put(0);
+                get(0);
                 stop = !__all_sync(0xffffffffu, wait_bar(accf0 + 8 * b, tph, abort_flag, a.err));
                 if (stop) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -457,15 +553,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 #pragma unroll 1
                 for (int c = 0; c < TB; c += 32) {
                     const int64_t id0 = (int64_t)bt * TB + c;
-                    if (!(c & 63)) {   // half a tile's norms
-                        __syncwarp();
-                        if (lane >> 4 == c >> 6) reinterpret_cast<float4*>(xs)[lane & 15] = xnow;
-                        __syncwarp();
-                    }
-                    float4 x[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        x[j] = reinterpret_cast<const float4*>(xs + (c & 32))[j];
                     tmem_wait32(r);
                     float v[32];
 #pragma unroll
@@ -477,7 +564,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 #pragma unroll
                         for (int j = 0; j < 32; ++j) v[j] = id0 + j < id_end ? v[j] : INFINITY;
                     }
-                    if (c + 32 < TB) tmem_ld32(tbase + c + 32, r);   // behind the checks
+                    if (c + 32 < TB) {   // the next columns, behind the checks
+                        if (c == 32) put(1);
+                        get(c + 32);
+                        tmem_ld32(tbase + c + 32, r);
+                    }
                     float mn[2];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -522,7 +613,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TMEM_COLS));
 }
 
 // FP32 rows -> BF16 high and low parts (row stride ms, zero padded) and the
@@ -829,12 +920,11 @@ bool make_map(CUtensorMap* map, const void* base, int64_t rows, int m, int ms) {
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// ring stages that the shared memory beside the heaps, pending buffers and a
-// resident query tile holds (at least two: 224 KB at KP = 64)
+// ring stages that the shared memory beside the lists and pending buffers holds
 template <int KP, bool QRES>
 cudaError_t run_tc(const CUtensorMap* maps, TcArgs a, int grid, cudaStream_t s) {
     const size_t fixed = 1024 + (size_t)(KP + PEND) * TQ * 8 + 4 * 64 * 4 + 8 * (2 * MAX_STAGES + 6) +
-                         16 + (QRES ? (size_t)a.nchunk * 2 * PART : 0);
+                         16;
     const size_t stage = (QRES ? 2 : 4) * PART;
     a.stages = (int)std::min<size_t>(MAX_STAGES, (227 * 1024 - fixed) / stage);
     const size_t smem = fixed + a.stages * stage;
@@ -900,6 +990,9 @@ cudaError_t run_items(finger_index* ix, const TcBase& x, const __nv_bfloat16* qh
     a.interleaved = order != CONTIGUOUS;
     a.nqt = (int)((nq + TQ - 1) / TQ);
     a.causal = order == CAUSAL ? 1 : 0;
+    a.qh = qh;
+    a.ql = ql;
+    a.ms = ms;
     a.qn = qn;
     a.xn = x.xn;
     a.keys = keys;
