@@ -205,7 +205,7 @@ finger_status finger_search_batch(finger_index* ix, const float* queries, int64_
 // Candidates: warps per block {2, 4, 8} x visited-hash slots {H/2, H, 2H}
 // around the default H x the kernel's register variants (the one with the
 // most resident warps that shared memory admits, and each one the mode has
-// with fewer: 64 / 80 / 96 registers, compiled for 32 / 24 / 20 resident
+// with fewer: 64 / 72 / 80 / 96 registers, compiled for 32 / 28 / 24 / 20 resident
 // warps) x the exact-row shape (the default groups of lanes per row, and rows
 // on all 32 lanes: fewer rows in flight per warp, the staging depth).
 // Returns the best time in *best_ms (may be NULL); finger_get_tuned reads
@@ -237,10 +237,10 @@ finger_status finger_autotune(finger_index* ix, const float* queries, int64_t nq
     SearchPlan bestp = def;
     const int Hs[3] = {std::max(256, def.H / 2), def.H, std::min(16384, def.H * 2)};
     const int Ws[3] = {2, 4, 8};
-    const int Os[4] = {0, 8, 6, 5};   // 0: the largest variant that fits
+    const int Os[5] = {0, 8, 7, 6, 5};   // 0: the largest variant that fits
     for (int wi = 0; wi < 3; ++wi)
         for (int hi = 0; hi < 3; ++hi)
-            for (int oi = 0; oi < 4; ++oi)
+            for (int oi = 0; oi < 5; ++oi)
                 for (int sh = 0; sh < 2; ++sh) {
             SearchPlan p;
             if (fg_make_plan(ix, ix->mode, ef, nq, &p, Ws[wi], Hs[hi], Os[oi], sh) != FINGER_OK) {

@@ -276,7 +276,7 @@ finger_status make_plan(finger_index* ix, int mode, int ef_max, int64_t nq, Sear
         p->occ = occ_force;
         bps = b;
     } else {
-        for (int occ : {8, 6}) {
+        for (int occ : {8, 7, 6}) {
             SearchPlan t = *p;
             t.occ = occ;
             int b = 0;

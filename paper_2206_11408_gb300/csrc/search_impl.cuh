@@ -1547,21 +1547,33 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
 // Instantiate and dispatch one mode over the (G, VPL, NPL) variants and the
 // resident-block target OCC: COOP_OCC (search_coop_*.cu) one query per block;
 // else blocks of 4 warps per SM, which sets the registers: 5 blocks (96)
-// everywhere, 6 (80) in all but the predictor and harvest modes, 8 (64) for
-// plain search and FP8 codes.  A pass of exact rows needs 16 VPL registers for
-// its loads in flight and a code block 32, so
+// everywhere, 6 (80) in all but the predictor and harvest modes, 7 (72) and 8
+// (64) where they do not cost more in spills than the residency brings.  A pass of
+// exact rows needs 16 VPL registers for its loads in flight and a code block 32
+// (FP16, 4 k steps) or 16, so
 //   * 64 registers serve one chunk per lane only (rows of at most 64 floats:
 //     10,000 x 64 plain 519 us against 540 at 80); with two, 1M x 128 plain
 //     took 2.87 ms against 2.65 at 80 registers and 2.75 at 96;
-//   * code modes with more than 32 links (two slots per lane) spill at 80:
-//     m = 100, 48 links, FP16 codes 3.24 ms against 3.08 at 96, LP 3.68 against
-//     3.59; with 32 links 80 registers win (1M x 128 FP16 codes 2.97 against
-//     3.29, plain as above).
+//   * 72 registers serve plain search with two or four chunks per lane (1M x 128
+//     2.49 ms against 2.64 at 80), LP and FP8 codes (m = 100, 48 links, LP, 4,099
+//     queries 1.75 against 2.06, 10,000 queries 3.27 against 3.51; m = 128 FP8 2.46
+//     against 2.55) and FP16 codes of 2 k steps with up to 32 links (m = 96 1.13
+//     against 1.20); not FP16 codes of 4 k steps (1M x 128 3.21 against 2.96), of 2
+//     with 48 links (3.28 against 3.07), FP32 tables (3.48 against 3.14) or m = 960;
+//   * code modes with more than 32 links (two slots per lane) spill at 80: m =
+//     100, 48 links, FP16 codes 3.24 ms against 3.08 at 96; with 32 links 80
+//     registers win (1M x 128 FP16 codes 2.97 against 3.29).
 template <int MODE, int OCC>
 constexpr bool has_variant(int VPL, int NPL) {
-    const bool codes = MODE == MODE_F16_K2 || MODE == MODE_F16_K4 || MODE == MODE_LP_K2 ||
-                       MODE == MODE_LP_K4 || MODE == MODE_F8_K2 || MODE == MODE_F8_K4;
-    return OCC == 8 ? VPL == 1 && !(codes && NPL > 1) : OCC == 6 ? !(codes && NPL > 1) : true;
+    const bool fp8 = MODE == MODE_LP_K2 || MODE == MODE_LP_K4 || MODE == MODE_F8_K2 ||
+                     MODE == MODE_F8_K4;
+    const bool codes = fp8 || MODE == MODE_F16_K2 || MODE == MODE_F16_K4;
+    if (OCC == 8) return VPL == 1 && !(codes && NPL > 1);
+    if (OCC == 7)
+        return VPL < LONG_VPL && (MODE == FINGER_MODE_PLAIN ? VPL > 1
+                                  : MODE == MODE_F16_K2     ? NPL == 1
+                                                            : fp8);
+    return OCC != 6 || !(codes && NPL > 1);
 }
 
 #define LP_MODE(m) ((m) == MODE_LP_K2 || (m) == MODE_LP_K4 || (m) == MODE_F8_K2 || (m) == MODE_F8_K4)
@@ -1618,6 +1630,8 @@ cudaError_t launch_mode(const DevIndex& ix, const SearchArgs& a, const SearchPla
                         cudaStream_t s) {
     if constexpr (MODE == FINGER_MODE_PLAIN || F8_MODE(MODE))
         if (p.occ == 8) return launch_occ<MODE, 8>(ix, a, p, s);
+    if constexpr (MODE == FINGER_MODE_PLAIN || LP_MODE(MODE) || MODE == MODE_F16_K2)
+        if (p.occ == 7) return launch_occ<MODE, 7>(ix, a, p, s);
     if constexpr (MODE == FINGER_MODE_PLAIN || MODE == FINGER_MODE_FINGER ||
                   LP_MODE(MODE) || MODE == MODE_F16_K2 || MODE == MODE_F16_K4)
         if (p.occ == 6) return launch_occ<MODE, 6>(ix, a, p, s);
@@ -1631,6 +1645,8 @@ template <int MODE>
 cudaError_t occupancy_mode(const SearchPlan& p, int* blocks) {
     if constexpr (MODE == FINGER_MODE_PLAIN || F8_MODE(MODE))
         if (p.occ == 8) return occupancy_occ<MODE, 8>(p, blocks);
+    if constexpr (MODE == FINGER_MODE_PLAIN || LP_MODE(MODE) || MODE == MODE_F16_K2)
+        if (p.occ == 7) return occupancy_occ<MODE, 7>(p, blocks);
     if constexpr (MODE == FINGER_MODE_PLAIN || MODE == FINGER_MODE_FINGER ||
                   LP_MODE(MODE) || MODE == MODE_F16_K2 || MODE == MODE_F16_K4)
         if (p.occ == 6) return occupancy_occ<MODE, 6>(p, blocks);
