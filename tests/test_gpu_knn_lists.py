@@ -61,3 +61,25 @@ def test_large_k(n, m, clustered):
         assert np.array_equal(ids.cpu().numpy(), order[:nq, :K])
         assert np.array_equal(d.cpu().numpy(), np.take_along_axis(D[:nq], order[:nq, :K], 1))
     ix.close()
+
+
+@pytest.mark.parametrize("candidates", [40, 64])
+def test_graph_of_bounded_segments(candidates):
+    """From 4 query tiles per SM on, the first segments' lists bound the later ones.  Up to
+    64 candidates no list can drop one, so on integer rows (exact products, many equal
+    distances) the graph must be the one that the FP32 candidates give."""
+    import torch
+
+    import paper_2206_11408_gb300 as fg
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(candidates)
+    X = rng.integers(0, 40, (4 * sms * 128 + 77, 6)).astype(np.float32)
+    graphs = []
+    for fp32 in (False, True):
+        ix = fg.Index(X)
+        ix.build_graph(8, candidates=candidates, level_seed=3, fp32_candidates=fp32)
+        graphs.append(ix.get_graph())
+        ix.close()
+    for key in ("adj0", "up_adj", "up_off", "level"):
+        assert np.array_equal(graphs[0][key], graphs[1][key]), key
