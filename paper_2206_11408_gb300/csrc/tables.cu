@@ -576,17 +576,20 @@ __global__ void k_sum_part(const double* Xc, const double* Yc, int64_t np, int m
         for (int k = 0; k < 3; ++k) part[blockIdx.x * 3 + k] = s[k][0];
 }
 
-__global__ void k_sum_final(const double* part, int nb, double* out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double a = 0, b = 0, c = 0;
-    for (int i = 0; i < nb; ++i) {
-        a += part[3 * i];
-        b += part[3 * i + 1];
-        c += part[3 * i + 2];
-    }
-    out[0] = a;
-    out[1] = b;
-    out[2] = c;
+// the blocks' sums in block order, a thread per component, from shared memory (one
+// thread reading them from global memory as it added took 85 us of a table
+// build, three times)
+constexpr int SUM_BLOCKS = 512;
+
+__global__ void k_sum_final(const double* part, double* out) {
+    __shared__ double s[3 * SUM_BLOCKS];
+    for (int i = threadIdx.x; i < 3 * SUM_BLOCKS; i += blockDim.x) s[i] = part[i];
+    __syncthreads();
+    if (threadIdx.x >= 3) return;
+    double a = 0;
+#pragma unroll 16
+    for (int i = 0; i < SUM_BLOCKS; ++i) a += s[3 * i + threadIdx.x];
+    out[threadIdx.x] = a;
 }
 
 // FP8-e4m3 codes of scale * u, 16 bytes per (node c, tile T, step kk of 32
@@ -884,9 +887,8 @@ done:
 static finger_status run_sums(const double* Xc, const double* Yc, int64_t np, int mode, double mu,
                               double muh, double ratio, double* part, double* sums, double h[3],
                               cudaStream_t s) {
-    const int nbp = 512;
-    k_sum_part<<<nbp, 256, 0, s>>>(Xc, Yc, np, mode, mu, muh, ratio, part);
-    k_sum_final<<<1, 32, 0, s>>>(part, nbp, sums);
+    k_sum_part<<<SUM_BLOCKS, 256, 0, s>>>(Xc, Yc, np, mode, mu, muh, ratio, part);
+    k_sum_final<<<1, 256, 0, s>>>(part, sums);
     if (cudaMemcpyAsync(h, sums, 3 * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return FINGER_ERR_CUDA;
@@ -964,7 +966,7 @@ finger_status build_tables(finger_index* ix, const finger_build_params* p, cudaS
     pairs = dalloc<int3>((size_t)np);
     Xc = dalloc<double>((size_t)np);
     Yc = dalloc<double>((size_t)np);
-    part = dalloc<double>(3 * 512);
+    part = dalloc<double>(3 * SUM_BLOCKS);
     sums = dalloc<double>(3);
     evals = dalloc<double>((size_t)m);
     if (!pairs || !Xc || !Yc || !part || !sums || !evals) {
@@ -1073,7 +1075,7 @@ finger_status select_rank(finger_index* ix, const finger_build_params* p, double
     int3* pairs = dalloc<int3>((size_t)np);
     double* Xc = dalloc<double>((size_t)np);
     double* Yk = dalloc<double>((size_t)np * nr);
-    double* part = dalloc<double>(3 * 512);
+    double* part = dalloc<double>(3 * SUM_BLOCKS);
     double* sums = dalloc<double>(3);
     double* evals = dalloc<double>((size_t)m);
     float* P = dalloc<float>((size_t)rp_max * m_pad);
