@@ -289,7 +289,8 @@ finger_status finger_search_batch(finger_index* ix, const float* queries, int64_
  * power-of-two ef bucket of `ef` (16, 32, ..., 1024).  finger_search,
  * finger_search_host and finger_search_batch then launch with it at any ef of
  * that bucket where it fits (a batch plans for the bucket's largest ef), else
- * with the default shape.  The best time in milliseconds is written to
+ * with the default shape; batches too small to fill the GPU with a warp per query
+ * run several warps per query whether tuned or not.  The best time in milliseconds is written to
  * *best_ms when it is not NULL. */
 finger_status finger_autotune(finger_index* ix, const float* queries, int64_t nq, int K, int ef,
                               int64_t* scratch_ids, float* scratch_dists, float* best_ms,
@@ -397,12 +398,13 @@ finger_status finger_mlp_predict(finger_index* ix, const float* feat, int64_t n,
 
 /* Exact K nearest neighbours of nq queries (device, nq x m) over all n base
  * rows by brute force on the GPU; ascending (distance, id), distances summed
- * as (q - x)^2 in FP32.  K <= 256.  For K <= 40 the distance matrix runs on
- * the tensor cores (q.x from BF16 high/low split products accumulated in FP32
- * in tensor memory, candidate lists of 32 or 64 per row, then an exact FP32
- * re-rank); larger K use FP32 FFMA tiles.  Asynchronous (stream-ordered
- * temporaries; the first tensor-core call caches a BF16 split of the base rows,
- * 4 bytes per element). */
+ * as (q - x)^2 in FP32.  K <= 256.  The distance matrix runs on the tensor
+ * cores (q.x from BF16 high/low split products accumulated in FP32 in tensor
+ * memory, candidate lists of 32 or 64 per row and base segment, then an exact
+ * FP32 re-rank); for K > 40 on bases below 4,096 rows, in stream capture, or
+ * without memory for the lists, FP32 FFMA tiles give the same bits.
+ * Asynchronous (stream-ordered temporaries; the first tensor-core call caches a
+ * BF16 split of the base rows, 4 bytes per element). */
 finger_status finger_knn(finger_index* ix, const float* queries, int64_t nq, int K,
                          int64_t* out_ids, float* out_dists, void* stream);
 

@@ -164,7 +164,7 @@ cudaError_t launch_knn(const float4* Xb, int64_t nb, int m4, const float* Q, int
                        int64_t* out_ids, float* out_d, cudaStream_t s, bool causal = false,
                        const int32_t* only = nullptr);
 size_t knn_smem(int K);
-// tensor-core exact kNN (knn_tc.cu): K <= knn_tc_max_k()
+// tensor-core exact kNN (knn_tc.cu): launch_knn_tc for K <= knn_tc_max_k(), _big above
 int knn_tc_max_k();
 cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, int64_t* out_ids,
                           float* out_d, cudaStream_t s);

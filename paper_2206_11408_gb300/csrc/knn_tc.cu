@@ -783,14 +783,20 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
 // block per query sorts the keys of its nseg lists of 64 (np: their count rounded
 // up to a power of two), takes the R = K' smallest, sums their exact distances in
 // the order of the FP32 kernel (a thread per row, dimension after dimension, so
-// both paths return the same bits) and ranks them.  A full list whose keys are all
-// among the R smallest may have dropped more of them: such a query goes on `redo`
-// (count in redo[0]) for the FP32 kernel.
+// both paths return the same bits) and ranks them.  The result has to be certain:
+// a row that is not among the R has an approximate distance of at least the R-th
+// and an exact one of at least that less the approximation's error, so the K-th
+// exact distance has to lie below.  The error is at most 2 (3 2^-18 + 3 ceil(m / 16)
+// 2^-22) |q| max |x| (the dropped parts' products, and an FP32 rounding, taken four
+// times over, for each product added) and 2^-21 of the norms' sum.  A query that is
+// not certain, that has fewer than R candidates (rows before it, or finite
+// distances), or a full list whose keys are all among the R (it may have dropped
+// more) goes on `redo` (count in redo[0]) for the FP32 kernel.
 __global__ void __launch_bounds__(256)
     k_rerank_big(const float4* __restrict__ X, int m4, const float* __restrict__ Q,
                  int64_t q_stride, int q_m, const u64* __restrict__ keys, int nseg, int np, int R,
-                 int K, const int32_t* __restrict__ remap, int64_t* out_ids, float* out_d,
-                 int32_t* redo) {
+                 int K, const int32_t* __restrict__ remap, const float* __restrict__ qn,
+                 const float* __restrict__ xmax, int64_t* out_ids, float* out_d, int32_t* redo) {
     extern __shared__ __align__(16) float4 rb_s[];
     float* qs = reinterpret_cast<float*>(rb_s);          // 4 m4: the query, zero padded
     u64* bk = reinterpret_cast<u64*>(rb_s + m4);         // np keys
@@ -820,10 +826,9 @@ __global__ void __launch_bounds__(256)
         }
     __syncthreads();
     const u64 last = bk[min(R, np) - 1];
-    bool lost = false;
+    bool lost = last >= NO_KEY;
     for (int s = t; s < nseg; s += 256) lost |= top[s] < NO_KEY && top[s] <= last;
-    lost = __syncthreads_or(lost);
-    if (lost) {
+    if (__syncthreads_or(lost)) {
         if (t == 0) redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
         return;
     }
@@ -852,12 +857,28 @@ __global__ void __launch_bounds__(256)
         const u64 k = ex[i];
         int rank = 0;
         for (int j = 0; j < R; ++j) rank += ex[j] < k || (ex[j] == k && j < i);
+        if (rank == K - 1) {
+            const float nq = qn[q], nx = *xmax;
+            const float err = 2.f * (3.f * 0x1p-18f + 3.f * ((q_m + 15) / 16) * 0x1p-22f) * sqrtf(nq) *
+                                  sqrtf(nx) + 0x1p-21f * (nq + nx);
+            if (!(dist_of(k) < dist_of(last) - err)) redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
+        }
         if (rank < K) {
             const int32_t id = (int32_t)(uint32_t)k;
             out_ids[(size_t)q * K + rank] = id < 0 ? (int64_t)-1 : (int64_t)(remap ? remap[id] : id);
             out_d[(size_t)q * K + rank] = id < 0 ? INFINITY : dist_of(k);
         }
     }
+}
+
+// largest of n norms as bits (a NaN's are the largest), atomically into *out
+__global__ void k_max_norm(const float* __restrict__ xn, int64_t n, uint32_t* out) {
+    uint32_t m = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        m = max(m, __float_as_uint(xn[i]) & 0x7FFFFFFFu);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
 }
 
 // ascending bitonic sort of a warp's 32 E keys; lane l holds places E l .. E l + E - 1
@@ -964,6 +985,11 @@ int knn_tc_max_k() { return 40; }
 
 namespace {
 
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+}
+
 // BF16 split of the base rows, made once per index
 cudaError_t ensure_split(finger_index* ix, cudaStream_t s) {
     if (ix->xs_hi) return cudaSuccess;
@@ -979,7 +1005,9 @@ cudaError_t ensure_split(finger_index* ix, cudaStream_t s) {
     }
     k_split_bf16<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(ix->X, n, m, ix->m_pad, ms,
                                                                   ix->xs_hi, ix->xs_lo, nullptr);
-    return cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
+    // done before a call on another stream finds it there
+    return e != cudaSuccess || capturing(s) ? e : cudaStreamSynchronize(s);
 }
 
 // what a launch needs of the base rows (BF16 parts with row stride m rounded to 8)
@@ -1181,18 +1209,22 @@ cudaError_t knn_big(finger_index* ix, const TcBase& x, const float4* Xb, int m4,
     float* qn = nullptr;
     u64* keys = nullptr;
     int32_t* redo = nullptr;
+    float* xmax = nullptr;
     cudaError_t e = cudaSuccess;
     if ((!causal && (cudaMallocAsync(&qh, 2 * (size_t)chunk * ms, s) != cudaSuccess ||
                      cudaMallocAsync(&ql, 2 * (size_t)chunk * ms, s) != cudaSuccess ||
                      cudaMallocAsync(&qn, sizeof(float) * (size_t)chunk, s) != cudaSuccess)) ||
         cudaMallocAsync(&keys, sizeof(u64) * (size_t)chunk * nseg * 64, s) != cudaSuccess ||
-        cudaMallocAsync(&redo, sizeof(int32_t) * (size_t)(chunk + 1), s) != cudaSuccess ||
+        cudaMallocAsync(&redo, sizeof(int32_t) * (size_t)(chunk + 2), s) != cudaSuccess ||
         cudaFuncSetAttribute(k_rerank_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess) {
         cudaGetLastError();
         e = launch_knn(Xb, x.n, m4, Q, q_stride, q_m, nq, K, causal, remap, out_ids, out_d, s, causal);
         goto done;
     }
+    xmax = reinterpret_cast<float*>(redo) + chunk + 1;
+    if ((e = cudaMemsetAsync(xmax, 0, sizeof(float), s)) != cudaSuccess) goto done;
+    k_max_norm<<<256, 256, 0, s>>>(x.xn, x.n, reinterpret_cast<uint32_t*>(xmax));
     for (int64_t lo = 0; lo < nq && e == cudaSuccess; lo += chunk) {
         const int64_t c = std::min(chunk, nq - lo);
         const float* q = Q + lo * q_stride;
@@ -1205,7 +1237,8 @@ cudaError_t knn_big(finger_index* ix, const TcBase& x, const float4* Xb, int m4,
                       causal ? CAUSAL : INTERLEAVED, keys, nullptr, s);
         if (e != cudaSuccess) break;
         k_rerank_big<<<(unsigned)c, 256, smem, s>>>(Xb, m4, q, q_stride, q_m, keys, nseg, np, R, K,
-                                                    remap, out_ids + lo * K, out_d + lo * K, redo);
+                                                    remap, causal ? x.xn : qn, xmax, out_ids + lo * K,
+                                                    out_d + lo * K, redo);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         e = launch_knn(Xb, x.n, m4, q, q_stride, q_m, c, K, causal, remap, out_ids + lo * K,
                        out_d + lo * K, s, causal, redo);
@@ -1221,11 +1254,6 @@ done:
 
 // rows from which the tensor cores serve K > 40: 32 tiles, two per segment
 constexpr int64_t BIG_MIN_ROWS = 32 * TB;
-
-bool capturing(cudaStream_t s) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
-}
 
 }  // namespace
 
