@@ -73,6 +73,14 @@ __device__ __forceinline__ float dist_of(u64 k) {
     return __uint_as_float(o ^ (o & 0x80000000u ? 0x80000000u : 0xFFFFFFFFu));
 }
 
+// Bound on |approximate - exact| squared distance for norms nq and nx and m dimensions:
+// 2 (3 2^-18 + 3 ceil(m / 16) 2^-22) |q| |x| (the dropped parts' products, and an FP32
+// rounding, taken four times over, for each product added) and 2^-21 of the norms' sum
+__device__ __forceinline__ float split_error(float nq, float nx, int m) {
+    return 2.f * (3.f * 0x1p-18f + 3.f * ((m + 15) / 16) * 0x1p-22f) * sqrtf(nq) * sqrtf(nx) +
+           0x1p-21f * (nq + nx);
+}
+
 struct TcArgs {
     int64_t nq, n;
     int nchunk;           // ceil(m / 64)
@@ -89,6 +97,8 @@ struct TcArgs {
     const float* qn;      // ||q||^2 (FP32), nq
     const float* xn;      // ||x||^2 (FP32), n
     u64* keys;            // nq x nseg x KP candidate keys
+    const float* xmax;    // with bound: the largest base norm
+    int m;
     uint32_t* bound;      // optional: per row, the smallest K'-th distance of its finished
                           // segments (ord_of), 0xFFFFFFFF before the first
     int* err;             // device status word (FINGER_ERR_LIMIT on a wait timeout)
@@ -515,7 +525,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             uint32_t bound = 0xFF800000u;
             if (a.pilot && seg >= a.pilot) bound = min(bound, pilots);
             if (a.bound && qi < a.nq) bound = min(bound, *(volatile uint32_t*)(a.bound + qi));
-            const float cap = bound < 0xFF800000u ? dist_of((u64)(bound + 1u) << 32) : INFINITY;
+            float cap = bound < 0xFF800000u ? dist_of((u64)(bound + 1u) << 32) : INFINITY;
+            // (a kNN launch keeps what the approximation may have misplaced, see k_rerank)
+            if (a.bound) cap += 2.f * split_error(qn, *a.xmax, a.m);
             float thr = qi < a.nq ? cap : -INFINITY;
             int cnt = 0;                                    // pending candidates of the row
             top.clear();
@@ -686,12 +698,16 @@ __device__ __forceinline__ void warp_smallest(u64 (&k)[E], int R, u64* out, int 
 }
 
 // Final step of a kNN launch: the KP smallest approximate keys of a query's lists,
-// their exact FP32 distances, the K best by (distance, id).  W warps per query
-// (E keys per lane: 32 E W >= the query's keys); with W = 1 four queries per block.
+// their exact FP32 distances, the K best by (distance, id).  Where the approximation's
+// error reaches from the KP-th approximate distance to the K-th exact one (rows far
+// from the origin, many equal distances), the lists' other keys get their exact
+// distances too.  W warps per query (E keys per lane: 32 E W >= the query's keys); with
+// W = 1 four queries per block.
 template <int W, int E>
 __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
     k_rerank(const float4* __restrict__ X, int m4, const float* __restrict__ Q, int m, int64_t nq,
-             const u64* __restrict__ keys, int nc, int KP, int K, int64_t* out_ids, float* out_d) {
+             const u64* __restrict__ keys, int nc, int KP, int K, const float* __restrict__ qn,
+             const float* __restrict__ xmax, int64_t* out_ids, float* out_d) {
     constexpr int QPB = W == 1 ? 4 : 1;
     __shared__ u64 sel_s[QPB][64];
     __shared__ u64 part_s[W == 1 ? 1 : W * 64];
@@ -721,6 +737,9 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
         }
         __syncthreads();
     }
+    const u64 last = sel[KP - 1];   // the KP-th approximate key
+    if constexpr (W == 1) __syncwarp();
+    else __syncthreads();
     // exact distances, four rows in flight per warp; each key gets its exact distance
     const float* qr = Q + (size_t)q * m;
     constexpr int U = 4;
@@ -764,6 +783,51 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
     if constexpr (W == 1) __syncwarp();
     else __syncthreads();
     if (wq != 0) return;
+    if (last < NO_KEY) {
+        // the K-th exact key: the one that K - 1 others precede
+        u64 kth = ~0ull;
+        for (int i = lane; i < KP; i += 32) {
+            int rank = 0;
+            for (int j = 0; j < KP; ++j) rank += sel[j] < sel[i];
+            if (rank == K - 1) kth = sel[i];
+        }
+        kth = warp_min(kth);
+        const float err = split_error(qn[q], *xmax, m);
+        if (!(dist_of(kth) < dist_of(last) - err)) {
+            const float lim = dist_of(kth) + err;   // above it no key can be nearer
+            for (int c0 = 0; c0 < nc; c0 += 32) {
+                const u64 kc = c0 + lane < nc ? kr[c0 + lane] : NO_KEY;
+                unsigned more = __ballot_sync(
+                    0xffffffffu, kc < NO_KEY && kc > last && !(dist_of(kc) > lim));
+                while (more) {
+                    const uint32_t id = __shfl_sync(0xffffffffu, (uint32_t)kc, __ffs(more) - 1);
+                    more &= more - 1;
+                    float acc = 0.f;
+                    for (int c = lane; c < m4; c += 32) {
+                        const float4 x = __ldg(X + (size_t)id * m4 + c);
+                        const int e = 4 * c;
+                        float dlt;
+                        dlt = (e < m ? qr[e] : 0.f) - x.x; acc = fmaf(dlt, dlt, acc);
+                        dlt = (e + 1 < m ? qr[e + 1] : 0.f) - x.y; acc = fmaf(dlt, dlt, acc);
+                        dlt = (e + 2 < m ? qr[e + 2] : 0.f) - x.z; acc = fmaf(dlt, dlt, acc);
+                        dlt = (e + 3 < m ? qr[e + 3] : 0.f) - x.w; acc = fmaf(dlt, dlt, acc);
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                    // in the place of the largest kept key, if it is smaller
+                    const u64 key = (u64)ord_of(acc) << 32 | id;
+                    const u64 a = sel[lane], b = KP > 32 ? sel[lane + 32] : 0ull;
+                    const u64 top = ~warp_min(~(a > b ? a : b));
+                    __syncwarp();
+                    if (key < top) {
+                        if (a == top) sel[lane] = key;
+                        else if (KP > 32 && b == top) sel[lane + 32] = key;
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+    }
     for (int i = lane; i < KP; i += 32) {
         const u64 ki = sel[i];
         int rank = 0;
@@ -786,10 +850,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
 // both paths return the same bits) and ranks them.  The result has to be certain:
 // a row that is not among the R has an approximate distance of at least the R-th
 // and an exact one of at least that less the approximation's error, so the K-th
-// exact distance has to lie below.  The error is at most 2 (3 2^-18 + 3 ceil(m / 16)
-// 2^-22) |q| max |x| (the dropped parts' products, and an FP32 rounding, taken four
-// times over, for each product added) and 2^-21 of the norms' sum.  A query that is
-// not certain, that has fewer than R candidates (rows before it, or finite
+// exact distance has to lie below.  A query that is not certain, that has fewer than R candidates (rows before it, or finite
 // distances), or a full list whose keys are all among the R (it may have dropped
 // more) goes on `redo` (count in redo[0]) for the FP32 kernel.
 __global__ void __launch_bounds__(256)
@@ -858,10 +919,7 @@ __global__ void __launch_bounds__(256)
         int rank = 0;
         for (int j = 0; j < R; ++j) rank += ex[j] < k || (ex[j] == k && j < i);
         if (rank == K - 1) {
-            const float nq = qn[q], nx = *xmax;
-            const float err = 2.f * (3.f * 0x1p-18f + 3.f * ((q_m + 15) / 16) * 0x1p-22f) * sqrtf(nq) *
-                                  sqrtf(nx) + 0x1p-21f * (nq + nx);
-            if (!(dist_of(k) < dist_of(last) - err)) redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
+            if (!(dist_of(k) < dist_of(last) - split_error(qn[q], *xmax, q_m))) redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
         }
         if (rank < K) {
             const int32_t id = (int32_t)(uint32_t)k;
@@ -1025,7 +1083,8 @@ enum TcOrder { CONTIGUOUS, INTERLEAVED, CAUSAL };
 // one launch of k_knn_tc over nq query rows (BF16 parts qh/ql) against the base
 cudaError_t run_items(finger_index* ix, const TcBase& x, const __nv_bfloat16* qh,
                       const __nv_bfloat16* ql, const float* qn, int64_t nq, int KP, int nseg,
-                      TcOrder order, u64* keys, uint32_t* bound, cudaStream_t s, int want = 0) {
+                      TcOrder order, u64* keys, uint32_t* bound, const float* xmax, cudaStream_t s,
+                      int want = 0) {
     const int ms = (x.m + 7) & ~7;
     CUtensorMap maps[4];
     if (!make_map(&maps[0], qh, nq, x.m, ms) || !make_map(&maps[1], ql, nq, x.m, ms) ||
@@ -1047,6 +1106,8 @@ cudaError_t run_items(finger_index* ix, const TcBase& x, const __nv_bfloat16* qh
     a.xn = x.xn;
     a.keys = keys;
     a.bound = bound;
+    a.xmax = xmax;
+    a.m = x.m;
     a.err = ix->err;
     // want > 0: the smallest `want` keys of a causal launch's lists are used.  With query
     // tiles enough for all SMs a CTA keeps a tile's segments, and the first of them
@@ -1102,7 +1163,9 @@ cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, i
     float* qn = nullptr;
     u64* keys = nullptr;
     uint32_t* bound = nullptr;
+    float* xmax = nullptr;
     if (cudaMallocAsync(&bound, sizeof(uint32_t) * (size_t)nq, s) != cudaSuccess ||
+        cudaMallocAsync(&xmax, sizeof(float), s) != cudaSuccess ||
         cudaMallocAsync(&qh, sizeof(__nv_bfloat16) * (size_t)nq * ms, s) != cudaSuccess ||
         cudaMallocAsync(&ql, sizeof(__nv_bfloat16) * (size_t)nq * ms, s) != cudaSuccess ||
         cudaMallocAsync(&qn, sizeof(float) * (size_t)nq, s) != cudaSuccess ||
@@ -1111,16 +1174,18 @@ cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, i
         goto done;
     }
     if ((e = cudaMemsetAsync(bound, 0xFF, sizeof(uint32_t) * (size_t)nq, s)) != cudaSuccess) goto done;
+    if ((e = cudaMemsetAsync(xmax, 0, sizeof(float), s)) != cudaSuccess) goto done;
+    k_max_norm<<<256, 256, 0, s>>>(ix->xnorm2, n, reinterpret_cast<uint32_t*>(xmax));
     k_split_bf16<<<(unsigned)((nq * 32 + 255) / 256), 256, 0, s>>>(Q, nq, m, m, ms, qh, ql, qn);
     if ((e = cudaGetLastError()) != cudaSuccess) goto done;
-    if ((e = run_items(ix, base_of(ix), qh, ql, qn, nq, KP, nseg, CONTIGUOUS, keys, bound, s)) != cudaSuccess)
+    if ((e = run_items(ix, base_of(ix), qh, ql, qn, nq, KP, nseg, CONTIGUOUS, keys, bound, xmax, s)) != cudaSuccess)
         goto done;
     {
         const float4* X = reinterpret_cast<const float4*>(ix->X);
         // a query tile's lists: a few for large batches, up to one per SM for small ones
 #define FG_RERANK(W_, E_)                                                                        \
     k_rerank<W_, E_><<<(unsigned)(W_ == 1 ? (nq + 3) / 4 : nq), W_ == 1 ? 128 : 32 * W_, 0, s>>>( \
-        X, ix->m4, Q, m, nq, keys, nc, KP, K, out_ids, out_d)
+        X, ix->m4, Q, m, nq, keys, nc, KP, K, qn, xmax, out_ids, out_d)
         if (nc <= 32 * 4) FG_RERANK(1, 4);
         else if (nc <= 32 * 16) FG_RERANK(1, 16);
         else if (nc <= 8 * 32 * 16) FG_RERANK(8, 16);
@@ -1135,6 +1200,7 @@ done:
     if (ql) cudaFreeAsync(ql, s);
     if (qn) cudaFreeAsync(qn, s);
     if (bound) cudaFreeAsync(bound, s);
+    if (xmax) cudaFreeAsync(xmax, s);
     if (keys) cudaFreeAsync(keys, s);
     return e;
 }
@@ -1160,7 +1226,7 @@ cudaError_t launch_knn_tc_causal(finger_index* ix, int K, int64_t* out_ids, floa
         goto done;
     }
     if ((e = run_items(ix, base_of(ix), ix->xs_hi, ix->xs_lo, ix->xnorm2, n, KP, NSEG, CAUSAL, keys,
-                       nullptr, s, K)) != cudaSuccess)
+                       nullptr, nullptr, s, K)) != cudaSuccess)
         goto done;
     k_merge_topk<<<(unsigned)((n + 3) / 4), 128, 0, s>>>(keys, n, K, out_ids, out_d);
     e = cudaGetLastError();
@@ -1234,7 +1300,7 @@ cudaError_t knn_big(finger_index* ix, const TcBase& x, const float4* Xb, int m4,
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         if ((e = cudaMemsetAsync(redo, 0, sizeof(int32_t), s)) != cudaSuccess) break;
         e = run_items(ix, x, causal ? x.hi : qh, causal ? x.lo : ql, causal ? x.xn : qn, c, 64, nseg,
-                      causal ? CAUSAL : INTERLEAVED, keys, nullptr, s);
+                      causal ? CAUSAL : INTERLEAVED, keys, nullptr, nullptr, s);
         if (e != cudaSuccess) break;
         k_rerank_big<<<(unsigned)c, 256, smem, s>>>(Xb, m4, q, q_stride, q_m, keys, nseg, np, R, K,
                                                     remap, causal ? x.xn : qn, xmax, out_ids + lo * K,

@@ -85,10 +85,13 @@ def test_graph_of_bounded_segments(candidates):
         assert np.array_equal(graphs[0][key], graphs[1][key]), key
 
 
-@pytest.mark.parametrize("kind", ["offset", "inf_query", "inf_row", "overflow"])
-def test_large_k_where_the_products_decide_nothing(kind):
-    """Rows far from the origin (the split products' error exceeds the distances' spread),
-    infinities, and norms that overflow: the FP32 kernel's keys, as without tensor cores."""
+@pytest.mark.parametrize("kind,K", [("near", 10), ("near", 16), ("near", 40), ("near", 100),
+                                    ("offset", 100), ("inf_query", 100), ("inf_row", 100),
+                                    ("overflow", 100)])
+def test_where_the_products_decide_little(kind, K):
+    """Rows away from the origin: the split products' error reaches over the kept keys
+    ("near": their order alone; "offset": everything); infinities; norms that overflow.
+    The nearest by the rows' own FP32 differences all the same."""
     import torch
 
     import paper_2206_11408_gb300 as fg
@@ -96,9 +99,9 @@ def test_large_k_where_the_products_decide_nothing(kind):
     rng = np.random.default_rng(5)
     X = rng.standard_normal((5000, 32)).astype(np.float32)
     Q = rng.standard_normal((40, 32)).astype(np.float32)
-    if kind == "offset":
-        X += 3000
-        Q += 3000
+    if kind in ("near", "offset"):
+        X += 60 if kind == "near" else 3000
+        Q += 60 if kind == "near" else 3000
     elif kind == "inf_query":
         Q[3, 4] = np.inf
     elif kind == "inf_row":
@@ -107,7 +110,7 @@ def test_large_k_where_the_products_decide_nothing(kind):
         X[:, 0] += 2e19
         Q[:, 0] += 2e19
     ix = fg.Index(X)
-    ids, d = ix.knn(torch.from_numpy(Q).cuda(), 100)
+    ids, d = ix.knn(torch.from_numpy(Q).cuda(), K)
     ix.sync()
     ix.close()
     ids, d = ids.cpu().numpy(), d.cpu().numpy()
@@ -116,10 +119,10 @@ def test_large_k_where_the_products_decide_nothing(kind):
             diff = (Q[i] - X).astype(np.float64)
             ref = (diff ** 2).sum(1)
         if np.isnan(ref).any() or np.isinf(ref).all():
-            assert np.array_equal(ids[i], np.arange(100)) and np.isinf(d[i]).all()
+            assert np.array_equal(ids[i], np.arange(K)) and np.isinf(d[i]).all()
             continue
         # every returned distance is the row's own, ascending, and none nearer is missing
         got = ref[ids[i]]
         np.testing.assert_allclose(d[i], got, rtol=1e-5)
-        assert (np.diff(d[i]) >= 0).all() and len(set(ids[i])) == 100
-        assert np.sort(ref)[99] >= got.max() * (1 - 1e-5)
+        assert (np.diff(d[i]) >= 0).all() and len(set(ids[i])) == K
+        assert np.sort(ref)[K - 1] >= got.max() * (1 - 1e-5)
