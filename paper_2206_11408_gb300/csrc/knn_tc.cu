@@ -81,6 +81,22 @@ __device__ __forceinline__ float split_error(float nq, float nx, int m) {
            0x1p-21f * (nq + nx);
 }
 
+// The base's norms as the error bounds need them: the largest finite one, and whether
+// some are +inf (rows with infinities, or whose norm overflows).  A NaN's row is nobody's
+// neighbour, and a row of infinite norm has no finite approximate distance.
+struct NormMax {
+    float finite;
+    uint32_t inf;
+};
+
+// Whether a row of infinite norm may be nearer than kth: its length is at least
+// 1.8e19 (the root of the largest float, less 2 %), so |q - x| >= 1.8e19 - |q|.
+// (A NaN or infinite nq or kth: it may.)
+__device__ __forceinline__ bool inf_rows_reach(const NormMax& x, float nq, float kth) {
+    const float gap = 1.8e19f - 1.01f * sqrtf(nq);
+    return x.inf && !(gap > 0.f && kth < 0.99f * gap * gap);
+}
+
 struct TcArgs {
     int64_t nq, n;
     int nchunk;           // ceil(m / 64)
@@ -97,7 +113,7 @@ struct TcArgs {
     const float* qn;      // ||q||^2 (FP32), nq
     const float* xn;      // ||x||^2 (FP32), n
     u64* keys;            // nq x nseg x KP candidate keys
-    const float* xmax;    // with bound: the largest base norm
+    const NormMax* xmax;  // with bound: the base's norms
     int m;
     uint32_t* bound;      // optional: per row, the smallest K'-th distance of its finished
                           // segments (ord_of), 0xFFFFFFFF before the first
@@ -527,7 +543,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             if (a.bound && qi < a.nq) bound = min(bound, *(volatile uint32_t*)(a.bound + qi));
             float cap = bound < 0xFF800000u ? dist_of((u64)(bound + 1u) << 32) : INFINITY;
             // (a kNN launch keeps what the approximation may have misplaced, see k_rerank)
-            if (a.bound) cap += 2.f * split_error(qn, *a.xmax, a.m);
+            if (a.bound) cap += 2.f * split_error(qn, a.xmax->finite, a.m);
             float thr = qi < a.nq ? cap : -INFINITY;
             int cnt = 0;                                    // pending candidates of the row
             top.clear();
@@ -707,7 +723,7 @@ template <int W, int E>
 __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
     k_rerank(const float4* __restrict__ X, int m4, const float* __restrict__ Q, int m, int64_t nq,
              const u64* __restrict__ keys, int nc, int KP, int K, const float* __restrict__ qn,
-             const float* __restrict__ xmax, int64_t* out_ids, float* out_d) {
+             const NormMax* __restrict__ xmax, int64_t* out_ids, float* out_d) {
     constexpr int QPB = W == 1 ? 4 : 1;
     __shared__ u64 sel_s[QPB][64];
     __shared__ u64 part_s[W == 1 ? 1 : W * 64];
@@ -792,7 +808,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
             if (rank == K - 1) kth = sel[i];
         }
         kth = warp_min(kth);
-        const float err = split_error(qn[q], *xmax, m);
+        const float err = split_error(qn[q], xmax->finite, m);
         if (!(dist_of(kth) < dist_of(last) - err)) {
             const float lim = dist_of(kth) + err;   // above it no key can be nearer
             for (int c0 = 0; c0 < nc; c0 += 32) {
@@ -857,7 +873,7 @@ __global__ void __launch_bounds__(256)
     k_rerank_big(const float4* __restrict__ X, int m4, const float* __restrict__ Q,
                  int64_t q_stride, int q_m, const u64* __restrict__ keys, int nseg, int np, int R,
                  int K, const int32_t* __restrict__ remap, const float* __restrict__ qn,
-                 const float* __restrict__ xmax, int64_t* out_ids, float* out_d, int32_t* redo) {
+                 const NormMax* __restrict__ xmax, int64_t* out_ids, float* out_d, int32_t* redo) {
     extern __shared__ __align__(16) float4 rb_s[];
     float* qs = reinterpret_cast<float*>(rb_s);          // 4 m4: the query, zero padded
     u64* bk = reinterpret_cast<u64*>(rb_s + m4);         // np keys
@@ -919,7 +935,10 @@ __global__ void __launch_bounds__(256)
         int rank = 0;
         for (int j = 0; j < R; ++j) rank += ex[j] < k || (ex[j] == k && j < i);
         if (rank == K - 1) {
-            if (!(dist_of(k) < dist_of(last) - split_error(qn[q], *xmax, q_m))) redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
+            const float kth = dist_of(k);
+            if (!(kth < dist_of(last) - split_error(qn[q], xmax->finite, q_m)) ||
+                inf_rows_reach(*xmax, qn[q], kth))
+                redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
         }
         if (rank < K) {
             const int32_t id = (int32_t)(uint32_t)k;
@@ -929,14 +948,21 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// largest of n norms as bits (a NaN's are the largest), atomically into *out
-__global__ void k_max_norm(const float* __restrict__ xn, int64_t n, uint32_t* out) {
-    uint32_t m = 0;
+// the NormMax of n norms (zeroed before)
+__global__ void k_max_norm(const float* __restrict__ xn, int64_t n, NormMax* out) {
+    uint32_t m = 0, inf = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, __float_as_uint(xn[i]) & 0x7FFFFFFFu);
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const float x = xn[i];
+        if (x < INFINITY) m = max(m, __float_as_uint(x));
+        inf |= x == INFINITY;
+    }
     m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+    inf = __reduce_or_sync(0xffffffffu, inf);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(reinterpret_cast<uint32_t*>(&out->finite), m);
+        if (inf) atomicOr(&out->inf, 1u);
+    }
 }
 
 // ascending bitonic sort of a warp's 32 E keys; lane l holds places E l .. E l + E - 1
@@ -1083,7 +1109,7 @@ enum TcOrder { CONTIGUOUS, INTERLEAVED, CAUSAL };
 // one launch of k_knn_tc over nq query rows (BF16 parts qh/ql) against the base
 cudaError_t run_items(finger_index* ix, const TcBase& x, const __nv_bfloat16* qh,
                       const __nv_bfloat16* ql, const float* qn, int64_t nq, int KP, int nseg,
-                      TcOrder order, u64* keys, uint32_t* bound, const float* xmax, cudaStream_t s,
+                      TcOrder order, u64* keys, uint32_t* bound, const NormMax* xmax, cudaStream_t s,
                       int want = 0) {
     const int ms = (x.m + 7) & ~7;
     CUtensorMap maps[4];
@@ -1163,9 +1189,9 @@ cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, i
     float* qn = nullptr;
     u64* keys = nullptr;
     uint32_t* bound = nullptr;
-    float* xmax = nullptr;
+    NormMax* xmax = nullptr;
     if (cudaMallocAsync(&bound, sizeof(uint32_t) * (size_t)nq, s) != cudaSuccess ||
-        cudaMallocAsync(&xmax, sizeof(float), s) != cudaSuccess ||
+        cudaMallocAsync(&xmax, sizeof(NormMax), s) != cudaSuccess ||
         cudaMallocAsync(&qh, sizeof(__nv_bfloat16) * (size_t)nq * ms, s) != cudaSuccess ||
         cudaMallocAsync(&ql, sizeof(__nv_bfloat16) * (size_t)nq * ms, s) != cudaSuccess ||
         cudaMallocAsync(&qn, sizeof(float) * (size_t)nq, s) != cudaSuccess ||
@@ -1174,8 +1200,8 @@ cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, i
         goto done;
     }
     if ((e = cudaMemsetAsync(bound, 0xFF, sizeof(uint32_t) * (size_t)nq, s)) != cudaSuccess) goto done;
-    if ((e = cudaMemsetAsync(xmax, 0, sizeof(float), s)) != cudaSuccess) goto done;
-    k_max_norm<<<256, 256, 0, s>>>(ix->xnorm2, n, reinterpret_cast<uint32_t*>(xmax));
+    if ((e = cudaMemsetAsync(xmax, 0, sizeof(NormMax), s)) != cudaSuccess) goto done;
+    k_max_norm<<<256, 256, 0, s>>>(ix->xnorm2, n, xmax);
     k_split_bf16<<<(unsigned)((nq * 32 + 255) / 256), 256, 0, s>>>(Q, nq, m, m, ms, qh, ql, qn);
     if ((e = cudaGetLastError()) != cudaSuccess) goto done;
     if ((e = run_items(ix, base_of(ix), qh, ql, qn, nq, KP, nseg, CONTIGUOUS, keys, bound, xmax, s)) != cudaSuccess)
@@ -1275,22 +1301,22 @@ cudaError_t knn_big(finger_index* ix, const TcBase& x, const float4* Xb, int m4,
     float* qn = nullptr;
     u64* keys = nullptr;
     int32_t* redo = nullptr;
-    float* xmax = nullptr;
+    NormMax* xmax = nullptr;
     cudaError_t e = cudaSuccess;
     if ((!causal && (cudaMallocAsync(&qh, 2 * (size_t)chunk * ms, s) != cudaSuccess ||
                      cudaMallocAsync(&ql, 2 * (size_t)chunk * ms, s) != cudaSuccess ||
                      cudaMallocAsync(&qn, sizeof(float) * (size_t)chunk, s) != cudaSuccess)) ||
         cudaMallocAsync(&keys, sizeof(u64) * (size_t)chunk * nseg * 64, s) != cudaSuccess ||
-        cudaMallocAsync(&redo, sizeof(int32_t) * (size_t)(chunk + 2), s) != cudaSuccess ||
+        cudaMallocAsync(&xmax, sizeof(NormMax), s) != cudaSuccess ||
+        cudaMallocAsync(&redo, sizeof(int32_t) * (size_t)(chunk + 1), s) != cudaSuccess ||
         cudaFuncSetAttribute(k_rerank_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess) {
         cudaGetLastError();
         e = launch_knn(Xb, x.n, m4, Q, q_stride, q_m, nq, K, causal, remap, out_ids, out_d, s, causal);
         goto done;
     }
-    xmax = reinterpret_cast<float*>(redo) + chunk + 1;
-    if ((e = cudaMemsetAsync(xmax, 0, sizeof(float), s)) != cudaSuccess) goto done;
-    k_max_norm<<<256, 256, 0, s>>>(x.xn, x.n, reinterpret_cast<uint32_t*>(xmax));
+    if ((e = cudaMemsetAsync(xmax, 0, sizeof(NormMax), s)) != cudaSuccess) goto done;
+    k_max_norm<<<256, 256, 0, s>>>(x.xn, x.n, xmax);
     for (int64_t lo = 0; lo < nq && e == cudaSuccess; lo += chunk) {
         const int64_t c = std::min(chunk, nq - lo);
         const float* q = Q + lo * q_stride;
@@ -1314,6 +1340,7 @@ done:
     if (ql) cudaFreeAsync(ql, s);
     if (qn) cudaFreeAsync(qn, s);
     if (keys) cudaFreeAsync(keys, s);
+    if (xmax) cudaFreeAsync(xmax, s);
     if (redo) cudaFreeAsync(redo, s);
     return e;
 }
