@@ -1145,33 +1145,64 @@ cudaError_t run_items(finger_index* ix, const TcBase& x, const __nv_bfloat16* qh
     return res ? run_tc<64, true>(maps, a, grid, s) : run_tc<64, false>(maps, a, grid, s);
 }
 
-// Base segments of a kNN launch.  The items (query tile, segment) are dealt to one
-// CTA per SM in waves, segment by segment, so the CTAs of a wave scan the same rows
-// at the same time: a segment of at most 48 MB of BF16 parts stays in L2 for
-// them.  (One equal range of the (query tile, base tile) sequence per CTA balances
-// without waves, but each CTA then scans rows of its own and DRAM bounds it: 10,000
-// queries x 1M x 128 took 11.6 ms.)  From there the smallest count whose last
-// wave costs at most 3 %, or the best of the next 32; each segment adds a list of
-// K' per row to fill and to merge.
-int base_segments(const finger_index* ix, int nqt, int nbt) {
-    const int64_t bytes = (int64_t)nbt * TB * ((ix->m + 7) & ~7) * 4;
-    const int lo = (int)std::min<int64_t>(nbt, std::max<int64_t>(bytes / (48 << 20), 1));
-    const int64_t G = ix->num_sms;
-    int best = lo;
+// How a kNN of K <= 40 is divided: queries per pass, and base segments.  The items
+// (query tile, segment) are dealt to one CTA per SM in waves, segment by segment, so
+// the CTAs of a wave scan the same rows at the same time: a segment of at most 48 MB of
+// BF16 parts stays in L2 for them.  (One equal range of the (query tile, base tile)
+// sequence per CTA balances without waves, but each CTA then scans rows of its own and
+// DRAM bounds it: 10,000 queries x 1M x 128 took 11.6 ms.)  From there the smallest
+// count whose last wave costs at most 3 %, or the best of the next 32; each segment
+// adds a list of K' per row to fill and to merge.  Above MAX_KEYS / K' such segments
+// (12.9 or 25.8 GB of parts) they grow instead: k_rerank takes MAX_KEYS keys per query
+// and each pass reads the base from DRAM anyway.  Passes keep the lists below twice
+// LIST_BYTES for any number of queries; one still has 4,096 items or more.
+constexpr int MAX_KEYS = 16 * 32 * 32;   // the widest k_rerank: 16 warps of 32 keys per lane
+constexpr int64_t LIST_BYTES = 256 << 20;
+
+struct KnnPlan {
+    int KP, nseg;
+    int64_t chunk;   // queries per pass
+};
+
+KnnPlan knn_plan(int64_t n, int m, int64_t nq, int K, int num_sms, int64_t most) {
+    KnnPlan p;
+    p.KP = K <= 16 ? 32 : 64;
+    const int64_t nbt = (n + TB - 1) / TB, G = num_sms;
+    const int64_t bytes = nbt * TB * ((m + 7) & ~7) * 4;
+    const int64_t top = std::min<int64_t>(nbt, MAX_KEYS / p.KP);
+    const int64_t lo = std::min<int64_t>(top, std::max<int64_t>(bytes / (48 << 20), 1));
+    const int64_t row = 8 * p.KP;   // list bytes per query and segment
+    int64_t c = std::min(nq, std::min(most, std::max<int64_t>(TQ, LIST_BYTES / (row * lo))));
+    const int64_t passes = (nq + c - 1) / c;
+    c = std::min(nq, ((nq + passes - 1) / passes + TQ - 1) / TQ * TQ);
+    p.chunk = c;
+    const int64_t nqt = (c + TQ - 1) / TQ;
+    const int64_t hi = std::min(std::min(top, std::max(lo + 32, (G + nqt - 1) / nqt)),
+                                std::max(lo, 2 * LIST_BYTES / (row * c)));
+    p.nseg = (int)lo;
     double best_eff = 0;
-    for (int S = lo; S <= std::min<int64_t>(nbt, std::max<int64_t>(lo + 32, (G + nqt - 1) / nqt)); ++S) {
-        const int64_t items = (int64_t)nqt * S;
+    for (int64_t S = lo; S <= hi; ++S) {
+        const int64_t items = nqt * S;
         const double eff = (double)items / ((items + G - 1) / G * G);
         if (eff > best_eff + 0.002) {
             best_eff = eff;
-            best = S;
+            p.nseg = (int)S;
         }
         if (best_eff >= 0.97) break;
     }
-    return best;
+    return p;
 }
 
 }  // namespace
+
+// the plan of a call, for tests on the host: {K', segments, queries per pass, most keys}
+extern "C" void fg_knn_plan(int64_t n, int m, int64_t nq, int K, int num_sms, int64_t* out) {
+    const KnnPlan p = knn_plan(n, m, nq, K, num_sms, nq);
+    out[0] = p.KP;
+    out[1] = p.nseg;
+    out[2] = p.chunk;
+    out[3] = MAX_KEYS;
+}
 
 cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, int64_t* out_ids,
                           float* out_d, cudaStream_t s) {
@@ -1180,54 +1211,66 @@ cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, i
     const int64_t n = ix->n;
     cudaError_t e = ensure_split(ix, s);
     if (e != cudaSuccess) return e;
-    const int KP = K <= 16 ? 32 : 64;
-    const int nqt = (int)((nq + TQ - 1) / TQ);
-    const int nbt = (int)((n + TB - 1) / TB);
-    const int nseg = base_segments(ix, nqt, nbt);   // any is exact here: K <= KP
-    const int nc = nseg * KP;
     __nv_bfloat16 *qh = nullptr, *ql = nullptr;
     float* qn = nullptr;
     u64* keys = nullptr;
     uint32_t* bound = nullptr;
     NormMax* xmax = nullptr;
-    if (cudaMallocAsync(&bound, sizeof(uint32_t) * (size_t)nq, s) != cudaSuccess ||
-        cudaMallocAsync(&xmax, sizeof(NormMax), s) != cudaSuccess ||
-        cudaMallocAsync(&qh, sizeof(__nv_bfloat16) * (size_t)nq * ms, s) != cudaSuccess ||
-        cudaMallocAsync(&ql, sizeof(__nv_bfloat16) * (size_t)nq * ms, s) != cudaSuccess ||
-        cudaMallocAsync(&qn, sizeof(float) * (size_t)nq, s) != cudaSuccess ||
-        cudaMallocAsync(&keys, sizeof(u64) * (size_t)nq * nc, s) != cudaSuccess) {
-        e = cudaErrorMemoryAllocation;
-        goto done;
+    // stream-ordered frees: the temporaries live until the kernels below finish
+    auto release = [&]() {
+        if (qh) cudaFreeAsync(qh, s);
+        if (ql) cudaFreeAsync(ql, s);
+        if (qn) cudaFreeAsync(qn, s);
+        if (bound) cudaFreeAsync(bound, s);
+        if (xmax) cudaFreeAsync(xmax, s);
+        if (keys) cudaFreeAsync(keys, s);
+        qh = ql = nullptr;
+        qn = nullptr;
+        bound = nullptr;
+        xmax = nullptr;
+        keys = nullptr;
+    };
+    KnnPlan p;
+    for (int64_t most = nq;; most = p.chunk / 2) {   // fewer queries per pass where memory is short
+        p = knn_plan(n, m, nq, K, ix->num_sms, most);
+        const size_t c = (size_t)p.chunk;
+        if (cudaMallocAsync(&bound, sizeof(uint32_t) * c, s) == cudaSuccess &&
+            cudaMallocAsync(&xmax, sizeof(NormMax), s) == cudaSuccess &&
+            cudaMallocAsync(&qh, sizeof(__nv_bfloat16) * c * ms, s) == cudaSuccess &&
+            cudaMallocAsync(&ql, sizeof(__nv_bfloat16) * c * ms, s) == cudaSuccess &&
+            cudaMallocAsync(&qn, sizeof(float) * c, s) == cudaSuccess &&
+            cudaMallocAsync(&keys, sizeof(u64) * c * p.nseg * p.KP, s) == cudaSuccess)
+            break;
+        cudaGetLastError();
+        release();
+        if (p.chunk <= TQ) return cudaErrorMemoryAllocation;
     }
-    if ((e = cudaMemsetAsync(bound, 0xFF, sizeof(uint32_t) * (size_t)nq, s)) != cudaSuccess) goto done;
+    const int nc = p.nseg * p.KP, KP = p.KP;
+    const float4* X = reinterpret_cast<const float4*>(ix->X);
     if ((e = cudaMemsetAsync(xmax, 0, sizeof(NormMax), s)) != cudaSuccess) goto done;
     k_max_norm<<<256, 256, 0, s>>>(ix->xnorm2, n, xmax);
-    k_split_bf16<<<(unsigned)((nq * 32 + 255) / 256), 256, 0, s>>>(Q, nq, m, m, ms, qh, ql, qn);
-    if ((e = cudaGetLastError()) != cudaSuccess) goto done;
-    if ((e = run_items(ix, base_of(ix), qh, ql, qn, nq, KP, nseg, CONTIGUOUS, keys, bound, xmax, s)) != cudaSuccess)
-        goto done;
-    {
-        const float4* X = reinterpret_cast<const float4*>(ix->X);
+    for (int64_t lo = 0; lo < nq && e == cudaSuccess; lo += p.chunk) {
+        const int64_t c = std::min(p.chunk, nq - lo);
+        const float* q = Q + lo * m;
+        if ((e = cudaMemsetAsync(bound, 0xFF, sizeof(uint32_t) * (size_t)c, s)) != cudaSuccess) break;
+        k_split_bf16<<<(unsigned)((c * 32 + 255) / 256), 256, 0, s>>>(q, c, m, m, ms, qh, ql, qn);
+        if ((e = cudaGetLastError()) != cudaSuccess) break;
+        if ((e = run_items(ix, base_of(ix), qh, ql, qn, c, KP, p.nseg, CONTIGUOUS, keys, bound, xmax,
+                           s)) != cudaSuccess)
+            break;
         // a query tile's lists: a few for large batches, up to one per SM for small ones
-#define FG_RERANK(W_, E_)                                                                        \
-    k_rerank<W_, E_><<<(unsigned)(W_ == 1 ? (nq + 3) / 4 : nq), W_ == 1 ? 128 : 32 * W_, 0, s>>>( \
-        X, ix->m4, Q, m, nq, keys, nc, KP, K, qn, xmax, out_ids, out_d)
+#define FG_RERANK(W_, E_)                                                                     \
+    k_rerank<W_, E_><<<(unsigned)(W_ == 1 ? (c + 3) / 4 : c), W_ == 1 ? 128 : 32 * W_, 0, s>>>( \
+        X, ix->m4, q, m, c, keys, nc, KP, K, qn, xmax, out_ids + lo * K, out_d + lo * K)
         if (nc <= 32 * 4) FG_RERANK(1, 4);
         else if (nc <= 32 * 16) FG_RERANK(1, 16);
         else if (nc <= 8 * 32 * 16) FG_RERANK(8, 16);
-        else if (nc <= 16 * 32 * 32) FG_RERANK(16, 32);
-        else e = cudaErrorInvalidValue;   // (more than 256 SMs)
+        else FG_RERANK(16, 32);   // up to MAX_KEYS
 #undef FG_RERANK
-        if (e == cudaSuccess) e = cudaGetLastError();
+        e = cudaGetLastError();
     }
 done:
-    // stream-ordered frees: the temporaries live until the kernels above finish
-    if (qh) cudaFreeAsync(qh, s);
-    if (ql) cudaFreeAsync(ql, s);
-    if (qn) cudaFreeAsync(qn, s);
-    if (bound) cudaFreeAsync(bound, s);
-    if (xmax) cudaFreeAsync(xmax, s);
-    if (keys) cudaFreeAsync(keys, s);
+    release();
     return e;
 }
 
