@@ -401,8 +401,11 @@ finger_status finger_mlp_predict(finger_index* ix, const float* feat, int64_t n,
  * as (q - x)^2 in FP32.  K <= 256.  The distance matrix runs on the tensor
  * cores (q.x from BF16 high/low split products accumulated in FP32 in tensor
  * memory, candidate lists of 32 or 64 per row and base segment, then an exact
- * FP32 re-rank); for K > 40 on bases below 4,096 rows, in stream capture, or
- * without memory for the lists, FP32 FFMA tiles give the same bits.
+ * FP32 re-rank); queries that the products' error leaves open (rows much farther
+ * from the origin than from one another) are done again with FP32 FFMA tiles.  For
+ * K > 40 on bases below 4,096 rows, in stream capture, or without memory for the
+ * lists, those tiles do all queries, with the same bits.  Rows with a NaN are no
+ * results; nor, for K <= 40, are rows at an infinite distance.
  * Asynchronous (stream-ordered temporaries; the first tensor-core call caches a
  * BF16 split of the base rows, 4 bytes per element). */
 finger_status finger_knn(finger_index* ix, const float* queries, int64_t nq, int K,

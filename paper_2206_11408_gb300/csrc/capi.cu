@@ -540,7 +540,7 @@ void finger_index_free(finger_index* ix) {
                     ix->edge_u, ix->edge_s, ix->Xh, ix->edge_q, ix->W1f, ix->W2f, ix->w3,
                     ix->b1, ix->b2, ix->work, ix->err, ix->cnt, ix->bitmap, ix->spill,
                     ix->stage_q, ix->stage_ids, ix->stage_d, ix->eig_G, ix->eig_V, ix->xs_hi,
-                    ix->xs_lo, ix->edge_h, ix->adj_t};
+                    ix->xs_lo, ix->xs_max, ix->edge_h, ix->adj_t};
     for (void* p : ptrs) cudaFree(p);
     delete ix;
 }

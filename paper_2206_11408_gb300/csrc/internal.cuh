@@ -164,6 +164,24 @@ cudaError_t launch_knn(const float4* Xb, int64_t nb, int m4, const float* Q, int
                        int64_t* out_ids, float* out_d, cudaStream_t s, bool causal = false,
                        const int32_t* only = nullptr);
 size_t knn_smem(int K);
+// the same for a few queries, the base in parts over the GPU: lists of K keys (distance
+// bits mapped to unsigned order, then the id), KNN_NO_KEY where there are fewer
+constexpr unsigned long long KNN_NO_KEY = 0xFF800000FFFFFFFFull;
+constexpr int REDO_PARTS = 64;
+// parts of the base for `count` queries: as many as the grid has blocks and the buffer
+// lists for, at most REDO_PARTS and one per tile of 128 rows
+__host__ __device__ inline int redo_parts(int count, int grid, int64_t room, int64_t nb) {
+    const int groups = (count + 31) / 32;
+    if (groups == 0) return 1;
+    int64_t p = grid / groups;
+    if (p > REDO_PARTS) p = REDO_PARTS;
+    if (p > (nb + 127) / 128) p = (nb + 127) / 128;
+    if (p > room / count) p = room / count;
+    return p < 1 ? 1 : (int)p;
+}
+cudaError_t launch_knn_parts(const float4* Xb, int64_t nb, int m4, const float* Q, int m, int64_t nq,
+                             int K, const int32_t* only, unsigned long long* parts, int64_t room,
+                             int* grid_out, cudaStream_t s);
 // tensor-core exact kNN (knn_tc.cu): launch_knn_tc for K <= knn_tc_max_k(), _big above
 int knn_tc_max_k();
 cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, int64_t* out_ids,
@@ -188,6 +206,15 @@ cudaError_t launch_to_bf16(const float* X, int64_t n, int m_pad, int m8, __nv_bf
 }  // namespace fg
 
 // The index object behind the opaque handle.
+// The base's norms as the error bounds of the tensor-core kNN need them: the largest
+// finite one, and whether some are +inf (rows with infinities, or whose norm overflows).
+// A NaN's row is nobody's neighbour, and a row of infinite norm has no finite
+// approximate distance.
+struct NormMax {
+    float finite;
+    uint32_t inf;
+};
+
 struct finger_index {
     int device = 0;
     int num_sms = 0;
@@ -197,6 +224,7 @@ struct finger_index {
     float* xnorm2 = nullptr;
     __nv_bfloat16* xs_hi = nullptr;   // BF16 high / low parts of X (tensor-core kNN), lazily
     __nv_bfloat16* xs_lo = nullptr;
+    NormMax* xs_max = nullptr;        // and what its error bounds need of the norms
     // graph
     int deg0 = 0, M = 0, maxlevel = 0, entry = 0;
     int64_t up_rows = 0;

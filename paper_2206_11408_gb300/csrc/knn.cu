@@ -11,6 +11,8 @@
 // only, and tiles above the diagonal are not computed.
 #include <float.h>
 
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace fg {
@@ -23,12 +25,17 @@ __device__ __forceinline__ bool klt(float da, int ia, float db, int ib) {
     return da < db || (da == db && ia < ib);
 }
 
+// ONLY: the queries only[1 .. only[0]] instead of all nq.  PARTS (with ONLY): the
+// base is split over blocks (redo_parts of them for a group of QB queries), and part p
+// of the i-th such query leaves its list as K keys at parts + (i P + p) K.
+template <bool ONLY, bool PARTS>
 __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_t nb, int m4,
                                             const float* __restrict__ Q, int64_t q_stride,
                                             int q_m, int64_t nq, int K, int exclude_self,
                                             int causal, const int32_t* __restrict__ remap,
                                             int64_t* out_ids, float* out_d,
-                                            const int32_t* __restrict__ only) {
+                                            const int32_t* __restrict__ only,
+                                            unsigned long long* parts, int64_t room) {
     extern __shared__ __align__(16) unsigned char sm[];
     float* Qs = reinterpret_cast<float*>(sm);          // KC x QB
     float* Xs = Qs + KC * QB;                          // KC x XB
@@ -40,13 +47,14 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
     float* thr_d = reinterpret_cast<float*>(li + QB * K);
     int* thr_i = reinterpret_cast<int*>(thr_d + QB);
     int* lsz = thr_i + QB;
-    __shared__ int64_t qid[QB];   // query of each of the block's rows (-1: none)
+    __shared__ int64_t qid_s[ONLY ? QB : 1];   // ONLY: query of each of the block's rows (-1: none)
 
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int64_t q0 = (int64_t)blockIdx.x * QB;
-    // `only`: the queries only[1 .. only[0]] instead of all nq
-    if (only) nq = only[0];
+    if (ONLY) nq = only[0];
+    const int P = PARTS ? redo_parts((int)nq, gridDim.x, room, nb) : 1;
+    const int64_t q0 = (int64_t)(blockIdx.x / P) * QB;
     if (q0 >= nq) return;
+    auto qid = [&](int i) -> int64_t { return ONLY ? qid_s[i] : q0 + i < nq ? q0 + i : -1; };
     const int tq = t >> 5;     // 0..7 -> queries tq*4 .. +4
     const int tx = t & 31;     // 0..31 -> rows tx*4 .. +4
     for (int i = t; i < QB; i += NT) {
@@ -54,17 +62,25 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
         lsz[i] = 0;
         thr_d[i] = INFINITY;
         thr_i[i] = 0x7fffffff;
-        qid[i] = q0 + i >= nq ? -1 : only ? (int64_t)only[1 + q0 + i] : q0 + i;
+        if (ONLY) qid_s[i] = q0 + i < nq ? (int64_t)only[1 + q0 + i] : -1;
     }
     __syncthreads();
     const int m = m4 * 4;
-    int64_t x_end = nb;
-    if (causal) {
-        x_end = 0;
-        for (int i = 0; i < QB; ++i) x_end = max(x_end, qid[i]);   // rows below the last query
+    int64_t x_begin = 0, x_end = nb;
+    if (causal) {   // rows below the last query
+        x_end = q0 + QB;
+        if (ONLY) {
+            x_end = 0;
+            for (int i = 0; i < QB; ++i) x_end = max(x_end, qid(i));
+        }
         x_end = min(x_end, nb);
     }
-    for (int64_t x0 = 0; x0 < x_end; x0 += XB) {
+    if (PARTS) {
+        const int64_t tiles = (nb + XB - 1) / XB, p = blockIdx.x % P;
+        x_begin = tiles * p / P * XB;
+        x_end = min(tiles * (p + 1) / P * XB, nb);
+    }
+    for (int64_t x0 = x_begin; x0 < x_end; x0 += XB) {
         float acc[4][4];
 #pragma unroll
         for (int a = 0; a < 4; ++a)
@@ -75,7 +91,7 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
             // stage Q chunk (transposed): QB x KC
             for (int i = t; i < QB * KC; i += NT) {
                 const int qq = i / KC, kk = i % KC;
-                const int64_t gq = qid[qq];
+                const int64_t gq = qid(qq);
                 const int gk = k0 + kk;
                 Qs[kk * QB + qq] = (gq >= 0 && gk < q_m) ? Q[gq * q_stride + gk] : 0.f;
             }
@@ -115,7 +131,7 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
             const int qq = tq * 4 + a;
-            const int64_t gq = qid[qq];
+            const int64_t gq = qid(qq);
             if (gq < 0) continue;
             const int64_t self = exclude_self ? (remap ? (int64_t)remap[gq] : gq) : -1;
             const float td = thr_d[qq];
@@ -185,9 +201,17 @@ __global__ void __launch_bounds__(NT) k_knn(const float4* __restrict__ X, int64_
     }
     for (int i = t; i < QB * K; i += NT) {
         const int qq = i / K, k = i % K;
-        const int64_t gq = qid[qq];
+        const int64_t gq = qid(qq);
         if (gq < 0) continue;
         const bool ok = k < lsz[qq];
+        if (PARTS) {   // (an infinite distance is no result)
+            const float d = ld[qq * K + k];
+            parts[((q0 + qq) * P + blockIdx.x % P) * K + k] =
+                ok && d < INFINITY
+                    ? (unsigned long long)(__float_as_uint(d) | 0x80000000u) << 32 | (uint32_t)li[qq * K + k]
+                    : KNN_NO_KEY;
+            continue;
+        }
         out_ids[gq * K + k] = ok ? (int64_t)li[qq * K + k] : (int64_t)-1;
         out_d[gq * K + k] = ok ? ld[qq * K + k] : INFINITY;
     }
@@ -210,12 +234,37 @@ cudaError_t launch_knn(const float4* Xb, int64_t nb, int m4, const float* Q, int
                        bool causal, const int32_t* only) {
     if (nq == 0) return cudaSuccess;
     const size_t smem = knn_smem(K);
-    cudaError_t e = cudaFuncSetAttribute(k_knn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = only ? cudaFuncSetAttribute(k_knn<true, false>,
+                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                         : cudaFuncSetAttribute(k_knn<false, false>,
+                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t grid = (nq + QB - 1) / QB;
-    k_knn<<<(unsigned)grid, NT, smem, s>>>(Xb, nb, m4, Q, q_stride, q_m, nq, K, exclude_self ? 1 : 0,
-                                           causal ? 1 : 0, remap, out_ids, out_d, only);
+    if (only)
+        k_knn<true, false><<<(unsigned)grid, NT, smem, s>>>(Xb, nb, m4, Q, q_stride, q_m, nq, K,
+                                                            exclude_self ? 1 : 0, causal ? 1 : 0, remap,
+                                                            out_ids, out_d, only, nullptr, 0);
+    else
+        k_knn<false, false><<<(unsigned)grid, NT, smem, s>>>(Xb, nb, m4, Q, q_stride, q_m, nq, K,
+                                                             exclude_self ? 1 : 0, causal ? 1 : 0, remap,
+                                                             out_ids, out_d, nullptr, nullptr, 0);
+    return cudaGetLastError();
+}
+
+// The K smallest keys of the queries only[1 .. only[0]] (at most nq; row stride m), the
+// base in parts: room = lists of K keys that fit at `parts`.  *grid_out: the grid, from
+// which k_redo_rank finds the number of parts.
+cudaError_t launch_knn_parts(const float4* Xb, int64_t nb, int m4, const float* Q, int m, int64_t nq,
+                             int K, const int32_t* only, unsigned long long* parts, int64_t room,
+                             int* grid_out, cudaStream_t s) {
+    const size_t smem = knn_smem(K);
+    cudaError_t e = cudaFuncSetAttribute(k_knn<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    const int grid = (int)std::max<int64_t>((nq + QB - 1) / QB, std::min<int64_t>(REDO_PARTS, (nb + XB - 1) / XB));
+    *grid_out = grid;
+    k_knn<true, true><<<grid, NT, smem, s>>>(Xb, nb, m4, Q, m, m, nq, K, 0, 0, nullptr, nullptr, nullptr,
+                                             only, parts, room);
     return cudaGetLastError();
 }
 

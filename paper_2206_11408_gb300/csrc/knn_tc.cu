@@ -7,9 +7,9 @@
 // the rounding of the parts are ~2^-17 of |q||x|).  Every query row keeps the
 // K' smallest approximate distances of its share of the base; a second kernel
 // takes the K' smallest of all shares, recomputes their distances exactly in
-// FP32 (sum of (q - x)^2) and returns the K best by (distance, id), so the
-// result is the exact kNN unless more than K' - K rows lie within the
-// approximation error of the K-th distance.
+// FP32 (sum of (q - x)^2) and returns the K best by (distance, id).  A query for
+// which the approximation's error leaves open whether another row is nearer is done
+// again by the FP32 kernel.
 //
 // k_knn_tc is persistent (one CTA per SM) and warp-specialised:
 //   warp 0     TMA producer: 64-column (128-byte, SWIZZLE_128B) chunks of the base
@@ -62,7 +62,7 @@ constexpr long WAIT_TRIES = 1L << 21;
 using u64 = unsigned long long;
 // candidate key: distance bits mapped to unsigned order, then the id (a kept
 // distance is finite).  NO_KEY and above: none
-constexpr u64 NO_KEY = 0xFF800000FFFFFFFFull;
+constexpr u64 NO_KEY = KNN_NO_KEY;
 
 __device__ __forceinline__ uint32_t ord_of(float d) {
     const uint32_t b = __float_as_uint(d);
@@ -81,13 +81,12 @@ __device__ __forceinline__ float split_error(float nq, float nx, int m) {
            0x1p-21f * (nq + nx);
 }
 
-// The base's norms as the error bounds need them: the largest finite one, and whether
-// some are +inf (rows with infinities, or whose norm overflows).  A NaN's row is nobody's
-// neighbour, and a row of infinite norm has no finite approximate distance.
-struct NormMax {
-    float finite;
-    uint32_t inf;
-};
+// split_error for the rows that may lie at a squared distance of at most d: their length
+// is at most |q| + sqrt(d) (2^-7 for the roundings), whatever other rows there are
+__device__ __forceinline__ float near_error(const NormMax& x, float nq, float d, int m) {
+    const float r = sqrtf(nq) + sqrtf(d);
+    return split_error(nq, fminf(x.finite, (1.f + 0x1p-7f) * r * r), m);
+}
 
 // Whether a row of infinite norm may be nearer than kth: its length is at least
 // 1.8e19 (the root of the largest float, less 2 %), so |q - x| >= 1.8e19 - |q|.
@@ -543,7 +542,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             if (a.bound && qi < a.nq) bound = min(bound, *(volatile uint32_t*)(a.bound + qi));
             float cap = bound < 0xFF800000u ? dist_of((u64)(bound + 1u) << 32) : INFINITY;
             // (a kNN launch keeps what the approximation may have misplaced, see k_rerank)
-            if (a.bound) cap += 2.f * split_error(qn, a.xmax->finite, a.m);
+            // for the rows at the bound's distance or nearer, whose exact one is at most
+            // 1.001 (bound + 0.001 |q|^2): the error is below 2^-11 of |q|^2 + |x|^2
+            if (a.bound)
+                cap += 2.f * near_error(*a.xmax, qn, 1.001f * (fmaxf(cap, 0.f) + 0.001f * qn), a.m);
             float thr = qi < a.nq ? cap : -INFINITY;
             int cnt = 0;                                    // pending candidates of the row
             top.clear();
@@ -713,26 +715,10 @@ __device__ __forceinline__ void warp_smallest(u64 (&k)[E], int R, u64* out, int 
     __syncwarp();
 }
 
-// Final step of a kNN launch: the KP smallest approximate keys of a query's lists,
-// their exact FP32 distances, the K best by (distance, id).  Where the approximation's
-// error reaches from the KP-th approximate distance to the K-th exact one (rows far
-// from the origin, many equal distances), the lists' other keys get their exact
-// distances too.  W warps per query (E keys per lane: 32 E W >= the query's keys); with
-// W = 1 four queries per block.
+// The KP smallest of the nc keys kr[], ascending, into sel[].  W warps (this one is wq;
+// part: W KP keys of shared memory), E keys per lane: nc <= 32 E W.
 template <int W, int E>
-__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
-    k_rerank(const float4* __restrict__ X, int m4, const float* __restrict__ Q, int m, int64_t nq,
-             const u64* __restrict__ keys, int nc, int KP, int K, const float* __restrict__ qn,
-             const NormMax* __restrict__ xmax, int64_t* out_ids, float* out_d) {
-    constexpr int QPB = W == 1 ? 4 : 1;
-    __shared__ u64 sel_s[QPB][64];
-    __shared__ u64 part_s[W == 1 ? 1 : W * 64];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int64_t q = W == 1 ? (int64_t)blockIdx.x * 4 + wib : (int64_t)blockIdx.x;
-    const int wq = W == 1 ? 0 : wib;
-    if (q >= nq) return;
-    u64* sel = sel_s[W == 1 ? wib : 0];
-    const u64* kr = keys + (size_t)q * nc;
+__device__ __forceinline__ void pick(const u64* kr, int nc, int KP, u64* sel, u64* part, int wq, int lane) {
     u64 k[E];
 #pragma unroll
     for (int j = 0; j < E; ++j) {
@@ -742,22 +728,24 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
     if constexpr (W == 1) {
         warp_smallest<E>(k, KP, sel, lane);
     } else {
-        warp_smallest<E>(k, KP, part_s + wq * KP, lane);
+        warp_smallest<E>(k, KP, part + wq * KP, lane);
         __syncthreads();
         if (wq == 0) {
             u64 k2[2 * W];
 #pragma unroll
             for (int j = 0; j < 2 * W; ++j)
-                k2[j] = 32 * j + lane < W * KP ? part_s[32 * j + lane] : NO_KEY;
+                k2[j] = 32 * j + lane < W * KP ? part[32 * j + lane] : NO_KEY;
             warp_smallest<2 * W>(k2, KP, sel, lane);
         }
         __syncthreads();
     }
-    const u64 last = sel[KP - 1];   // the KP-th approximate key
-    if constexpr (W == 1) __syncwarp();
-    else __syncthreads();
-    // exact distances, four rows in flight per warp; each key gets its exact distance
-    const float* qr = Q + (size_t)q * m;
+}
+
+// the distance of each key of sel[] gives way to its row's exact one, sum of (q - x)^2 in
+// FP32; four rows in flight per warp
+template <int W>
+__device__ __forceinline__ void exact_keys(const float4* __restrict__ X, int m4, const float* qr, int m,
+                                           u64* sel, int KP, int wq, int lane) {
     constexpr int U = 4;
     for (int i = wq * U; i < KP; i += W * U) {
         uint32_t id[U];
@@ -798,52 +786,22 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
     }
     if constexpr (W == 1) __syncwarp();
     else __syncthreads();
-    if (wq != 0) return;
-    if (last < NO_KEY) {
-        // the K-th exact key: the one that K - 1 others precede
-        u64 kth = ~0ull;
-        for (int i = lane; i < KP; i += 32) {
-            int rank = 0;
-            for (int j = 0; j < KP; ++j) rank += sel[j] < sel[i];
-            if (rank == K - 1) kth = sel[i];
-        }
-        kth = warp_min(kth);
-        const float err = split_error(qn[q], xmax->finite, m);
-        if (!(dist_of(kth) < dist_of(last) - err)) {
-            const float lim = dist_of(kth) + err;   // above it no key can be nearer
-            for (int c0 = 0; c0 < nc; c0 += 32) {
-                const u64 kc = c0 + lane < nc ? kr[c0 + lane] : NO_KEY;
-                unsigned more = __ballot_sync(
-                    0xffffffffu, kc < NO_KEY && kc > last && !(dist_of(kc) > lim));
-                while (more) {
-                    const uint32_t id = __shfl_sync(0xffffffffu, (uint32_t)kc, __ffs(more) - 1);
-                    more &= more - 1;
-                    float acc = 0.f;
-                    for (int c = lane; c < m4; c += 32) {
-                        const float4 x = __ldg(X + (size_t)id * m4 + c);
-                        const int e = 4 * c;
-                        float dlt;
-                        dlt = (e < m ? qr[e] : 0.f) - x.x; acc = fmaf(dlt, dlt, acc);
-                        dlt = (e + 1 < m ? qr[e + 1] : 0.f) - x.y; acc = fmaf(dlt, dlt, acc);
-                        dlt = (e + 2 < m ? qr[e + 2] : 0.f) - x.z; acc = fmaf(dlt, dlt, acc);
-                        dlt = (e + 3 < m ? qr[e + 3] : 0.f) - x.w; acc = fmaf(dlt, dlt, acc);
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                    // in the place of the largest kept key, if it is smaller
-                    const u64 key = (u64)ord_of(acc) << 32 | id;
-                    const u64 a = sel[lane], b = KP > 32 ? sel[lane + 32] : 0ull;
-                    const u64 top = ~warp_min(~(a > b ? a : b));
-                    __syncwarp();
-                    if (key < top) {
-                        if (a == top) sel[lane] = key;
-                        else if (KP > 32 && b == top) sel[lane + 32] = key;
-                    }
-                    __syncwarp();
-                }
-            }
-        }
+}
+
+// the K-th smallest key of sel[0..KP) (one warp); NO_KEY or above if there are fewer
+__device__ __forceinline__ u64 kth_key(const u64* sel, int KP, int K, int lane) {
+    u64 kth = ~0ull;
+    for (int i = lane; i < KP; i += 32) {
+        int rank = 0;
+        for (int j = 0; j < KP; ++j) rank += sel[j] < sel[i];
+        if (rank == K - 1) kth = sel[i];
     }
+    return warp_min(kth);
+}
+
+// the K smallest keys of sel[0..KP) in order (one warp)
+__device__ __forceinline__ void put_best(const u64* sel, int KP, int K, int64_t* out_ids, float* out_d,
+                                         int lane) {
     for (int i = lane; i < KP; i += 32) {
         const u64 ki = sel[i];
         int rank = 0;
@@ -853,9 +811,118 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
         }
         if (rank < K) {
             const bool ok = (int32_t)(uint32_t)ki >= 0;
-            out_ids[(size_t)q * K + rank] = ok ? (int64_t)(uint32_t)ki : (int64_t)-1;
-            out_d[(size_t)q * K + rank] = ok ? dist_of(ki) : INFINITY;
+            out_ids[rank] = ok ? (int64_t)(uint32_t)ki : (int64_t)-1;
+            out_d[rank] = ok ? dist_of(ki) : INFINITY;
         }
+    }
+}
+
+// Final step of a kNN launch: the KP smallest approximate keys of a query's lists,
+// their exact FP32 distances, the K best by (distance, id).  A row outside the lists has
+// an approximate distance of at least the KP-th, so an exact one of at least that less
+// the approximation's error: the K-th exact distance lies below, and the result stands.
+// Where it does not (rows far from the origin, many equal distances), the lists' other
+// keys get their exact distances too, and the nearest row that a full list may have
+// dropped takes the place of the KP-th.  A query that still does not stand, or whose
+// approximate distances may not be finite, goes on `redo` (count in redo[0]) for
+// launch_knn_parts and k_redo_rank.  W warps per query (E keys per lane: 32 E W >= the
+// query's keys); with W = 1 four queries per block.
+template <int W, int E>
+__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
+    k_rerank(const float4* __restrict__ X, int m4, const float* __restrict__ Q, int m, int64_t nq,
+             const u64* __restrict__ keys, int nc, int KP, int K, const float* __restrict__ qn,
+             const NormMax* __restrict__ xmax, int64_t* out_ids, float* out_d, int32_t* redo) {
+    constexpr int QPB = W == 1 ? 4 : 1;
+    __shared__ u64 sel_s[QPB][64];
+    __shared__ u64 part_s[W == 1 ? 1 : W * 64];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int64_t q = W == 1 ? (int64_t)blockIdx.x * 4 + wib : (int64_t)blockIdx.x;
+    const int wq = W == 1 ? 0 : wib;
+    if (q >= nq) return;
+    u64* sel = sel_s[W == 1 ? wib : 0];
+    const u64* kr = keys + (size_t)q * nc;
+    const float* qr = Q + (size_t)q * m;
+    pick<W, E>(kr, nc, KP, sel, part_s, wq, lane);
+    const u64 last = sel[KP - 1];   // the KP-th approximate key
+    if constexpr (W == 1) __syncwarp();
+    else __syncthreads();
+    exact_keys<W>(X, m4, qr, m, sel, KP, wq, lane);
+    if (wq != 0) return;
+    const float nrm = qn[q];
+    const u64 k0 = kth_key(sel, KP, K, lane);
+    const float kth = k0 < NO_KEY ? dist_of(k0) : INFINITY;
+    const float err = near_error(*xmax, nrm, kth, m);
+    bool stands = err < INFINITY && !inf_rows_reach(*xmax, nrm, kth);
+    if (!stands && !(nrm < INFINITY)) {   // a query that is not finite has no neighbours
+        bool bad = false;
+        for (int i = lane; i < m; i += 32) bad |= !(fabsf(qr[i]) < INFINITY);
+        stands = __any_sync(0xffffffffu, bad);
+    }
+    if (stands && last < NO_KEY && !(kth < dist_of(last) - err)) {
+        const float lim = kth + err;   // above it no key can be nearer
+        uint32_t most = 0;             // the largest distance of the list so far
+        float edge = INFINITY;         // the smallest of the full lists' largest
+        for (int c0 = 0; c0 < nc; c0 += 32) {
+            const u64 kc = kr[c0 + lane];   // (nc and KP: multiples of 32)
+            most = max(most, __reduce_max_sync(0xffffffffu, (uint32_t)(kc >> 32)));
+            if ((c0 + 32) % KP == 0) {
+                if (most < (uint32_t)(NO_KEY >> 32)) edge = fminf(edge, dist_of((u64)most << 32));
+                most = 0;
+            }
+            unsigned more = __ballot_sync(0xffffffffu,
+                                          kc < NO_KEY && kc > last && !(dist_of(kc) > lim));
+            while (more) {
+                const uint32_t id = __shfl_sync(0xffffffffu, (uint32_t)kc, __ffs(more) - 1);
+                more &= more - 1;
+                float acc = 0.f;
+                for (int c = lane; c < m4; c += 32) {
+                    const float4 x = __ldg(X + (size_t)id * m4 + c);
+                    const int e = 4 * c;
+                    float dlt;
+                    dlt = (e < m ? qr[e] : 0.f) - x.x; acc = fmaf(dlt, dlt, acc);
+                    dlt = (e + 1 < m ? qr[e + 1] : 0.f) - x.y; acc = fmaf(dlt, dlt, acc);
+                    dlt = (e + 2 < m ? qr[e + 2] : 0.f) - x.z; acc = fmaf(dlt, dlt, acc);
+                    dlt = (e + 3 < m ? qr[e + 3] : 0.f) - x.w; acc = fmaf(dlt, dlt, acc);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                // in the place of the largest kept key, if it is smaller
+                const u64 key = (u64)ord_of(acc) << 32 | id;
+                const u64 a = sel[lane], b = KP > 32 ? sel[lane + 32] : 0ull;
+                const u64 top = ~warp_min(~(a > b ? a : b));
+                __syncwarp();
+                if (key < top) {
+                    if (a == top) sel[lane] = key;
+                    else if (KP > 32 && b == top) sel[lane + 32] = key;
+                }
+                __syncwarp();
+            }
+        }
+        stands = dist_of(kth_key(sel, KP, K, lane)) < edge - err;
+    }
+    if (stands) put_best(sel, KP, K, out_ids + (size_t)q * K, out_d + (size_t)q * K, lane);
+    else if (lane == 0) redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
+}
+
+// The queries on `redo` from the FP32 kernel's lists (launch_knn_parts with this grid
+// and room): KP smallest keys of all parts, then as k_rerank, whose sums they get.  10,000
+// queries x 1M x 128, K = 10: 6.33 ms with none, 8.07 with one, 227 with all of them (the
+// rows 10,000 from the origin in every dimension; 1,000 needs none, 7.3 ms).
+__global__ void __launch_bounds__(256)
+    k_redo_rank(const float4* __restrict__ X, int64_t n, int m4, const float* __restrict__ Q, int m,
+                const u64* __restrict__ parts, int grid, int64_t room, int KP, int K,
+                const int32_t* __restrict__ redo, int64_t* out_ids, float* out_d) {
+    constexpr int W = 8, E = 16;
+    static_assert(32 * E * W >= 64 * REDO_PARTS, "the keys of a query's parts");
+    __shared__ u64 sel[64], part_s[W * 64];
+    const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+    const int count = redo[0], nc = redo_parts(count, grid, room, n) * KP;
+    for (int i = blockIdx.x; i < count; i += gridDim.x) {
+        const int64_t q = redo[1 + i];
+        pick<W, E>(parts + (size_t)i * nc, nc, KP, sel, part_s, wq, lane);
+        exact_keys<W>(X, m4, Q + (size_t)q * m, m, sel, KP, wq, lane);
+        if (wq == 0) put_best(sel, KP, K, out_ids + (size_t)q * K, out_d + (size_t)q * K, lane);
+        __syncthreads();
     }
 }
 
@@ -936,7 +1003,7 @@ __global__ void __launch_bounds__(256)
         for (int j = 0; j < R; ++j) rank += ex[j] < k || (ex[j] == k && j < i);
         if (rank == K - 1) {
             const float kth = dist_of(k);
-            if (!(kth < dist_of(last) - split_error(qn[q], xmax->finite, q_m)) ||
+            if (!(kth < dist_of(last) - near_error(*xmax, qn[q], kth, q_m)) ||
                 inf_rows_reach(*xmax, qn[q], kth))
                 redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
         }
@@ -1074,42 +1141,63 @@ bool capturing(cudaStream_t s) {
     return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
 }
 
-// BF16 split of the base rows, made once per index
+cudaError_t max_norm(const float* xn, int64_t n, NormMax* out, cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(NormMax), s);
+    if (e != cudaSuccess) return e;
+    k_max_norm<<<256, 256, 0, s>>>(xn, n, out);
+    return cudaGetLastError();
+}
+
+// BF16 split and largest norm of the base rows, made once per index
 cudaError_t ensure_split(finger_index* ix, cudaStream_t s) {
     if (ix->xs_hi) return cudaSuccess;
     const int m = ix->m, ms = (m + 7) & ~7;
     const int64_t n = ix->n;
-    if (cudaMalloc(&ix->xs_hi, sizeof(__nv_bfloat16) * (size_t)n * ms) != cudaSuccess ||
-        cudaMalloc(&ix->xs_lo, sizeof(__nv_bfloat16) * (size_t)n * ms) != cudaSuccess) {
-        cudaFree(ix->xs_hi);
-        ix->xs_hi = nullptr;
-        ix->xs_lo = nullptr;
-        cudaGetLastError();
-        return cudaErrorMemoryAllocation;
+    __nv_bfloat16 *hi = nullptr, *lo = nullptr;
+    NormMax* mx = nullptr;
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (cudaMalloc(&hi, sizeof(__nv_bfloat16) * (size_t)n * ms) == cudaSuccess &&
+        cudaMalloc(&lo, sizeof(__nv_bfloat16) * (size_t)n * ms) == cudaSuccess &&
+        cudaMalloc(&mx, sizeof(NormMax)) == cudaSuccess) {
+        k_split_bf16<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(ix->X, n, m, ix->m_pad, ms, hi, lo,
+                                                                      nullptr);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = max_norm(ix->xnorm2, n, mx, s);
+        // done before a call on another stream finds it there
+        if (e == cudaSuccess && !capturing(s)) e = cudaStreamSynchronize(s);
     }
-    k_split_bf16<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(ix->X, n, m, ix->m_pad, ms,
-                                                                  ix->xs_hi, ix->xs_lo, nullptr);
-    const cudaError_t e = cudaGetLastError();
-    // done before a call on another stream finds it there
-    return e != cudaSuccess || capturing(s) ? e : cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+        cudaFree(hi);
+        cudaFree(lo);
+        cudaFree(mx);
+        cudaGetLastError();
+        return e;
+    }
+    ix->xs_hi = hi;
+    ix->xs_lo = lo;
+    ix->xs_max = mx;
+    return cudaSuccess;
 }
 
 // what a launch needs of the base rows (BF16 parts with row stride m rounded to 8)
 struct TcBase {
     const __nv_bfloat16 *hi, *lo;
     const float* xn;
+    const NormMax* xmax;
     int64_t n;
     int m;
 };
 
-TcBase base_of(const finger_index* ix) { return {ix->xs_hi, ix->xs_lo, ix->xnorm2, ix->n, ix->m}; }
+TcBase base_of(const finger_index* ix) {
+    return {ix->xs_hi, ix->xs_lo, ix->xnorm2, ix->xs_max, ix->n, ix->m};
+}
 
 enum TcOrder { CONTIGUOUS, INTERLEAVED, CAUSAL };
 
 // one launch of k_knn_tc over nq query rows (BF16 parts qh/ql) against the base
 cudaError_t run_items(finger_index* ix, const TcBase& x, const __nv_bfloat16* qh,
                       const __nv_bfloat16* ql, const float* qn, int64_t nq, int KP, int nseg,
-                      TcOrder order, u64* keys, uint32_t* bound, const NormMax* xmax, cudaStream_t s,
+                      TcOrder order, u64* keys, uint32_t* bound, cudaStream_t s,
                       int want = 0) {
     const int ms = (x.m + 7) & ~7;
     CUtensorMap maps[4];
@@ -1132,7 +1220,7 @@ cudaError_t run_items(finger_index* ix, const TcBase& x, const __nv_bfloat16* qh
     a.xn = x.xn;
     a.keys = keys;
     a.bound = bound;
-    a.xmax = xmax;
+    a.xmax = x.xmax;
     a.m = x.m;
     a.err = ix->err;
     // want > 0: the smallest `want` keys of a causal launch's lists are used.  With query
@@ -1211,66 +1299,62 @@ cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, i
     const int64_t n = ix->n;
     cudaError_t e = ensure_split(ix, s);
     if (e != cudaSuccess) return e;
-    __nv_bfloat16 *qh = nullptr, *ql = nullptr;
-    float* qn = nullptr;
-    u64* keys = nullptr;
-    uint32_t* bound = nullptr;
-    NormMax* xmax = nullptr;
-    // stream-ordered frees: the temporaries live until the kernels below finish
-    auto release = [&]() {
-        if (qh) cudaFreeAsync(qh, s);
-        if (ql) cudaFreeAsync(ql, s);
-        if (qn) cudaFreeAsync(qn, s);
-        if (bound) cudaFreeAsync(bound, s);
-        if (xmax) cudaFreeAsync(xmax, s);
-        if (keys) cudaFreeAsync(keys, s);
-        qh = ql = nullptr;
-        qn = nullptr;
-        bound = nullptr;
-        xmax = nullptr;
-        keys = nullptr;
-    };
+    // one stream-ordered allocation for all temporaries (a pool that keeps nothing between
+    // calls maps each of them anew)
+    unsigned char* tmp = nullptr;
     KnnPlan p;
+    size_t at[6];
     for (int64_t most = nq;; most = p.chunk / 2) {   // fewer queries per pass where memory is short
         p = knn_plan(n, m, nq, K, ix->num_sms, most);
         const size_t c = (size_t)p.chunk;
-        if (cudaMallocAsync(&bound, sizeof(uint32_t) * c, s) == cudaSuccess &&
-            cudaMallocAsync(&xmax, sizeof(NormMax), s) == cudaSuccess &&
-            cudaMallocAsync(&qh, sizeof(__nv_bfloat16) * c * ms, s) == cudaSuccess &&
-            cudaMallocAsync(&ql, sizeof(__nv_bfloat16) * c * ms, s) == cudaSuccess &&
-            cudaMallocAsync(&qn, sizeof(float) * c, s) == cudaSuccess &&
-            cudaMallocAsync(&keys, sizeof(u64) * c * p.nseg * p.KP, s) == cudaSuccess)
-            break;
+        const size_t bytes[6] = {8 * c * p.nseg * p.KP, 4 * c, 2 * c * ms, 2 * c * ms, 4 * c, 4 * (c + 1)};
+        size_t total = 0;
+        for (int i = 0; i < 6; ++i) {
+            at[i] = total;
+            total += (bytes[i] + 255) & ~size_t(255);
+        }
+        if (cudaMallocAsync(&tmp, total, s) == cudaSuccess) break;
         cudaGetLastError();
-        release();
         if (p.chunk <= TQ) return cudaErrorMemoryAllocation;
     }
+    u64* keys = reinterpret_cast<u64*>(tmp + at[0]);
+    uint32_t* bound = reinterpret_cast<uint32_t*>(tmp + at[1]);
+    __nv_bfloat16* qh = reinterpret_cast<__nv_bfloat16*>(tmp + at[2]);
+    __nv_bfloat16* ql = reinterpret_cast<__nv_bfloat16*>(tmp + at[3]);
+    float* qn = reinterpret_cast<float*>(tmp + at[4]);
+    int32_t* redo = reinterpret_cast<int32_t*>(tmp + at[5]);
     const int nc = p.nseg * p.KP, KP = p.KP;
     const float4* X = reinterpret_cast<const float4*>(ix->X);
-    if ((e = cudaMemsetAsync(xmax, 0, sizeof(NormMax), s)) != cudaSuccess) goto done;
-    k_max_norm<<<256, 256, 0, s>>>(ix->xnorm2, n, xmax);
     for (int64_t lo = 0; lo < nq && e == cudaSuccess; lo += p.chunk) {
         const int64_t c = std::min(p.chunk, nq - lo);
         const float* q = Q + lo * m;
+        if ((e = cudaMemsetAsync(redo, 0, sizeof(int32_t), s)) != cudaSuccess) break;
         if ((e = cudaMemsetAsync(bound, 0xFF, sizeof(uint32_t) * (size_t)c, s)) != cudaSuccess) break;
         k_split_bf16<<<(unsigned)((c * 32 + 255) / 256), 256, 0, s>>>(q, c, m, m, ms, qh, ql, qn);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
-        if ((e = run_items(ix, base_of(ix), qh, ql, qn, c, KP, p.nseg, CONTIGUOUS, keys, bound, xmax,
-                           s)) != cudaSuccess)
+        if ((e = run_items(ix, base_of(ix), qh, ql, qn, c, KP, p.nseg, CONTIGUOUS, keys, bound, s)) !=
+            cudaSuccess)
             break;
         // a query tile's lists: a few for large batches, up to one per SM for small ones
 #define FG_RERANK(W_, E_)                                                                     \
     k_rerank<W_, E_><<<(unsigned)(W_ == 1 ? (c + 3) / 4 : c), W_ == 1 ? 128 : 32 * W_, 0, s>>>( \
-        X, ix->m4, q, m, c, keys, nc, KP, K, qn, xmax, out_ids + lo * K, out_d + lo * K)
+        X, ix->m4, q, m, c, keys, nc, KP, K, qn, ix->xs_max, out_ids + lo * K, out_d + lo * K, redo)
         if (nc <= 32 * 4) FG_RERANK(1, 4);
         else if (nc <= 32 * 16) FG_RERANK(1, 16);
         else if (nc <= 8 * 32 * 16) FG_RERANK(8, 16);
         else FG_RERANK(16, 32);   // up to MAX_KEYS
 #undef FG_RERANK
+        if ((e = cudaGetLastError()) != cudaSuccess) break;
+        // the lists are done with: their buffer takes those of the queries on redo
+        const int64_t room = p.chunk * p.nseg;
+        int grid = 0;
+        if ((e = launch_knn_parts(X, n, ix->m4, q, m, c, KP, redo, keys, room, &grid, s)) != cudaSuccess)
+            break;
+        k_redo_rank<<<(unsigned)std::min<int64_t>(c, 2 * ix->num_sms), 256, 0, s>>>(
+            X, n, ix->m4, q, m, keys, grid, room, KP, K, redo, out_ids + lo * K, out_d + lo * K);
         e = cudaGetLastError();
     }
-done:
-    release();
+    cudaFreeAsync(tmp, s);   // in stream order: when the kernels above are done
     return e;
 }
 
@@ -1295,7 +1379,7 @@ cudaError_t launch_knn_tc_causal(finger_index* ix, int K, int64_t* out_ids, floa
         goto done;
     }
     if ((e = run_items(ix, base_of(ix), ix->xs_hi, ix->xs_lo, ix->xnorm2, n, KP, NSEG, CAUSAL, keys,
-                       nullptr, nullptr, s, K)) != cudaSuccess)
+                       nullptr, s, K)) != cudaSuccess)
         goto done;
     k_merge_topk<<<(unsigned)((n + 3) / 4), 128, 0, s>>>(keys, n, K, out_ids, out_d);
     e = cudaGetLastError();
@@ -1344,13 +1428,11 @@ cudaError_t knn_big(finger_index* ix, const TcBase& x, const float4* Xb, int m4,
     float* qn = nullptr;
     u64* keys = nullptr;
     int32_t* redo = nullptr;
-    NormMax* xmax = nullptr;
     cudaError_t e = cudaSuccess;
     if ((!causal && (cudaMallocAsync(&qh, 2 * (size_t)chunk * ms, s) != cudaSuccess ||
                      cudaMallocAsync(&ql, 2 * (size_t)chunk * ms, s) != cudaSuccess ||
                      cudaMallocAsync(&qn, sizeof(float) * (size_t)chunk, s) != cudaSuccess)) ||
         cudaMallocAsync(&keys, sizeof(u64) * (size_t)chunk * nseg * 64, s) != cudaSuccess ||
-        cudaMallocAsync(&xmax, sizeof(NormMax), s) != cudaSuccess ||
         cudaMallocAsync(&redo, sizeof(int32_t) * (size_t)(chunk + 1), s) != cudaSuccess ||
         cudaFuncSetAttribute(k_rerank_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess) {
@@ -1358,8 +1440,6 @@ cudaError_t knn_big(finger_index* ix, const TcBase& x, const float4* Xb, int m4,
         e = launch_knn(Xb, x.n, m4, Q, q_stride, q_m, nq, K, causal, remap, out_ids, out_d, s, causal);
         goto done;
     }
-    if ((e = cudaMemsetAsync(xmax, 0, sizeof(NormMax), s)) != cudaSuccess) goto done;
-    k_max_norm<<<256, 256, 0, s>>>(x.xn, x.n, xmax);
     for (int64_t lo = 0; lo < nq && e == cudaSuccess; lo += chunk) {
         const int64_t c = std::min(chunk, nq - lo);
         const float* q = Q + lo * q_stride;
@@ -1369,10 +1449,10 @@ cudaError_t knn_big(finger_index* ix, const TcBase& x, const float4* Xb, int m4,
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         if ((e = cudaMemsetAsync(redo, 0, sizeof(int32_t), s)) != cudaSuccess) break;
         e = run_items(ix, x, causal ? x.hi : qh, causal ? x.lo : ql, causal ? x.xn : qn, c, 64, nseg,
-                      causal ? CAUSAL : INTERLEAVED, keys, nullptr, nullptr, s);
+                      causal ? CAUSAL : INTERLEAVED, keys, nullptr, s);
         if (e != cudaSuccess) break;
         k_rerank_big<<<(unsigned)c, 256, smem, s>>>(Xb, m4, q, q_stride, q_m, keys, nseg, np, R, K,
-                                                    remap, causal ? x.xn : qn, xmax, out_ids + lo * K,
+                                                    remap, causal ? x.xn : qn, x.xmax, out_ids + lo * K,
                                                     out_d + lo * K, redo);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         e = launch_knn(Xb, x.n, m4, q, q_stride, q_m, c, K, causal, remap, out_ids + lo * K,
@@ -1383,7 +1463,6 @@ done:
     if (ql) cudaFreeAsync(ql, s);
     if (qn) cudaFreeAsync(qn, s);
     if (keys) cudaFreeAsync(keys, s);
-    if (xmax) cudaFreeAsync(xmax, s);
     if (redo) cudaFreeAsync(redo, s);
     return e;
 }
@@ -1414,10 +1493,12 @@ cudaError_t launch_knn_layer(finger_index* ix, const float4* X, int64_t cnt, int
     const int m = ix->m, ms = (m + 7) & ~7;
     __nv_bfloat16 *hi = nullptr, *lo = nullptr;
     float* xn = nullptr;
+    NormMax* xmax = nullptr;
     cudaError_t e;
     if (cnt < BIG_MIN_ROWS || K <= 40 ||
         cudaMallocAsync(&hi, 2 * (size_t)cnt * ms, s) != cudaSuccess ||
         cudaMallocAsync(&lo, 2 * (size_t)cnt * ms, s) != cudaSuccess ||
+        cudaMallocAsync(&xmax, sizeof(NormMax), s) != cudaSuccess ||
         cudaMallocAsync(&xn, sizeof(float) * (size_t)cnt, s) != cudaSuccess) {
         cudaGetLastError();
         e = launch_knn(X, cnt, ix->m4, Xf, ix->m_pad, ix->m_pad, cnt, K, true, remap, out_ids, out_d, s,
@@ -1426,13 +1507,15 @@ cudaError_t launch_knn_layer(finger_index* ix, const float4* X, int64_t cnt, int
         k_split_bf16<<<(unsigned)((cnt * 32 + 255) / 256), 256, 0, s>>>(Xf, cnt, m, ix->m_pad, ms, hi,
                                                                         lo, xn);
         e = cudaGetLastError();
+        if (e == cudaSuccess) e = max_norm(xn, cnt, xmax, s);
         if (e == cudaSuccess)
-            e = knn_big(ix, {hi, lo, xn, cnt, m}, X, ix->m4, Xf, ix->m_pad, ix->m_pad, cnt, K, remap,
+            e = knn_big(ix, {hi, lo, xn, xmax, cnt, m}, X, ix->m4, Xf, ix->m_pad, ix->m_pad, cnt, K, remap,
                         out_ids, out_d, true, s);
     }
     if (hi) cudaFreeAsync(hi, s);
     if (lo) cudaFreeAsync(lo, s);
     if (xn) cudaFreeAsync(xn, s);
+    if (xmax) cudaFreeAsync(xmax, s);
     return e;
 }
 
