@@ -4,7 +4,7 @@
 // - 2 q.x.  q.x runs on tcgen05.mma (kind::f16, BF16 operands, FP32
 // accumulators in tensor memory) with each FP32 operand split into a BF16 high
 // part and a BF16 low part: q.x ~ qh.xh + qh.xl + ql.xh (the dropped ql.xl and
-// the rounding of the parts are ~2^-17 of |q||x|).  Every query row keeps the
+// the rounding of the parts are at most 2^-15 of |q||x|).  Every query row keeps the
 // K' smallest approximate distances of its share of the base; a second kernel
 // takes the K' smallest of all shares, recomputes their distances exactly in
 // FP32 (sum of (q - x)^2) and returns the K best by (distance, id).  A query for
@@ -73,12 +73,29 @@ __device__ __forceinline__ float dist_of(u64 k) {
     return __uint_as_float(o ^ (o & 0x80000000u ? 0x80000000u : 0xFFFFFFFFu));
 }
 
-// Bound on |approximate - exact| squared distance for norms nq and nx and m dimensions:
-// 2 (3 2^-18 + 3 ceil(m / 16) 2^-22) |q| |x| (the dropped parts' products, and an FP32
-// rounding, taken four times over, for each product added) and 2^-21 of the norms' sum
+// Bound on |approximate - true| squared distance for norms nq and nx and m dimensions
+// (u = 2^-24, an FP32 rounding):
+//   2 |q| |x| (2^-15 + 3 ceil(m / 16) 4 u): a low part is at most 2^-8 of its value (half a
+//     unit of BF16's 8 bits) and what both parts leave out 2^-17, so ql.xl and the two
+//     remainders' products make 2^-15 |q| |x| (Cauchy-Schwarz); and 4 u for each product added
+//     in tensor memory, whose additions are not IEEE ones (an assumption: the largest error
+//     found, over 48 distributions of m = 8 to 1024, was 0.74 of this term)
+//   (ceil(m / 32) + 12) u (|q|^2 + |x|^2): the norms' sums (m / 32 + 4 per lane, 5 between
+//     lanes) and the two roundings that put the distance together
+// +inf where a distance could overflow.
 __device__ __forceinline__ float split_error(float nq, float nx, int m) {
-    return 2.f * (3.f * 0x1p-18f + 3.f * ((m + 15) / 16) * 0x1p-22f) * sqrtf(nq) * sqrtf(nx) +
-           0x1p-21f * (nq + nx);
+    return 2.f * (0x1p-15f + 3.f * ((m + 15) / 16) * 0x1p-22f) * sqrtf(nq) * sqrtf(nx) +
+           ((m + 31) / 32 + 12) * 0x1p-26f * (4.f * (nq + nx));
+}
+
+// Bound on the relative error of an exact distance, the FP32 sum of (q - x)^2 in any
+// order: m additions, a subtraction's error twice, a product's
+__device__ __forceinline__ float sum_error(int m) { return (m + 8) * 0x1p-24f; }
+
+// Whether every row whose approximate distance is v or more, with error err, has an exact
+// one above d
+__device__ __forceinline__ bool all_beyond(float v, float err, float d, int m) {
+    return d < (v - err) * (1.f - sum_error(m));
 }
 
 // split_error for the rows that may lie at a squared distance of at most d: their length
@@ -544,8 +561,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             // (a kNN launch keeps what the approximation may have misplaced, see k_rerank)
             // for the rows at the bound's distance or nearer, whose exact one is at most
             // 1.001 (bound + 0.001 |q|^2): the error is below 2^-11 of |q|^2 + |x|^2
-            if (a.bound)
-                cap += 2.f * near_error(*a.xmax, qn, 1.001f * (fmaxf(cap, 0.f) + 0.001f * qn), a.m);
+            if (a.bound) {
+                const float err = near_error(*a.xmax, qn, 1.001f * (fmaxf(cap, 0.f) + 0.001f * qn), a.m);
+                cap = (cap + 2.f * err) * (1.f + 4.f * sum_error(a.m));
+            }
             float thr = qi < a.nq ? cap : -INFINITY;
             int cnt = 0;                                    // pending candidates of the row
             top.clear();
@@ -858,8 +877,8 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
         for (int i = lane; i < m; i += 32) bad |= !(fabsf(qr[i]) < INFINITY);
         stands = __any_sync(0xffffffffu, bad);
     }
-    if (stands && last < NO_KEY && !(kth < dist_of(last) - err)) {
-        const float lim = kth + err;   // above it no key can be nearer
+    if (stands && last < NO_KEY && !all_beyond(dist_of(last), err, kth, m)) {
+        const float lim = kth * (1.f + 2.f * sum_error(m)) + err;   // above it no key can be nearer
         uint32_t most = 0;             // the largest distance of the list so far
         float edge = INFINITY;         // the smallest of the full lists' largest
         for (int c0 = 0; c0 < nc; c0 += 32) {
@@ -898,7 +917,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
                 __syncwarp();
             }
         }
-        stands = dist_of(kth_key(sel, KP, K, lane)) < edge - err;
+        stands = all_beyond(edge, err, dist_of(kth_key(sel, KP, K, lane)), m);
     }
     if (stands) put_best(sel, KP, K, out_ids + (size_t)q * K, out_d + (size_t)q * K, lane);
     else if (lane == 0) redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
@@ -930,10 +949,10 @@ __global__ void __launch_bounds__(256)
 // block per query sorts the keys of its nseg lists of 64 (np: their count rounded
 // up to a power of two), takes the R = K' smallest, sums their exact distances in
 // the order of the FP32 kernel (a thread per row, dimension after dimension, so
-// both paths return the same bits) and ranks them.  The result has to be certain:
-// a row that is not among the R has an approximate distance of at least the R-th
-// and an exact one of at least that less the approximation's error, so the K-th
-// exact distance has to lie below.  A query that is not certain, that has fewer than R candidates (rows before it, or finite
+// both paths return the same bits) and ranks them.  A row that is not among the R has
+// an approximate distance of at least the R-th and an exact one of at least that less
+// both errors (all_beyond), so the K-th exact distance has to lie below.  A query for
+// which it does not, that has fewer than R candidates (rows before it, or finite
 // distances), or a full list whose keys are all among the R (it may have dropped
 // more) goes on `redo` (count in redo[0]) for the FP32 kernel.
 __global__ void __launch_bounds__(256)
@@ -1001,17 +1020,19 @@ __global__ void __launch_bounds__(256)
         const u64 k = ex[i];
         int rank = 0;
         for (int j = 0; j < R; ++j) rank += ex[j] < k || (ex[j] == k && j < i);
-        if (rank == K - 1) {
-            const float kth = dist_of(k);
-            if (!(kth < dist_of(last) - near_error(*xmax, qn[q], kth, q_m)) ||
-                inf_rows_reach(*xmax, qn[q], kth))
-                redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
-        }
+        if (rank == K - 1) top[0] = k;   // (the lists' largest keys are done with)
         if (rank < K) {
             const int32_t id = (int32_t)(uint32_t)k;
             out_ids[(size_t)q * K + rank] = id < 0 ? (int64_t)-1 : (int64_t)(remap ? remap[id] : id);
             out_d[(size_t)q * K + rank] = id < 0 ? INFINITY : dist_of(k);
         }
+    }
+    __syncthreads();
+    if (t == 0) {
+        const float kth = dist_of(top[0]), nq = qn[q];
+        if (!all_beyond(dist_of(last), near_error(*xmax, nq, kth, q_m), kth, q_m) ||
+            inf_rows_reach(*xmax, nq, kth))
+            redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
     }
 }
 
