@@ -290,16 +290,19 @@ finger_status finger_search_batch(finger_index* ix, const float* queries, int64_
  * finger_search_host and finger_search_batch then launch with it at any ef of
  * that bucket where it fits (a batch plans for the bucket's largest ef), else
  * with the default shape; batches too small to fill the GPU with a warp per query
- * run several warps per query whether tuned or not.  The best time in milliseconds is written to
- * *best_ms when it is not NULL. */
+ * run several warps per query whether tuned or not (a sample of that size is timed
+ * so, and tunes the hash size and row shape).  The best time in milliseconds, of the
+ * launch that a search of the sample's size makes, is written to *best_ms when it is
+ * not NULL. */
 finger_status finger_autotune(finger_index* ix, const float* queries, int64_t nq, int K, int ef,
                               int64_t* scratch_ids, float* scratch_dists, float* best_ms,
                               void* stream);
 
 /* The autotuner's pick for the current mode and the ef bucket of `ef` (any
- * pointer may be NULL): warps per block, visited-hash slots, resident warps
- * per SM, exact rows in flight per warp (the staging depth of the row
- * gathers) and the best sample-batch time in milliseconds.
+ * pointer may be NULL), as batches with a warp per query launch it: warps per
+ * block, visited-hash slots, resident warps per SM, exact rows in flight per warp
+ * (the staging depth of the row gathers) and the best sample-batch time in
+ * milliseconds.
  * FINGER_ERR_NOT_BUILT when that bucket was not tuned in this mode (it then
  * uses the default plan). */
 finger_status finger_get_tuned(const finger_index* ix, int ef, int* warps_per_block,

@@ -207,7 +207,8 @@ finger_status finger_search_batch(finger_index* ix, const float* queries, int64_
 // most resident warps that shared memory admits, and each one the mode has
 // with fewer: 64 / 72 / 80 / 96 registers, compiled for 32 / 28 / 24 / 20 resident
 // warps) x the exact-row shape (the default groups of lanes per row, and rows
-// on all 32 lanes: fewer rows in flight per warp, the staging depth).
+// on all 32 lanes: fewer rows in flight per warp, the staging depth); a sample that
+// takes several warps per query is timed in that form, over hash sizes and row shapes.
 // Returns the best time in *best_ms (may be NULL); finger_get_tuned reads
 // the pick back.
 finger_status finger_autotune(finger_index* ix, const float* queries, int64_t nq, int K, int ef,
@@ -254,7 +255,12 @@ finger_status finger_autotune(finger_index* ix, const float* queries, int64_t nq
                     Os[oi] >= a0.occ)
                     continue;
             }
-            SearchArgs a = fg_base_args(ix, p);
+            // what a search of this size launches with the candidate: several warps per
+            // query for a small sample, whatever the width and registers of the block
+            SearchPlan run = p;
+            fg_make_coop_plan(ix, ef, nq, &run);
+            if (run.occ == COOP_OCC && (p.wpb != def.wpb || oi > 0)) continue;
+            SearchArgs a = fg_base_args(ix, run);
             a.Q = queries;
             a.nq = nq;
             a.K = K;
@@ -265,7 +271,7 @@ finger_status finger_autotune(finger_index* ix, const float* queries, int64_t nq
             float tbest = 1e30f;
             for (int rep = 0; rep < 3; ++rep) {
                 cudaEventRecord(e0, s);
-                if (fg_run_search(ix, p, a, s) != FINGER_OK) break;
+                if (fg_run_search(ix, run, a, s) != FINGER_OK) break;
                 cudaEventRecord(e1, s);
                 cudaEventSynchronize(e1);
                 float ms = 0;
