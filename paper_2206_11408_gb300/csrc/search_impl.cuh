@@ -292,6 +292,42 @@ __device__ __forceinline__ bool t_take(uint2* T, int n, uint32_t flag, int lane,
     return true;
 }
 
+// Output of at least this many keys sorts T instead of scanning it for each.  One query over
+// 200k x 128, FP16 codes, scans / sort: 16 keys of ef 64 185 / 183 us; of ef 140 32 keys 355 /
+// 357, 64 keys 362 / 357; of ef 500 32 keys 1,398 / 1,406, 100 keys 1,424 / 1,406; of ef 1,000 64
+// keys 3,157 / 3,165, all 3,750 / 3,165.
+constexpr int SORT_K = 64;
+
+// T[0..n) in ascending order (flags cleared before): a bitonic sort whose merges start
+// with mirrored partners, so that every exchange puts the smaller key first and
+// entries beyond n, if there were any, would stay there.
+__device__ __forceinline__ void t_sort(uint2* T, int n, int lane) {
+    auto exchange = [&](int lo, int hi) {
+        if (hi >= n) return;
+        const uint2 a = T[lo], b = T[hi];
+        if (t_key(b) < t_key(a)) {
+            T[lo] = b;
+            T[hi] = a;
+        }
+    };
+    int half = 1;   // pairs: the next power of two / 2
+    while (2 * half < n) half <<= 1;
+    for (int size = 2; size <= 2 * half; size <<= 1) {
+        for (int i = lane; i < half; i += 32) {
+            const int in = i & (size / 2 - 1);
+            exchange(2 * i - in, 2 * i - in + size - 1 - 2 * in);
+        }
+        __syncwarp();
+        for (int stride = size >> 2; stride > 0; stride >>= 1) {
+            for (int i = lane; i < half; i += 32) {
+                const int lo = 2 * i - (i & (stride - 1));
+                exchange(lo, lo + stride);
+            }
+            __syncwarp();
+        }
+    }
+}
+
 enum { V_SEEN = 0, V_NEW = 1, V_NEW_SPILL = 2, V_PENDING = 3 };
 
 // The visited hash in shared memory is bucketed: H slots form H/4 buckets of
@@ -1463,18 +1499,26 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
             __syncwarp();
         }
 
-        // ---- the head of T in order: its R smallest keys
+        // ---- the head of T in order: its R smallest keys, taken one at a time by scans of T
+        // where they are few, else after sorting it
         const int R = min(sz, LP ? max(K, a.rerank) : K);
         for (int i = lane; i < sz; i += 32) T[i].y &= ~EXPW;   // now: taken for the output
         __syncwarp();
+        const bool sorted = R >= SORT_K;
+        if (sorted) t_sort(T, sz, lane);
+        auto take = [&](int i) {   // the i-th key; i ascending from 0
+            uint2 e;
+            if (sorted) e = T[i];
+            else t_take(T, sz, EXPW, lane, e.x, e.y);
+            return e;
+        };
         if constexpr (LP) {
             // re-rank with FP32 rows; the plan keeps 2 ef_cap words in the table
             uint2* hd = reinterpret_cast<uint2*>(hash);
             for (int i = 0; i < R; ++i) {
-                uint32_t d, w;
-                t_take(T, sz, EXPW, lane, d, w);
-                const float x = exact_f32_row(qs, ix, w >> WSH, lane);
-                if (lane == 0) hd[i] = make_uint2(__float_as_uint(x), w >> WSH);
+                const uint32_t id = take(i).y >> WSH;
+                const float x = exact_f32_row(qs, ix, id, lane);
+                if (lane == 0) hd[i] = make_uint2(__float_as_uint(x), id);
             }
             __syncwarp();
             for (int i = lane; i < R; i += 32) {
@@ -1494,21 +1538,21 @@ __global__ void __launch_bounds__(OCC == COOP_OCC ? 32 * COOP_MAX_WARPS : 128,
 
         // ---- a7: output
         for (int k0 = 0; k0 < K; k0 += 32) {
-            uint32_t od = 0x7F800000u;   // +inf: no result
-            int64_t oi = -1;
-            if constexpr (!LP)
-                for (int k = k0; k < min(k0 + 32, R); ++k) {
-                    uint32_t d, w;
-                    t_take(T, sz, EXPW, lane, d, w);
-                    if (lane == k - k0) {
-                        od = d;
-                        oi = (int64_t)(w >> WSH);
+            const int k = k0 + lane;
+            uint2 o = make_uint2(0x7F800000u, ~0u);   // +inf: no result
+            if constexpr (!LP) {
+                if (sorted) {
+                    if (k < R) o = T[k];
+                } else {
+                    for (int i = k0; i < min(k0 + 32, R); ++i) {
+                        const uint2 e = take(i);
+                        if (lane == i - k0) o = e;
                     }
                 }
-            const int k = k0 + lane;
+            }
             if (k < K && (!LP || k >= R)) {
-                a.out_ids[ooff + k] = oi;
-                a.out_d[ooff + k] = __uint_as_float(od);
+                a.out_ids[ooff + k] = o.y == ~0u ? (int64_t)-1 : (int64_t)(o.y >> WSH);
+                a.out_d[ooff + k] = __uint_as_float(o.x);
             }
         }
         for (int i = lane; i < nspill; i += 32) bitmap[spl[i] >> 5] = 0u;
