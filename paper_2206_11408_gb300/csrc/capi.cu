@@ -242,23 +242,41 @@ finger_status make_plan(finger_index* ix, int mode, int ef_max, int64_t nq, Sear
     }
     p->NPL = ix->deg0 > 32 ? 2 : 1;
     p->ef_cap = (ef_max + 3) & ~3;
+    p->H_auto = H <= 0;
     if (H <= 0) H = pow2ceil(std::min(std::max(16 * ef_max, 512), 2048));
     // the code modes, and every mode with long rows, keep the staged query in a
     // region of its own; else it is staged in the hash region
     const bool own_qs = code_mode(mode) || p->VPL >= LONG_VPL;
+    const bool long_rows = own_qs && !code_mode(mode);
     if (mode == FINGER_MODE_FINGER_LP) H = std::max(H, pow2ceil(2 * p->ef_cap));
-    else H = std::max(H, pow2ceil(ix->m_pad));
-    p->H = H;
+    else if (p->H_auto || !long_rows) H = std::max(H, pow2ceil(ix->m_pad));
+    p->wpb = wpb;
+    p->blk_smem = 0;
+    p->occ = occ_force;
     // 16-bit visited slots: ids must fit the bucket index plus 15 bits
     // (n <= 4096 H), and what reuses the table's H / 2 words must fit there:
     // the staged query (m_pad words) outside LP mode, the re-rank buffer
     // (2 ef_cap words) in LP mode
-    p->h16 = ix->visited_bits != 32 && ix->n <= 4096 * (int64_t)H &&
-             (mode == FINGER_MODE_FINGER_LP ? H >= 4 * p->ef_cap : H >= 2 * ix->m_pad);
-    p->wpb = wpb;
-    p->smem_per_warp = search_smem_per_warp(d, mode, p->ef_cap, p->H, p->NPL, p->h16, own_qs);
-    p->blk_smem = 0;
-    p->occ = occ_force;
+    auto set_table = [&](int slots, bool query_there) {
+        p->H = slots;
+        p->h16 = ix->visited_bits != 32 && ix->n <= 4096 * (int64_t)slots &&
+                 (mode == FINGER_MODE_FINGER_LP ? slots >= 4 * p->ef_cap
+                                                : !query_there || slots >= 2 * ix->m_pad);
+        p->smem_per_warp = search_smem_per_warp(d, mode, p->ef_cap, p->H, p->NPL, p->h16, own_qs);
+    };
+    set_table(H, p->H_auto || !long_rows);
+    // Long rows in the modes without codes: the staged query's region (3,840 bytes at m =
+    // 960) may cost the fifth block of an SM.  A smaller table makes up for it, down to a
+    // quarter: at such ef most ids are in the bitmap either way.  m = 960, 3,000 queries, 16
+    // resident warps with 2,048 slots -> 20 with 1,024: plain ef 300 3.93 -> 3.51 ms, 500 5.51 ->
+    // 4.73; FP32 tables 500 6.26 -> 5.35; 512 slots, ef 600: plain 6.06 -> 5.20.  10,000
+    // queries: the same within 2 % (ef 400 10.87 -> 10.58, 500 12.71 -> 12.62).
+    if (p->H_auto && occ_force == 0 && long_rows) {
+        const int room = (228 * 1024 / 5 - 1024) / wpb;   // per warp, for five blocks
+        const int full = p->H;
+        for (int h = full; h >= full / 4 && h >= 256 && p->smem_per_warp > room; h >>= 1) set_table(h, false);
+        if (p->smem_per_warp > room) set_table(full, true);
+    }
     if (plan_smem(*p) > 227 * 1024) return FINGER_ERR_UNSUPPORTED;
     // the variant with the most resident blocks that shared memory admits, among
     // those the mode and shape have (has_variant in search_impl.cuh)
@@ -320,7 +338,8 @@ void make_coop_plan(finger_index* ix, int ef_max, int64_t nq, SearchPlan* p) {
     for (int W = COOP_MAX_WARPS; W >= narrowest; W >>= 1) {
         if (nq > (int64_t)ix->num_sms * (2 * COOP_MAX_WARPS / W)) continue;
         SearchPlan t;
-        if (make_plan(ix, p->mode, ef_max, nq, &t, W, p->H, COOP_OCC, p->shape) != FINGER_OK) {
+        if (make_plan(ix, p->mode, ef_max, nq, &t, W, p->H_auto ? 0 : p->H, COOP_OCC, p->shape) !=
+            FINGER_OK) {
             cudaGetLastError();
             return;
         }

@@ -130,6 +130,7 @@ struct SearchPlan {
     int wpb;            // warps per block
     int blocks;
     int ef_cap, H;
+    int H_auto;         // H is the default for its ef (not the autotuner's)
     int h16;            // visited hash in 16-bit slots
     int occ;            // resident blocks of 4 warps per SM the kernel variant is compiled for,
                         // or COOP_OCC: one query per block of wpb warps
