@@ -41,13 +41,14 @@ __device__ __forceinline__ bool klt(float da, uint32_t ia, float db, uint32_t ib
 // requested early: 32 candidates' ids and distances at a time, the next
 // candidate's row while this one is compared, and four kept rows per step (their
 // comparisons are independent; one closer to the candidate rejects it).  One
-// kept row per step with its loads waited for: 9.2 ms for the forward links of 200k
-// x 128 rows (200 candidates) and 4.1 for the second pass; now 6.3 and 1.7.
+// kept row per step with its loads waited for (k_select_long): 9.2 ms for the
+// forward links of 200k x 128 rows (200 candidates) and 4.1 for the second pass; 6.3
+// and 1.7 here.
 template <int VPL>
 __global__ void k_select(const float4* __restrict__ X, int m4, const int64_t* __restrict__ cid,
                          const float* __restrict__ cd, int kc, int64_t rows, int Mmax,
                          uint32_t* out, float* out_d, int out_w, const int64_t* __restrict__ out_row) {
-    constexpr int U = VPL > 2 ? 2 : 4;   // kept rows per step
+    constexpr int U = 4;   // kept rows per step
     __shared__ uint32_t kept_s[4][64];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
@@ -127,6 +128,66 @@ __global__ void k_select(const float4* __restrict__ X, int m4, const int64_t* __
     }
 }
 
+// The same for rows of more than 256 floats, whose own loads are enough for a warp to have
+// in flight: one kept row per step, nothing requested ahead.  30,000 rows, 200
+// candidates, forward links and second pass: m = 400 2.49 + 1.01 ms (k_select with two
+// kept rows per step 2.91 + 1.29), 700 3.07 + 1.50 (6.29 + 2.76), 960 3.52 + 1.60 (8.16 + 3.66);
+// m = 200 2.23 + 0.82 (1.82 + 0.49).
+__global__ void k_select_long(const float4* __restrict__ X, int m4, const int64_t* __restrict__ cid,
+                              const float* __restrict__ cd, int kc, int64_t rows, int Mmax,
+                              uint32_t* out, float* out_d, int out_w,
+                              const int64_t* __restrict__ out_row) {
+    __shared__ uint32_t kept_s[4][64];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
+    if (w >= rows) return;
+    uint32_t* kept = kept_s[wib];
+    float kd[2] = {0.f, 0.f};   // as above
+    int nk = 0;
+    for (int i = 0; i < kc && nk < Mmax; ++i) {
+        const int64_t e = cid[w * kc + i];
+        if (e < 0) break;
+        const float de = cd[w * kc + i];
+        float4 xe[8];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            const int k = lane + 32 * v;
+            xe[v] = k < m4 ? __ldg(X + e * m4 + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        bool good = true;
+        for (int j = 0; j < nk && good; ++j) {
+            const float4* row = X + (size_t)kept[j] * m4;
+            float acc = 0.f;
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                const int k = lane + 32 * v;
+                if (k < m4) {
+                    const float4 y = __ldg(row + k);
+                    float d;
+                    d = xe[v].x - y.x; acc = fmaf(d, d, acc);
+                    d = xe[v].y - y.y; acc = fmaf(d, d, acc);
+                    d = xe[v].z - y.z; acc = fmaf(d, d, acc);
+                    d = xe[v].w - y.w; acc = fmaf(d, d, acc);
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            good = de < acc;
+        }
+        if (good) {
+            if (lane == 0) kept[nk] = (uint32_t)e;
+            if (lane == (nk & 31)) kd[nk >> 5] = de;
+            __syncwarp();
+            nk++;
+        }
+    }
+    const int64_t orow = out_row ? out_row[w] : w;
+    for (int j = lane; j < out_w; j += 32) {
+        out[orow * out_w + j] = j < nk ? kept[j] : PAD;
+        if (out_d) out_d[orow * out_w + j] = j < nk ? kd[j >> 5] : INFINITY;
+    }
+}
+
 cudaError_t launch_select(const float4* X, int m4, const int64_t* cid, const float* cd, int kc,
                           int64_t rows, int Mmax, uint32_t* out, float* out_d, int out_w,
                           const int64_t* out_row, cudaStream_t s) {
@@ -135,10 +196,8 @@ cudaError_t launch_select(const float4* X, int m4, const int64_t* cid, const flo
         k_select<1><<<blocks, 128, 0, s>>>(X, m4, cid, cd, kc, rows, Mmax, out, out_d, out_w, out_row);
     else if (m4 <= 64)
         k_select<2><<<blocks, 128, 0, s>>>(X, m4, cid, cd, kc, rows, Mmax, out, out_d, out_w, out_row);
-    else if (m4 <= 128)
-        k_select<4><<<blocks, 128, 0, s>>>(X, m4, cid, cd, kc, rows, Mmax, out, out_d, out_w, out_row);
     else
-        k_select<8><<<blocks, 128, 0, s>>>(X, m4, cid, cd, kc, rows, Mmax, out, out_d, out_w, out_row);
+        k_select_long<<<blocks, 128, 0, s>>>(X, m4, cid, cd, kc, rows, Mmax, out, out_d, out_w, out_row);
     return cudaGetLastError();
 }
 
