@@ -16,7 +16,8 @@
 //               dz2 = dy w3 [h2 > 0], dz1 = W2^T dz2 [h1 > 0] and the squared errors
 //   k_weights   thread per weight: sums of dz1 x~, dz2 h1~, dy h2 over the batch (a
 //               bias is the weight of a constant 1), then Adam on the FP32 master
-// Every sum runs in a fixed order (units, inputs and rows ascending).  Weights are
+// Every sum of outputs and gradients runs in a fixed order (units, inputs and rows
+// ascending); the reported losses and eps' add their blocks' sums as they come, in 64 bits.  Weights are
 // rounded to BF16 as they are read.  Between the two kernels a quantity is stored
 // unit-major (one row of B values per unit), so that both sides move 16 bytes per
 // lane.  A step of 4,096 rows with r = 24 took 500 us as six kernels (the weight
@@ -65,7 +66,10 @@ constexpr int RT = 256;       // its threads: a warp per 8 units
 constexpr int WTJ = 8, WTK = 16, WTB = 128;   // weights per block of k_weights, rows per stage
 constexpr int WLD = WTB + 4;  // its row stride in shared memory (conflict-free 16-byte reads)
 
-size_t rows_smem(int nf) { return sizeof(float) * ((size_t)nf * (HID + RB) + 2 * HID * HID + 3 * HID * RB + 2 * HID + 4 * HID); }
+size_t rows_smem(int nf, bool train) {
+    return sizeof(float) * ((size_t)nf * (HID + RB) + HID * HID + 2 * HID * RB + HID + RB +
+                            (train ? HID * HID + HID * RB : 0));
+}
 
 // per-unit arrays of a batch: nf, 64, 64, 64, 64 and 1 rows of Bp values
 struct Batch {
@@ -73,7 +77,10 @@ struct Batch {
     int64_t Bp;
 };
 
-// rows idx[0 .. B) (or 0 .. B - 1) of X (N x nf).  g.x == nullptr: forward only.
+// rows idx[0 .. B) (or 0 .. B - 1) of X (N x nf).  TRAIN: a block per 32 rows.  Forward only:
+// the block goes on to further ones with its weights in place (2M rows, r = 24: 1.08 ms; 2.43
+// with a block per 32 rows, which spent it on the weights; 1.78 for a thread per row).
+template <bool TRAIN>
 __global__ void __launch_bounds__(RT) k_rows(const float* __restrict__ w, int nf,
                                              const float* __restrict__ X, const float* __restrict__ T,
                                              const int64_t* __restrict__ idx, int B, Batch g,
@@ -81,31 +88,22 @@ __global__ void __launch_bounds__(RT) k_rows(const float* __restrict__ w, int nf
     extern __shared__ __align__(16) float sw[];
     float* W1t = sw;                       // nf x 64: W1 transposed
     float* W2t = W1t + nf * HID;           // 64 x 64: W2 transposed
-    float* W2s = W2t + HID * HID;          // 64 x 64: W2
-    float* xs = W2s + HID * HID;           // nf x 32
+    float* xs = W2t + HID * HID;           // nf x 32
     float* h1 = xs + nf * RB;              // 64 x 32
     float* h2 = h1 + HID * RB;             // 64 x 32
-    float* dz = h2 + HID * RB;             // 64 x 32
-    float* w3 = dz + HID * RB;             // 64
+    float* w3 = h2 + HID * RB;             // 64
     float* dyv = w3 + HID;                 // 32
+    float* W2s = dyv + RB;                 // (TRAIN) 64 x 64: W2
+    float* dz = W2s + HID * HID;           // (TRAIN) 64 x 32
     const Off o(nf);
     const int t = threadIdx.x, lane = t & 31, u0 = (t >> 5) * 8;
-    const bool train = g.x != nullptr;
     for (int i = t; i < HID * nf; i += RT) W1t[(i % nf) * HID + i / nf] = bf(w[o.W1 + i]);
     for (int i = t; i < HID * HID; i += RT) {
         const float v = bf(w[o.W2 + i]);
-        W2s[i] = v;
+        if (TRAIN) W2s[i] = v;
         W2t[(i % HID) * HID + i / HID] = v;
     }
     if (t < HID) w3[t] = bf(w[o.w3 + t]);
-    const int b = blockIdx.x * RB + lane;
-    for (int i = t; i < RB * nf; i += RT) {   // consecutive threads: consecutive features of a row
-        const int r = i / nf, f = i % nf, br = blockIdx.x * RB + r;
-        xs[f * RB + r] = br < B ? bf(X[(idx ? idx[br] : (int64_t)br) * nf + f]) : 0.f;
-    }
-    __syncthreads();
-    if (train && b < B)
-        for (int f = t >> 5; f < nf; f += RT / 32) g.x[f * g.Bp + b] = xs[f * RB + lane];
 
     // out[u0 .. u0 + 7][lane] = init + sum over i of M[i][u] v[i][lane], i ascending
     auto layer = [&](const float* M, const float* v, int n, float (&z)[8]) {
@@ -124,62 +122,73 @@ __global__ void __launch_bounds__(RT) k_rows(const float* __restrict__ w, int nf
             z[7] = fmaf(m1.w, a, z[7]);
         }
     };
-    float z[8];
+    for (int r0 = blockIdx.x * RB; r0 < B; r0 += gridDim.x * RB) {
+        const int b = r0 + lane;
+        for (int i = t; i < RB * nf; i += RT) {   // consecutive threads: consecutive features of a row
+            const int r = i / nf, f = i % nf, br = r0 + r;
+            xs[f * RB + r] = br < B ? bf(X[(idx ? idx[br] : (int64_t)br) * nf + f]) : 0.f;
+        }
+        __syncthreads();
+        if (TRAIN && b < B)
+            for (int f = t >> 5; f < nf; f += RT / 32) g.x[f * g.Bp + b] = xs[f * RB + lane];
+        float z[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) z[q] = w[o.b1 + u0 + q];
-    layer(W1t, xs, nf, z);
+        for (int q = 0; q < 8; ++q) z[q] = w[o.b1 + u0 + q];
+        layer(W1t, xs, nf, z);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const float h = bf(fmaxf(z[q], 0.f));
-        h1[(u0 + q) * RB + lane] = h;
-        if (train && b < B) g.h1[(u0 + q) * g.Bp + b] = h;
-        z[q] = w[o.b2 + u0 + q];
-    }
-    __syncthreads();
-    layer(W2t, h1, HID, z);
+        for (int q = 0; q < 8; ++q) {
+            const float h = bf(fmaxf(z[q], 0.f));
+            h1[(u0 + q) * RB + lane] = h;
+            if (TRAIN && b < B) g.h1[(u0 + q) * g.Bp + b] = h;
+            z[q] = w[o.b2 + u0 + q];
+        }
+        __syncthreads();
+        layer(W2t, h1, HID, z);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const float h = fmaxf(z[q], 0.f);
-        h2[(u0 + q) * RB + lane] = h;
-        if (train && b < B) g.h2[(u0 + q) * g.Bp + b] = h;
-    }
-    __syncthreads();
-    if (t < 32) {
-        float y = w[o.b3];
+        for (int q = 0; q < 8; ++q) {
+            const float h = fmaxf(z[q], 0.f);
+            h2[(u0 + q) * RB + lane] = h;
+            if (TRAIN && b < B) g.h2[(u0 + q) * g.Bp + b] = h;
+        }
+        __syncthreads();
+        if (t < 32) {
+            float y = w[o.b3];
 #pragma unroll 8
-        for (int k = 0; k < HID; ++k) y = fmaf(w3[k], h2[k * RB + lane], y);
-        float e = 0.f;
-        if (b < B) {
-            if (y_out) y_out[b] = y;
-            e = y - (T ? T[idx ? idx[b] : (int64_t)b] : 0.f);
-            if (res) res[b] = e;
+            for (int k = 0; k < HID; ++k) y = fmaf(w3[k], h2[k * RB + lane], y);
+            float e = 0.f;
+            if (b < B) {
+                if (y_out) y_out[b] = y;
+                e = y - (T ? T[idx ? idx[b] : (int64_t)b] : 0.f);
+                if (res) res[b] = e;
+            }
+            if (TRAIN) {
+                const float dy = 2.f * e / (float)B;
+                dyv[lane] = dy;
+                if (b < B) g.dy[b] = dy;
+                double a = (double)e * e;
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+                if (lane == 0) atomicAdd(sq, a);
+            }
         }
-        if (train) {
-            const float dy = 2.f * e / (float)B;
-            dyv[lane] = dy;
-            if (b < B) g.dy[b] = dy;
-            double a = (double)e * e;
+        if (!TRAIN) continue;   // (the next rows' barriers keep h2 until it is read)
+        __syncthreads();
+        const float dy = dyv[lane];
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-            if (lane == 0) atomicAdd(sq, a);
+        for (int q = 0; q < 8; ++q) {
+            const int k = u0 + q;
+            const float d = h2[k * RB + lane] > 0.f ? dy * w3[k] : 0.f;
+            dz[k * RB + lane] = d;
+            if (b < B) g.dz2[k * g.Bp + b] = d;
+            z[q] = 0.f;
         }
-    }
-    if (!train) return;
-    __syncthreads();
-    const float dy = dyv[lane];
+        __syncthreads();
+        layer(W2s, dz, HID, z);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int k = u0 + q;
-        const float d = h2[k * RB + lane] > 0.f ? dy * w3[k] : 0.f;
-        dz[k * RB + lane] = d;
-        if (b < B) g.dz2[k * g.Bp + b] = d;
-        z[q] = 0.f;
+        for (int q = 0; q < 8; ++q)
+            if (b < B) g.dz1[(u0 + q) * g.Bp + b] = h1[(u0 + q) * RB + lane] > 0.f ? z[q] : 0.f;
+        break;
     }
-    __syncthreads();
-    layer(W2s, dz, HID, z);
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-        if (b < B) g.dz1[(u0 + q) * g.Bp + b] = h1[(u0 + q) * RB + lane] > 0.f ? z[q] : 0.f;
 }
 
 __device__ __forceinline__ void adam(float* w, float* m, float* v, int64_t i, float gi, float lr,
@@ -309,13 +318,21 @@ bool get_batch(Buf& buf, int nf, int64_t B, Batch* g) {
     return g->x && g->h1 && g->h2 && g->dz1 && g->dz2 && g->dy;
 }
 
-cudaError_t run_rows(const float* w, int nf, const float* X, const float* T, const int64_t* idx,
+// g.x == nullptr: forward only
+cudaError_t run_rows(int num_sms, const float* w, int nf, const float* X, const float* T, const int64_t* idx,
                      int B, const Batch& g, float* res, float* y, double* sq, cudaStream_t s) {
-    const size_t smem = rows_smem(nf);
+    const bool train = g.x != nullptr;
+    const int smem = (int)rows_smem(nf, train), tiles = (B + RB - 1) / RB;
     const cudaError_t e =
-        cudaFuncSetAttribute(k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        train ? cudaFuncSetAttribute(k_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
+              : cudaFuncSetAttribute(k_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    k_rows<<<(B + RB - 1) / RB, RT, smem, s>>>(w, nf, X, T, idx, B, g, res, y, sq);
+    if (train) {
+        k_rows<true><<<tiles, RT, smem, s>>>(w, nf, X, T, idx, B, g, res, y, sq);
+    } else {   // (227 KB of shared memory, 8 blocks of 256 threads)
+        const int blocks = num_sms * std::min(8, 227 * 1024 / (smem + 1024));
+        k_rows<false><<<std::min(tiles, blocks), RT, smem, s>>>(w, nf, X, T, idx, B, g, res, y, sq);
+    }
     return cudaGetLastError();
 }
 
@@ -499,7 +516,7 @@ finger_status finger_mlp_loss_grad(finger_index* ix, int nf, const float* weight
         double h = 0;
         bool ok = cudaMemcpyAsync(w, weights, nw * 4, cudaMemcpyHostToDevice, s) == cudaSuccess;
         ok = ok && cudaMemsetAsync(acc, 0, 8, s) == cudaSuccess;
-        ok = ok && run_rows(w, nf, feat, target, nullptr, B, bt, nullptr, nullptr, acc, s) == cudaSuccess;
+        ok = ok && run_rows(ix->num_sms, w, nf, feat, target, nullptr, B, bt, nullptr, nullptr, acc, s) == cudaSuccess;
         ok = ok && run_weights(nf, B, bt, g, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, 1.f, 1.f, s) ==
                        cudaSuccess;
         ok = ok && cudaMemcpyAsync(grad, g, nw * 4, cudaMemcpyDeviceToHost, s) == cudaSuccess;
@@ -533,7 +550,7 @@ finger_status finger_mlp_predict(finger_index* ix, const float* feat, int64_t n,
         bool ok = cudaMemcpyAsync(w, ix->h_mlp.data(), nw * 4, cudaMemcpyHostToDevice, s) == cudaSuccess;
         for (int64_t lo = 0; lo < n && ok; lo += 1 << 20) {
             const int B = (int)std::min<int64_t>(n - lo, 1 << 20);
-            ok = run_rows(w, nf, feat + lo * nf, nullptr, nullptr, B, Batch{}, nullptr, out + lo, nullptr,
+            ok = run_rows(ix->num_sms, w, nf, feat + lo * nf, nullptr, nullptr, B, Batch{}, nullptr, out + lo, nullptr,
                           s) == cudaSuccess;
         }
         ok = ok && cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess;
@@ -594,7 +611,7 @@ finger_status finger_train_predictor(finger_index* ix, const finger_train_params
         for (int64_t lo = 0; lo + B <= p->n_train && ok; lo += B) {
             step++;
             const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-            ok = run_rows(w, nf, p->feat, p->target, idx + lo, B, bt, nullptr, nullptr, acc, s) ==
+            ok = run_rows(ix->num_sms, w, nf, p->feat, p->target, idx + lo, B, bt, nullptr, nullptr, acc, s) ==
                      cudaSuccess &&
                  run_weights(nf, B, bt, nullptr, w, m1, m2, p->lr, b1, b2, c1, c2, s) == cudaSuccess;
         }
@@ -611,7 +628,7 @@ finger_status finger_train_predictor(finger_index* ix, const finger_train_params
         const int64_t v0 = p->n_train, nv = p->n_val;
         for (int64_t lo = 0; lo < nv && ok; lo += B) {
             const int nb = (int)std::min<int64_t>(B, nv - lo);
-            ok = run_rows(w, nf, p->feat + (v0 + lo) * nf, p->target + v0 + lo, nullptr, nb, Batch{}, res,
+            ok = run_rows(ix->num_sms, w, nf, p->feat + (v0 + lo) * nf, p->target + v0 + lo, nullptr, nb, Batch{}, res,
                           nullptr, nullptr, s) == cudaSuccess;
             k_abs_sum<<<16, 256, 0, s>>>(res, nb, acc);
         }
