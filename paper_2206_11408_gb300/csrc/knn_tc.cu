@@ -31,7 +31,7 @@
 // per row (replace the largest key, find its group's next, then the row's).  A
 // warp-wide insertion of one candidate into one row's sorted list took 260 cycles
 // and bounded the launch: the causal candidate search over 200k x 128 rows spent
-// 145 ms there; now 35 ms (an insertion for 32 rows at once takes 500 cycles).
+// 145 ms there; now 27 ms (an insertion for 32 rows at once takes 500 cycles).
 //
 // Work is dealt out in items of one query tile and one base segment: contiguous
 // segments for a kNN launch, base tiles s, s + nseg, ... for the causal one.  Every mbarrier wait is bounded: on a timeout the kernel raises an
@@ -83,14 +83,17 @@ __device__ __forceinline__ float dist_of(u64 k) {
 //   (ceil(m / 32) + 12) u (|q|^2 + |x|^2): the norms' sums (m / 32 + 4 per lane, 5 between
 //     lanes) and the two roundings that put the distance together
 // +inf where a distance could overflow.
+__host__ __device__ constexpr float product_error(int m) {
+    return 2.f * (0x1p-15f + 3.f * ((m + 15) / 16) * 0x1p-22f);
+}
+__host__ __device__ constexpr float norm_error(int m) { return ((m + 31) / 32 + 12) * 0x1p-24f; }
 __device__ __forceinline__ float split_error(float nq, float nx, int m) {
-    return 2.f * (0x1p-15f + 3.f * ((m + 15) / 16) * 0x1p-22f) * sqrtf(nq) * sqrtf(nx) +
-           ((m + 31) / 32 + 12) * 0x1p-26f * (4.f * (nq + nx));
+    return product_error(m) * sqrtf(nq) * sqrtf(nx) + 0.25f * norm_error(m) * (4.f * (nq + nx));
 }
 
 // Bound on the relative error of an exact distance, the FP32 sum of (q - x)^2 in any
 // order: m additions, a subtraction's error twice, a product's
-__device__ __forceinline__ float sum_error(int m) { return (m + 8) * 0x1p-24f; }
+__host__ __device__ constexpr float sum_error(int m) { return (m + 8) * 0x1p-24f; }
 
 // Whether every row whose approximate distance is v or more, with error err, has an exact
 // one above d
@@ -129,8 +132,7 @@ struct TcArgs {
     const float* qn;      // ||q||^2 (FP32), nq
     const float* xn;      // ||x||^2 (FP32), n
     u64* keys;            // nq x nseg x KP candidate keys
-    const NormMax* xmax;  // with bound: the base's norms
-    int m;
+    float cap_scale, cap_norm;   // with bound: see margins()
     uint32_t* bound;      // optional: per row, the smallest K'-th distance of its finished
                           // segments (ord_of), 0xFFFFFFFF before the first
     int* err;             // device status word (FINGER_ERR_LIMIT on a wait timeout)
@@ -558,13 +560,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             if (a.pilot && seg >= a.pilot) bound = min(bound, pilots);
             if (a.bound && qi < a.nq) bound = min(bound, *(volatile uint32_t*)(a.bound + qi));
             float cap = bound < 0xFF800000u ? dist_of((u64)(bound + 1u) << 32) : INFINITY;
-            // (a kNN launch keeps what the approximation may have misplaced, see k_rerank)
-            // for the rows at the bound's distance or nearer, whose exact one is at most
-            // 1.001 (bound + 0.001 |q|^2): the error is below 2^-11 of |q|^2 + |x|^2
-            if (a.bound) {
-                const float err = near_error(*a.xmax, qn, 1.001f * (fmaxf(cap, 0.f) + 0.001f * qn), a.m);
-                cap = (cap + 2.f * err) * (1.f + 4.f * sum_error(a.m));
-            }
+            // (a kNN launch keeps what the approximation may have misplaced, see margins())
+            if (a.bound) cap = fmaf(fmaxf(cap, 0.f), a.cap_scale, qn * a.cap_norm);
             float thr = qi < a.nq ? cap : -INFINITY;
             int cnt = 0;                                    // pending candidates of the row
             top.clear();
@@ -925,8 +922,8 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
 
 // The queries on `redo` from the FP32 kernel's lists (launch_knn_parts with this grid
 // and room): KP smallest keys of all parts, then as k_rerank, whose sums they get.  10,000
-// queries x 1M x 128, K = 10: 6.33 ms with none, 8.07 with one, 227 with all of them (the
-// rows 10,000 from the origin in every dimension; 1,000 needs none, 7.3 ms).
+// queries x 1M x 128, K = 10: 6.35 ms with none, 8.11 with one, 227 with all of them (the
+// rows 10,000 from the origin in every dimension; at 1,000 most stand, 8.5 ms).
 __global__ void __launch_bounds__(256)
     k_redo_rank(const float4* __restrict__ X, int64_t n, int m4, const float* __restrict__ Q, int m,
                 const u64* __restrict__ parts, int grid, int64_t room, int KP, int K,
@@ -1215,6 +1212,21 @@ TcBase base_of(const finger_index* ix) {
 
 enum TcOrder { CONTIGUOUS, INTERLEAVED, CAUSAL };
 
+// What a finished segment's K'-th approximate distance c lets the row's other segments drop:
+// K' rows have exact distances of at most c plus both errors, so that a row is no
+// result whose approximate distance is above c + 2 split_error + the sums' errors, for
+// rows that may be as near (the others are farther by their length).  With |x| <= |q| +
+// sqrt(d), |q| |x| is at most 1.5 |q|^2 + d / 2 and |x|^2 at most 2 |q|^2 + 2 d, where d <=
+// 1.001 (c + 0.001 |q|^2) as the error is below 2^-11 (|q|^2 + |x|^2): a line in c and |q|^2.
+// (With square roots in the kernel 10,000 queries x 1M x 128 took 6.08 ms there instead of
+// 6.04.)
+void margins(int m, TcArgs* a) {
+    const double p = product_error(m), e = norm_error(m), s = 1 + 4 * (double)sum_error(m);
+    const double A = 1.5 * p + 3 * e, B = 0.5 * p + 2 * e, up = 1 + 0x1p-20;
+    a->cap_scale = (float)((1 + 2.002 * B) * s * up);
+    a->cap_norm = (float)((2 * A + 0.002002 * B) * s * up);
+}
+
 // one launch of k_knn_tc over nq query rows (BF16 parts qh/ql) against the base
 cudaError_t run_items(finger_index* ix, const TcBase& x, const __nv_bfloat16* qh,
                       const __nv_bfloat16* ql, const float* qn, int64_t nq, int KP, int nseg,
@@ -1241,12 +1253,14 @@ cudaError_t run_items(finger_index* ix, const TcBase& x, const __nv_bfloat16* qh
     a.xn = x.xn;
     a.keys = keys;
     a.bound = bound;
-    a.xmax = x.xmax;
-    a.m = x.m;
+    margins(x.m, &a);
     a.err = ix->err;
     // want > 0: the smallest `want` keys of a causal launch's lists are used.  With query
     // tiles enough for all SMs a CTA keeps a tile's segments, and the first of them
-    // bound the others (200k x 128 rows, 8 lists of 64 for 200 keys: 33.6 -> 27.3 ms)
+    // bound the others (200k x 128 rows, 8 lists of 64 for 200 keys: 33.6 -> 27.3 ms; whole
+// builds without / with: 120k x 128 29.9 / 26.7 ms, 80k 19.1 / 17.2, 80k x 960 36.8 /
+// 35.9.  Below, the items of few tiles fill the GPU unevenly: 20k x 960 9.13 / 9.47, 10k
+// x 128 4.10 / 4.37, though 40k x 128 would gain, 10.8 / 10.0)
     if (order == CAUSAL && want > 0 && a.nqt >= 4 * ix->num_sms) a.pilot = (want + 63) / 64;
     const int grid = (int)std::min<int64_t>(ix->num_sms, (int64_t)a.nqt * (a.pilot ? 1 : nseg));
     const bool res = a.nchunk <= QRES_CHUNKS;
@@ -1259,7 +1273,8 @@ cudaError_t run_items(finger_index* ix, const TcBase& x, const __nv_bfloat16* qh
 // the CTAs of a wave scan the same rows at the same time: a segment of at most 48 MB of
 // BF16 parts stays in L2 for them.  (One equal range of the (query tile, base tile)
 // sequence per CTA balances without waves, but each CTA then scans rows of its own and
-// DRAM bounds it: 10,000 queries x 1M x 128 took 11.6 ms.)  From there the smallest
+// DRAM bounds it: 10,000 queries x 1M x 128 took 11.6 ms; with segments of 12 MB 7.9, of 24
+// 7.1, of 48 to 192 6.5.)  From there the smallest
 // count whose last wave costs at most 3 %, or the best of the next 32; each segment
 // adds a list of K' per row to fill and to merge.  Above MAX_KEYS / K' such segments
 // (12.9 or 25.8 GB of parts) they grow instead: k_rerank takes MAX_KEYS keys per query
@@ -1416,7 +1431,7 @@ done:
 // either way.  Base rows Xb (n x m4 chunks, norms xn, BF16 parts hi / lo); causal:
 // the queries are the base rows and row i sees rows j < i, reported as remap[j].
 // Falls back to launch_knn where the base is small or memory for the lists is not
-// to be had.  1,000 queries x 100k x 960, K = 100: 75.6 ms with the FP32 kernel, 0.85
+// to be had.  1,000 queries x 100k x 960, K = 100: 75.6 ms with the FP32 kernel, 0.88
 // here; the 12.5k rows of the first upper layer of a 200k x 128 graph, 256
 // candidates: 13.6 ms and 3.4 (0.8 lists, 1.1 merge, 1.5 the first 500 rows again).
 namespace {
@@ -1488,7 +1503,9 @@ done:
     return e;
 }
 
-// rows from which the tensor cores serve K > 40: 32 tiles, two per segment
+// rows from which the tensor cores serve K > 40: 32 tiles, two per segment (K = 100, FP32 /
+// tensor cores: 4,096 x 64, one query 464 / 289 us, 2,000 queries 1,378 / 550; 1,024 x 64 245 /
+// 291 and 816 / 379)
 constexpr int64_t BIG_MIN_ROWS = 32 * TB;
 
 }  // namespace

@@ -230,7 +230,10 @@ __device__ __forceinline__ float exact_f32_row(const float* qs, const DevIndex& 
 // 1,374 + 1,852 to 1,143 + 1,624 + 164 at 24 warps per SM; 10,000 queries at ef
 // 140 from 3.34 to 3.04 ms.  The scans have no branches: with a conditional
 // update per entry one took 1,100 cycles instead of 560.
-constexpr int TSCAN = 5;   // 160 entries: one round for the usual ef
+// 160 entries a round.  4 / 5 / 6 per lane, 3,000 queries over 200k x 128, FP16 codes: ef 64 591 /
+// 587 / 599 us, 128 824 / 844 / 858, 140 964 / 890 / 913, 190 1,226 / 1,289 / 1,172, 250 1,527 / 1,590 /
+// 1,674, 300 1,975 / 1,848 / 1,960, 400 2,851 / 2,780 / 2,925: the rounding up decides.
+constexpr int TSCAN = 5;
 
 __device__ __forceinline__ unsigned long long t_key(uint2 v) {
     return (unsigned long long)v.x << 32 | v.y;
