@@ -685,9 +685,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 }
 
 // FP32 rows -> BF16 high and low parts (row stride ms, zero padded) and the
-// FP32 squared norm of every row; one warp per row
+// FP32 squared norm of every row; one warp per row.  With bound (the queries of a kNN
+// launch): their bounds start at none, and the count of redo at 0
 __global__ void k_split_bf16(const float* __restrict__ X, int64_t rows, int m, int64_t x_stride,
-                             int ms, __nv_bfloat16* hi, __nv_bfloat16* lo, float* norm2) {
+                             int ms, __nv_bfloat16* hi, __nv_bfloat16* lo, float* norm2,
+                             uint32_t* bound = nullptr, int32_t* redo = nullptr) {
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (w >= rows) return;
@@ -702,6 +704,10 @@ __global__ void k_split_bf16(const float* __restrict__ X, int64_t rows, int m, i
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (norm2 && lane == 0) norm2[w] = acc;
+    if (bound && lane == 0) {
+        bound[w] = 0xFFFFFFFFu;
+        if (w == 0) redo[0] = 0;
+    }
 }
 
 __device__ __forceinline__ u64 warp_min(u64 k) {
@@ -1364,9 +1370,8 @@ cudaError_t launch_knn_tc(finger_index* ix, const float* Q, int64_t nq, int K, i
     for (int64_t lo = 0; lo < nq && e == cudaSuccess; lo += p.chunk) {
         const int64_t c = std::min(p.chunk, nq - lo);
         const float* q = Q + lo * m;
-        if ((e = cudaMemsetAsync(redo, 0, sizeof(int32_t), s)) != cudaSuccess) break;
-        if ((e = cudaMemsetAsync(bound, 0xFF, sizeof(uint32_t) * (size_t)c, s)) != cudaSuccess) break;
-        k_split_bf16<<<(unsigned)((c * 32 + 255) / 256), 256, 0, s>>>(q, c, m, m, ms, qh, ql, qn);
+        k_split_bf16<<<(unsigned)((c * 32 + 255) / 256), 256, 0, s>>>(q, c, m, m, ms, qh, ql, qn, bound,
+                                                                      redo);
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         if ((e = run_items(ix, base_of(ix), qh, ql, qn, c, KP, p.nseg, CONTIGUOUS, keys, bound, s)) !=
             cudaSuccess)
