@@ -95,10 +95,10 @@ __device__ __forceinline__ float split_error(float nq, float nx, int m) {
 // order: m additions, a subtraction's error twice, a product's
 __host__ __device__ constexpr float sum_error(int m) { return (m + 8) * 0x1p-24f; }
 
-// Whether every row whose approximate distance is v or more, with error err, has an exact
-// one above d
-__device__ __forceinline__ bool all_beyond(float v, float err, float d, int m) {
-    return d < (v - err) * (1.f - sum_error(m));
+// Every row whose approximate distance is v or more, with error err, has an exact one above
+// any that is less than this
+__device__ __forceinline__ float below(float v, float err, int m) {
+    return (v - err) * (1.f - sum_error(m));
 }
 
 // split_error for the rows that may lie at a squared distance of at most d: their length
@@ -880,7 +880,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
         for (int i = lane; i < m; i += 32) bad |= !(fabsf(qr[i]) < INFINITY);
         stands = __any_sync(0xffffffffu, bad);
     }
-    if (stands && last < NO_KEY && !all_beyond(dist_of(last), err, kth, m)) {
+    if (stands && last < NO_KEY && !(kth < below(dist_of(last), err, m))) {
         const float lim = kth * (1.f + 2.f * sum_error(m)) + err;   // above it no key can be nearer
         uint32_t most = 0;             // the largest distance of the list so far
         float edge = INFINITY;         // the smallest of the full lists' largest
@@ -920,7 +920,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
                 __syncwarp();
             }
         }
-        stands = all_beyond(edge, err, dist_of(kth_key(sel, KP, K, lane)), m);
+        stands = dist_of(kth_key(sel, KP, K, lane)) < below(edge, err, m);
     }
     if (stands) put_best(sel, KP, K, out_ids + (size_t)q * K, out_d + (size_t)q * K, lane);
     else if (lane == 0) redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
@@ -954,7 +954,7 @@ __global__ void __launch_bounds__(256)
 // the order of the FP32 kernel (a thread per row, dimension after dimension, so
 // both paths return the same bits) and ranks them.  A row that is not among the R has
 // an approximate distance of at least the R-th and an exact one of at least that less
-// both errors (all_beyond), so the K-th exact distance has to lie below.  A query for
+// both errors, so the K-th exact distance has to lie below.  A query for
 // which it does not, that has fewer than R candidates (rows before it, or finite
 // distances), or a full list whose keys are all among the R (it may have dropped
 // more) goes on `redo` (count in redo[0]) for the FP32 kernel.
@@ -998,6 +998,12 @@ __global__ void __launch_bounds__(256)
         if (t == 0) redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
         return;
     }
+    // the result stands where the K-th exact distance lies below this (the error taken for
+    // rows as far as the R-th)
+    const float vr = dist_of(last), nq = qn[q];
+    const float proof = inf_rows_reach(*xmax, nq, vr)
+                            ? -1.f
+                            : below(vr, near_error(*xmax, nq, fmaxf(vr, 0.f), q_m), q_m);
     for (int i = t; i < R; i += 256) {
         const u64 k = i < np ? bk[i] : ~0ull;
         u64 e = ~0ull;
@@ -1023,19 +1029,12 @@ __global__ void __launch_bounds__(256)
         const u64 k = ex[i];
         int rank = 0;
         for (int j = 0; j < R; ++j) rank += ex[j] < k || (ex[j] == k && j < i);
-        if (rank == K - 1) top[0] = k;   // (the lists' largest keys are done with)
+        if (rank == K - 1 && !(dist_of(k) < proof)) redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
         if (rank < K) {
             const int32_t id = (int32_t)(uint32_t)k;
             out_ids[(size_t)q * K + rank] = id < 0 ? (int64_t)-1 : (int64_t)(remap ? remap[id] : id);
             out_d[(size_t)q * K + rank] = id < 0 ? INFINITY : dist_of(k);
         }
-    }
-    __syncthreads();
-    if (t == 0) {
-        const float kth = dist_of(top[0]), nq = qn[q];
-        if (!all_beyond(dist_of(last), near_error(*xmax, nq, kth, q_m), kth, q_m) ||
-            inf_rows_reach(*xmax, nq, kth))
-            redo[1 + atomicAdd(redo, 1)] = (int32_t)q;
     }
 }
 
