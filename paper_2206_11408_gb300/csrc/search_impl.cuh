@@ -361,6 +361,7 @@ __device__ __forceinline__ int visit(uint32_t* hash, int H, int logNB, uint32_t 
         const int e = v.x == PAD ? 0 : v.y == PAD ? 1 : v.z == PAD ? 2 : v.w == PAD ? 3 : -1;
         if (e < 0) {
             b = (b + 1) & mask;
+            retries = 0;
             continue;
         }
         // the id is in no bucket of its probe sequence
@@ -371,7 +372,9 @@ __device__ __forceinline__ int visit(uint32_t* hash, int H, int logNB, uint32_t 
         const uint32_t old = atomicCAS(&hash[4 * b + e], PAD, id);
         if (old == PAD) return V_NEW;
         if (old == id) return V_SEEN;
-        if (++retries <= 4) --probe;   // re-read this bucket (bounded)
+        // a loss means that another lane took a slot of the bucket, so after four it is full
+        // (counted per bucket: an id moved on past an empty slot would not be found again)
+        if (++retries <= 4) --probe;   // re-read this bucket
         else b = (b + 1) & mask;
     }
     return V_SEEN;  // unreachable: the table never fills (3/4 plus one batch < 1)
