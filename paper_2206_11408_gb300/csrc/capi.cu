@@ -266,16 +266,22 @@ finger_status make_plan(finger_index* ix, int mode, int ef_max, int64_t nq, Sear
     };
     set_table(H, p->H_auto || !long_rows);
     // Long rows in the modes without codes: the staged query's region (3,840 bytes at m =
-    // 960) may cost the fifth block of an SM.  A smaller table makes up for it, down to a
-    // quarter: at such ef most ids are in the bitmap either way.  m = 960, 3,000 queries, 16
-    // resident warps with 2,048 slots -> 20 with 1,024: plain ef 300 3.93 -> 3.51 ms, 500 5.51 ->
-    // 4.73; FP32 tables 500 6.26 -> 5.35; 512 slots, ef 600: plain 6.06 -> 5.20.  10,000
-    // queries: the same within 2 % (ef 400 10.87 -> 10.58, 500 12.71 -> 12.62).
+    // 960) may cost the fifth block of an SM.  A smaller table, down to a quarter, makes up
+    // for it where that brings all queries into one wave and the bitmaps, which then take
+    // more ids, stay in half of L2.  m = 960, 3,000 queries, 16 resident warps with 2,048 slots
+    // -> 20 with 1,024: 60k rows, plain ef 400 4.75 -> 4.06 ms, 500 5.51 -> 4.73, FP32 tables 500
+    // 6.26 -> 5.35; 512 slots, plain ef 600 6.06 -> 5.20.  Elsewhere it loses: 10,000 queries over
+    // 60k rows, ef 300 8.83 -> 9.01; over 1M rows, ef 546 71.2 -> 76.0, 3,000 queries 28.7 -> 30.1.
     if (p->H_auto && occ_force == 0 && long_rows) {
-        const int room = (228 * 1024 / 5 - 1024) / wpb;   // per warp, for five blocks
-        const int full = p->H;
-        for (int h = full; h >= full / 4 && h >= 256 && p->smem_per_warp > room; h >>= 1) set_table(h, false);
-        if (p->smem_per_warp > room) set_table(full, true);
+        const int sm = 228 * 1024, room = (sm / 5 - 1024) / wpb;   // per warp, for five blocks
+        const int64_t wave = (int64_t)ix->num_sms * wpb;           // queries per block of each SM
+        const int64_t bitmaps = 5 * wave * ((ix->n + 31) / 32) * 4;
+        if (nq <= 5 * wave && nq > sm / (p->smem_per_warp * wpb + 1024) * wave && bitmaps <= 64 << 20) {
+            const int full = p->H;
+            for (int h = full; h >= full / 4 && h >= 256 && p->smem_per_warp > room; h >>= 1)
+                set_table(h, false);
+            if (p->smem_per_warp > room) set_table(full, true);
+        }
     }
     if (plan_smem(*p) > 227 * 1024) return FINGER_ERR_UNSUPPORTED;
     // the variant with the most resident blocks that shared memory admits, among

@@ -1,5 +1,5 @@
-"""Long rows in the modes without codes: a smaller visited table where that keeps five blocks
-on an SM.  The same queries in a small batch (several warps per query, the full table), with
+"""Long rows in the modes without codes: a smaller visited table where that brings a batch into
+one wave of five blocks per SM.  The same queries in a small batch (several warps per query, the full table), with
 32-bit slots, and tuned (any table size) give the same ids, distances and counters."""
 import numpy as np
 import pytest
@@ -21,7 +21,8 @@ def test_table_sizes_agree(mode, n, m, M):
     if mode == "FINGER":
         ix.build_tables(16, 6)
     ix.set_mode(getattr(fg, "MODE_" + mode), 5)
-    q = torch.from_numpy((X[rng.integers(0, n, 1300)] + rng.standard_normal((1300, m))).astype(np.float32)).cuda()
+    wave = 18 * torch.cuda.get_device_properties(0).multi_processor_count   # more than four blocks of 4
+    q = torch.from_numpy((X[rng.integers(0, n, wave)] + rng.standard_normal((wave, m))).astype(np.float32)).cuda()
 
     def search(nq, ef):
         cnt = torch.zeros((nq, 8), dtype=torch.int32, device="cuda")
@@ -32,14 +33,14 @@ def test_table_sizes_agree(mode, n, m, M):
         return (*out, cnt)
 
     for ef in (290, 320, 500, 560, 640, 700):
-        whole = search(1300, ef)
+        whole = search(wave, ef)
         for a, b in zip(whole, search(100, ef)):
             assert torch.equal(a[:100], b), ef
         ix.set_visited_slots(32)
-        for a, b in zip(whole, search(1300, ef)):
+        for a, b in zip(whole, search(wave, ef)):
             assert torch.equal(a, b), ef
         ix.set_visited_slots(0)
     ix.autotune(q, 10, 500)
-    for a, b in zip(search(1300, 500), search(100, 500)):
+    for a, b in zip(search(wave, 500), search(100, 500)):
         assert torch.equal(a[:100], b)
     ix.close()
